@@ -272,8 +272,8 @@ def run(s):
             plan.run_graph(1)
             out = []
             for j in range(plan.n_regions):
-                theta, dist, idx, n, days = plan.results(j)
-                out.append(_sorted(theta, dist, idx) + (n, days))
+                theta, dist, idx, n, _ = plan.results(j)    # the fifth is the work done, not a result
+                out.append(_sorted(theta, dist, idx) + (n,))
         torch.cuda.current_stream().wait_stream(s["stream"])
         return out
     if kind == "flow_sample":
