@@ -91,7 +91,9 @@ typedef enum {
  * returns ABC_ERR_CAPACITY, *n_accepted holds the true count and the output
  * buffers hold an unspecified subset of `capacity` accepted samples.
  * Samples whose running distance^2 exceeds eps^2 are abandoned early (partial
- * sums only grow); the result is that of simulating all T days of every sample.
+ * sums only grow), and so are samples whose infected have died out when the
+ * days left must take it there; the result is that of simulating all T days of
+ * every sample.
  * Uses a small amount of device scratch memory (the observed series and three
  * counters) and pinned host memory to stage it, allocated on the first call of
  * each host thread on each device, grown when a longer series needs more and
@@ -715,9 +717,10 @@ abc_status abc_sample_noalloc(const abc_prior_box* prior, const int32_t* observe
 
 /* Number of model days simulated by the last successful abc_sample call on
  * this thread. abc_sample stops simulating a sample once its running distance^2
- * exceeds eps^2 (the partial sums only grow, so it could not be accepted); the
- * accept set is the same as simulating all T days of every sample. This count is
- * the work actually done: at most n_samples * T. */
+ * exceeds eps^2 (the partial sums only grow, so it could not be accepted), or
+ * once its infected have died out and a lower bound on the days left exceeds
+ * it; the accept set is the same as simulating all T days of every sample. This
+ * count is the work actually done: at most n_samples * T. */
 uint64_t abc_last_simulated_days(void);
 
 /* Static description of a status code. */

@@ -137,7 +137,7 @@ int kernel_mode(abc_mode mode)
            (((int)mode & ABC_VARIANCE_LITERAL) ? abcgb::kLiteral : 0);
 }
 
-// Observed [3][T+1] rows A, R, D -> per-day int4 (A, R, D, 0).
+// Observed [3][T+1] rows A, R, D -> per-day int4 (A, R, D, extinction_terms).
 abc_status pack_observed(const int32_t* observed, int32_t T, int64_t N_pop, std::vector<int4>& out)
 {
     if (!observed) return fail(ABC_ERR_INVALID_ARG, "observed is NULL");
@@ -147,6 +147,7 @@ abc_status pack_observed(const int32_t* observed, int32_t T, int64_t N_pop, std:
         if (A < 0 || R < 0 || D < 0) return fail(ABC_ERR_INVALID_ARG, "negative observed count on day %d", d);
         out[d] = make_int4(A, R, D, 0);
     }
+    abcgb::extinction_terms(out.data(), T);
     const int32_t ard0[3] = {out[0].x, out[0].y, out[0].z};
     return check_initial(ard0, N_pop);
 }
@@ -279,7 +280,7 @@ struct abc_observed_s {
     int32_t T = 0;
     int64_t N_pop = 0;
     int32_t ard0[3] = {0, 0, 0};
-    void* dev = nullptr;   // int4 [T+1] (A, R, D, 0)
+    void* dev = nullptr;   // int4 [T+1] (A, R, D, extinction_terms)
 };
 
 // Scratch of abc_sample_noalloc: bytes [0, 24) hold the three counters
@@ -322,6 +323,25 @@ abc_status noalloc_scratch(void** out)
 }  // namespace
 
 namespace abcgb {
+
+void extinction_terms(int4* obs, int32_t T)
+{
+    // backwards over the days, mean and squared deviations updated a day at a
+    // time (Welford): no cancellation for a flat series of large counts
+    double n = 0.0, mean = 0.0, dev = 0.0;
+    for (int32_t e = T - 1; e >= 2; --e) {
+        const double u = (double)obs[e + 1].x + (double)obs[e + 1].y + (double)obs[e + 1].z;
+        const double d = u - mean;
+        n += 1.0;
+        mean += d / n;
+        dev += d * (u - mean);
+        if (e & 1) continue;
+        const float m = (float)mean, v = (float)(dev * (1.0 - 1e-6));
+        std::memcpy(&obs[e].w, &m, sizeof m);
+        std::memcpy(&obs[e - 1].w, &v, sizeof v);
+    }
+}
+
 // Helpers shared with the batched-regions ABI (abc_plan.cu): the same error
 // reporting, checks and kernel parameters as the calls in this file.
 abc_status plan_fail(abc_status st, const char* msg) { return fail(st, "%s", msg); }
@@ -878,6 +898,7 @@ abc_status abc_sample_noalloc(const abc_prior_box* prior, const int32_t* observe
         if (A < 0 || R < 0 || D < 0) return fail(ABC_ERR_INVALID_ARG, "negative observed count on day %d", d);
         obs[d] = make_int4(A, R, D, 0);
     }
+    abcgb::extinction_terms(obs, T);
     const int32_t ard0[3] = {obs[0].x, obs[0].y, obs[0].z};
     if ((st = check_initial(ard0, N_pop)) != ABC_OK) return st;
     *n_accepted = 0;

@@ -64,11 +64,9 @@ struct LaneRegion {
 // moves them to the block's 64-bit per-region count when its region changes
 // (chunks are laid out region by region, so rarely) or the register passes
 // 2^31, and at the end. Adding each sample's days to the shared count with a
-// 64-bit shared-memory atomic cost 5 % of the 16-region stream (52.5 -> 49.7
-// ms) and 3 % of the three-region workload. The autotuner chooses between the
-// two forms; with the register count it takes the lean form on both
-// workloads (16-region stream 49.1 ms, three-region workload 2.12 ms, against
-// 56.4 and 2.18 ms for the standard form).
+// 64-bit shared-memory atomic cost 5 % of a 16-region run and 3 % of a
+// three-region one. The autotuner chooses between the two forms; it takes the
+// lean form on both workloads.
 template <int MODE, int BLOCK, int PAIRS, bool BELOW62, bool OBS_S, bool LEAN>
 __global__ void __launch_bounds__(BLOCK, LEAN ? 4 : 1) abc_batch_kernel(const __grid_constant__ ModelParams p,
                                                           const __grid_constant__ BatchArgs a)
@@ -216,13 +214,19 @@ __global__ void __launch_bounds__(BLOCK, LEAN ? 4 : 1) abc_batch_kernel(const __
                 const int4 o1 = OBS_S ? obs[d1] : __ldg(obs + d1);
                 acc = BELOW62 ? add_day_sq_below62(acc, x, o1) : add_day_sq(acc, x, o1);
                 const int32_t T = LEAN ? R.T : lr.T;
+                int32_t m_bits = 0;
                 if (d1 < T) {
                     model_day<MODE>(x, t, inv_p, z + 5);
                     const int4 o2 = OBS_S ? obs[d1 + 1] : __ldg(obs + d1 + 1);
+                    m_bits = o2.w;
                     acc = BELOW62 ? add_day_sq_below62(acc, x, o2) : add_day_sq(acc, x, o2);
                 }
-                const bool over = acc > (LEAN ? R.acc_max : lr.acc_max);
+                const uint64_t acc_max = LEAN ? R.acc_max : lr.acc_max;
+                bool over = acc > acc_max;
                 const bool last = d1 + 1 >= T;
+                // infected died out: dropped once it cannot be accepted, as in abc_reject_kernel
+                if (x.I == 0 && !over && !last && (BELOW62 || acc_max < kAccCap))
+                    over = extinct_over(x, o1.w, m_bits, T - d1 - 1, acc, acc_max);
                 accept = !over && last;
                 active = !(over || last);
                 ++k;

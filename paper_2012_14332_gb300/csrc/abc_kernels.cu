@@ -27,7 +27,8 @@ __device__ __forceinline__ void stage_observed(int4* obs_s, const int4* __restri
 // The partial sums of the distance^2 only grow, so a sample whose running sum
 // exceeds acc_max after some day pair can never be accepted: its lane drops it
 // and takes the next sample (the accept set and the accepted distances are
-// exactly those of running every sample for all T days). Each warp keeps a
+// exactly those of running every sample for all T days). So does the lane of a
+// sample whose infected have died out too far from the series (extinct_over). Each warp keeps a
 // 64-entry ring of prior draws in shared memory, refilled 32 at a time by the
 // whole warp (sample indices claimed with one atomicAdd per 32), so the theta
 // draw of a new sample costs one shared-memory read for the lane that needs
@@ -44,8 +45,9 @@ constexpr int kWarpsPerBlock = kBlockThreads / 32;
 // them are idle (all 32 always qualify): the hand-out (ring read, derived
 // parameters, initial state) runs on the whole warp, while a lane left idle
 // for a day pair costs a 32nd of one. Measured on P = 6e7, T = 100, 2^24
-// samples: 5.67 ms per launch at 1, 5.58 at 2 and at 4, 5.84 at 8. Which lane
-// runs a sample, and when, does not change the sample's result.
+// samples: 3.218 ms per launch at 1 (two pairs per pass), 3.209 at 2 and at 3,
+// 3.219 at 4; exact mode's 2^22 samples 2.020 ms at 2, 2.030 at 3, 2.050 at 4.
+// Which lane runs a sample, and when, does not change the sample's result.
 constexpr uint32_t kRefillMinIdle = 2;
 
 struct WarpRing {
@@ -137,10 +139,9 @@ __global__ void __launch_bounds__(kBlockThreads) abc_reject_kernel(const __grid_
         }
 
         // fast mode takes three day pairs per pass between hand-outs, cutting
-        // the refill and accept checks; per 2^24 samples of P = 6e7, T = 100
-        // (interleaved, three repeats): 1 pair 5.462 ms, 2 pairs 5.474, 3 pairs
-        // 5.424, 4 pairs 5.438, 5 pairs 5.503. Exact mode's longer day ran
-        // 13 % slower with two pairs.
+        // the refill and accept checks; per 2^24 samples of P = 6e7, T = 100:
+        // 1 pair 3.232 ms, 2 pairs 3.218, 3 pairs 3.209. Exact mode's longer
+        // day ran 13 % slower with two pairs.
         bool accept = false;
 #pragma unroll
         for (int rep = 0; rep < ((MODE & kFast) ? 3 : 1); ++rep)
@@ -149,13 +150,20 @@ __global__ void __launch_bounds__(kBlockThreads) abc_reject_kernel(const __grid_
             day_pair_normals<MODE>(p, i, k, z);
             const int32_t d1 = (int32_t)(2 * k - 1);
             model_day<MODE>(x, t, p.inv_p, z);
-            acc = BELOW62 ? add_day_sq_below62(acc, x, obs_s[d1]) : add_day_sq(acc, x, obs_s[d1]);
+            const int4 o1 = obs_s[d1];
+            int32_t m_bits = 0;
+            acc = BELOW62 ? add_day_sq_below62(acc, x, o1) : add_day_sq(acc, x, o1);
             if (d1 < T) {
                 model_day<MODE>(x, t, p.inv_p, z + 5);
-                acc = BELOW62 ? add_day_sq_below62(acc, x, obs_s[d1 + 1]) : add_day_sq(acc, x, obs_s[d1 + 1]);
+                const int4 o2 = obs_s[d1 + 1];
+                m_bits = o2.w;
+                acc = BELOW62 ? add_day_sq_below62(acc, x, o2) : add_day_sq(acc, x, o2);
             }
-            const bool over = acc > a.acc_max;
+            bool over = acc > a.acc_max;
             const bool last = d1 + 1 >= T;
+            // a threshold of 2^63 accepts sums that saturate there: nothing is over
+            if (x.I == 0 && !over && !last && (BELOW62 || a.acc_max < kAccCap))
+                over = extinct_over(x, o1.w, m_bits, T - d1 - 1, acc, a.acc_max);
             accept = !over && last;
             active = !(over || last);
             ++k;

@@ -38,8 +38,15 @@ inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 b
 
 struct ModelParams;
 
+// Fills the fourth word of a packed observed series (host int4 [T+1]: A, R, D
+// of day d) with what the rejection kernels need to drop a sample whose
+// infected have died out: for each even day e, 2 <= e < T, obs[e].w holds the
+// mean of A + R + D over days e + 1 .. T (float bits) and obs[e - 1].w their sum
+// of squared deviations from it, rounded down. The other fourth words are 0.
+void extinction_terms(int4* obs, int32_t T);
+
 struct RejectArgs {
-    const int4* obs;              // device [T+1] (A, R, D, 0)
+    const int4* obs;              // device [T+1] (A, R, D, extinction_terms)
     uint64_t first_index, n_samples;
     uint64_t acc_max;             // accept iff distance^2 <= acc_max
     unsigned long long* count;    // device counter of accepts, zeroed before launch
@@ -99,7 +106,7 @@ struct BatchArgs {
     const RegionDev* regions;      // device [n_regions]
     int32_t n_regions;
     uint64_t total_chunks;
-    const int4* obs;               // device, concatenated (A, R, D, 0) per day of every region
+    const int4* obs;               // device, concatenated (A, R, D, extinction_terms) per day of every region
     int32_t n_obs_smem;            // > 0: all n_obs_smem entries of obs are staged in shared memory
     unsigned long long* next;      // claimed chunks, zeroed before each run
 };

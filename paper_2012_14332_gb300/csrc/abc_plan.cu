@@ -157,6 +157,7 @@ abc_status abc_plan_create(const abc_prior_box* prior, const abc_region* regions
             }
             obs.push_back(make_int4(A, Rr, D, 0));
         }
+        abcgb::extinction_terms(obs.data() + R.obs_off, g.T);
         const int4 o0 = obs[R.obs_off];
         if ((int64_t)o0.x + o0.y + o0.z > g.N_pop) {
             snprintf(msg, sizeof msg, "region %d: A0 + R0 + D0 exceeds N_pop", r);
