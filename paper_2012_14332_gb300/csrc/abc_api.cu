@@ -714,6 +714,36 @@ abc_status abc_project(const float* theta, const uint64_t* sample_index, uint64_
     return ok();
 }
 
+}  // extern "C"
+
+namespace {
+
+// Scratch of a k-th smallest: `head` bytes for the caller at sc.ptr, then the
+// work area and room for `cap` candidates. Candidates above kSelectCandKeep
+// keys, or for which there is no memory, are done without (*cand NULL): the
+// radix select needs none.
+constexpr uint64_t kSelectCandKeep = 1ull << 27;   // 1 GiB of keys, what the pool keeps mapped
+abc_status alloc_select(Scratch& sc, size_t head, uint64_t cap, cudaStream_t s, abcgb::SelectWork** work,
+                        uint64_t** cand)
+{
+    const size_t at = (head + 255) / 256 * 256, after = at + (sizeof(abcgb::SelectWork) + 255) / 256 * 256;
+    *cand = nullptr;
+    abc_status st = ABC_ERR_NOMEM;
+    if (cap <= kSelectCandKeep) {
+        st = alloc_scratch(sc, after + sizeof(uint64_t) * cap, s);
+        if (st == ABC_OK) *cand = (uint64_t*)((char*)sc.ptr + after);
+        if (st == ABC_ERR_NOMEM) cudaGetLastError();   // answered by the smaller attempt
+    }
+    if (st == ABC_ERR_NOMEM) st = alloc_scratch(sc, after, s);
+    if (st != ABC_OK) return st;
+    *work = (abcgb::SelectWork*)((char*)sc.ptr + at);
+    return ABC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 abc_status abc_kth_smallest(const double* dist, uint64_t n, uint64_t k, double* eps_out, void* cuda_stream)
 {
     if (!dist || !eps_out) return fail(ABC_ERR_INVALID_ARG, "NULL pointer");
@@ -722,16 +752,24 @@ abc_status abc_kth_smallest(const double* dist, uint64_t n, uint64_t k, double* 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     abc_status st;
     Scratch sc;
-    const size_t bytes = 258 * sizeof(unsigned long long) + sizeof(abcgb::SelectState);
-    if ((st = alloc_scratch(sc, bytes, s)) != ABC_OK) return st;
-    unsigned long long* hist_d = (unsigned long long*)sc.ptr;
-    abcgb::SelectState* st_d = (abcgb::SelectState*)(hist_d + 258);   // 16-byte aligned after the 258 counters
-    CUDA_TRY(cudaMemsetAsync(sc.ptr, 0, bytes, s), "cudaMemsetAsync(select scratch)");
+    abcgb::SelectWork* w = nullptr;
+    uint64_t* cand = nullptr;
+    const uint64_t cap = abcgb::select_candidates(n, k);
+    if ((st = alloc_select(sc, 0, cap, s, &w, &cand)) != ABC_OK) return st;
+    CUDA_TRY(cudaMemsetAsync(w, 0, abcgb::kSelectZeroBytes, s), "cudaMemsetAsync(select scratch)");
     if (injected("launch")) return fail(ABC_ERR_CUDA, "kernel launch failed (injected)");
-    CUDA_TRY(abcgb::launch_kth_select(dist, n, k, hist_d, st_d, s), "radix select launch");
     abcgb::SelectState h;
-    CUDA_TRY(cudaMemcpyAsync(&h, st_d, sizeof h, cudaMemcpyDeviceToHost, s), "cudaMemcpyAsync(select state)");
-    CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    h.resolved = 0;
+    if (cand) {
+        CUDA_TRY(abcgb::launch_kth_bracket(dist, n, k, w, cand, cap, s), "bracket select launch");
+        CUDA_TRY(cudaMemcpyAsync(&h, &w->st, sizeof h, cudaMemcpyDeviceToHost, s), "cudaMemcpyAsync(select state)");
+        CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    }
+    if (!h.resolved) {
+        CUDA_TRY(abcgb::launch_kth_radix(dist, n, k, w, s), "radix select launch");
+        CUDA_TRY(cudaMemcpyAsync(&h, &w->st, sizeof h, cudaMemcpyDeviceToHost, s), "cudaMemcpyAsync(select state)");
+        CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    }
     // keys that are NaN or carry the sign bit do not order like values
     if (h.bad != 0) return fail(ABC_ERR_INVALID_ARG, "%llu distances are negative, -0 or NaN", h.bad);
     std::memcpy(eps_out, &h.prefix, sizeof h.prefix);
@@ -803,28 +841,30 @@ abc_status abc_sample_quantile(const abc_prior_box* prior, const int32_t* observ
     const abcgb::ModelParams p = make_params(prior, T, N_pop, seed, stream, ard0);
     cudaStream_t s = (cudaStream_t)cuda_stream;
 
-    // every distance and prior draw: stream-ordered scratch, 40 bytes a sample
+    // every distance and prior draw: stream-ordered scratch, 40 bytes a sample,
+    // and the selection's work area and candidates
     const size_t dist_bytes = ((sizeof(double) * n_samples + 255) / 256) * 256;
     Scratch big;
-    if ((st = alloc_scratch(big, dist_bytes + sizeof(float) * 8 * n_samples, s)) != ABC_OK) return st;
+    abcgb::SelectWork* w = nullptr;
+    uint64_t* cand = nullptr;
+    const uint64_t cap = abcgb::select_candidates(n_samples, k);
+    if ((st = alloc_select(big, dist_bytes + sizeof(float) * 8 * n_samples, cap, s, &w, &cand)) != ABC_OK) return st;
     double* dist_d = (double*)big.ptr;
     float* theta_d = (float*)((char*)big.ptr + dist_bytes);
-    // the radix select's histogram (258 counters) and state, the accept
-    // counter, then the observed series: zeroed and uploaded in one copy
-    // from pinned staging
+    // the accept counter, then the observed series: uploaded in one copy from
+    // pinned staging; the selection's state comes back behind the counter
     struct Tail {
-        abcgb::SelectState sel;
         unsigned long long count;
+        abcgb::SelectState sel;
     };
-    const size_t tail_off = 258 * sizeof(unsigned long long), obs_off = 2112;
-    static_assert(258 * sizeof(unsigned long long) + sizeof(Tail) <= 2112, "select scratch overlaps the series");
+    const size_t obs_off = 256;
+    static_assert(sizeof(Tail) <= 256, "the staged state overlaps the series");
     SampleScratch* sc = nullptr;
     if ((st = sample_scratch(obs_off + sizeof(int4) * obs.size(), &sc)) != ABC_OK) return st;
     std::memset(sc->host, 0, obs_off);
     std::memcpy((char*)sc->host + obs_off, obs.data(), sizeof(int4) * obs.size());
-    unsigned long long* hist_d = (unsigned long long*)sc->dev;
-    Tail* tail_d = (Tail*)((char*)sc->dev + tail_off);
-    Tail* tail_h = (Tail*)((char*)sc->host + tail_off);
+    unsigned long long* count_d = (unsigned long long*)sc->dev;
+    Tail* tail_h = (Tail*)sc->host;
     if (injected("launch")) return fail(ABC_ERR_CUDA, "kernel launch failed (injected)");
     // from here on the pinned staging buffer may be in use by the stream: every
     // error return first waits for the stream so the next call can reuse it
@@ -842,25 +882,37 @@ abc_status abc_sample_quantile(const abc_prior_box* prior, const int32_t* observ
     da.theta_out = theta_d;
     ce = abcgb::launch_distances(p, da, kernel_mode(mode), s);
     if (ce != cudaSuccess) return drain(cuda_fail(ce, "abc_distance_kernel launch"));
-    ce = abcgb::launch_kth_select(dist_d, n_samples, k, hist_d, &tail_d->sel, s);
-    if (ce != cudaSuccess) return drain(cuda_fail(ce, "radix select launch"));
     abcgb::SelectArgs a;
     a.dist = dist_d;
     a.theta = theta_d;
     a.n = n_samples;
     a.first_index = first_index;
     a.eps = 0.0;
-    a.eps_key = &tail_d->sel;
+    a.eps_key = &w->st;
     a.theta_out = theta_out;
     a.dist_out = dist_out;
     a.idx_out = idx_out;
     a.capacity = capacity;
-    a.count = &tail_d->count;
-    ce = abcgb::launch_select_below(a, s);
-    if (ce != cudaSuccess) return drain(cuda_fail(ce, "select_below launch"));
-    ce = cudaMemcpyAsync(tail_h, tail_d, sizeof(Tail), cudaMemcpyDeviceToHost, s);
-    if (ce != cudaSuccess) return drain(cuda_fail(ce, "cudaMemcpyAsync(select state)"));
-    CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    a.count = count_d;
+    // the key by the bracket; by the radix select where that left it open
+    for (int pass = cand ? 0 : 1; pass < 2; ++pass) {
+        if (pass == 0) {
+            ce = cudaMemsetAsync(w, 0, abcgb::kSelectZeroBytes, s);
+            if (ce == cudaSuccess) ce = abcgb::launch_kth_bracket(dist_d, n_samples, k, w, cand, cap, s);
+        } else {
+            ce = cudaMemsetAsync(count_d, 0, sizeof *count_d, s);
+            if (ce == cudaSuccess) ce = abcgb::launch_kth_radix(dist_d, n_samples, k, w, s);
+        }
+        if (ce != cudaSuccess) return drain(cuda_fail(ce, "k-th smallest launch"));
+        ce = abcgb::launch_select_below(a, s);
+        if (ce != cudaSuccess) return drain(cuda_fail(ce, "select_below launch"));
+        ce = cudaMemcpyAsync(&tail_h->count, count_d, sizeof *count_d, cudaMemcpyDeviceToHost, s);
+        if (ce == cudaSuccess)
+            ce = cudaMemcpyAsync(&tail_h->sel, &w->st, sizeof tail_h->sel, cudaMemcpyDeviceToHost, s);
+        if (ce != cudaSuccess) return drain(cuda_fail(ce, "cudaMemcpyAsync(select state)"));
+        CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+        if (tail_h->sel.resolved) break;
+    }
     // the distances of the model are never NaN or negative
     if (tail_h->sel.bad != 0)
         return fail(ABC_ERR_CUDA, "%llu distances are negative, -0 or NaN", tail_h->sel.bad);

@@ -1,6 +1,7 @@
 // abc_kernels.h -- internal launch interface between the C ABI (abc_api.cu) and
 // the kernels (abc_kernels.cu). Not part of the public ABI.
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -141,14 +142,33 @@ cudaError_t launch_simulate(const ModelParams& p, const SimulateArgs& a, int mod
 cudaError_t launch_step(const ModelParams& p, const StepArgs& a, int mode, cudaStream_t s);
 cudaError_t launch_bands(const int32_t* traj, uint32_t B, int32_t T, const float* qpos, int32_t n_q, float* bands,
                          cudaStream_t s);
-// Radix select of the k-th smallest of n distances, all passes on the device:
-// hist (258 counters: the histogram and a ticket counter) and st zeroed by the
-// caller, and left zeroed and holding the result; afterwards st->prefix is
-// the k-th smallest key and st->bad the number of invalid keys (NaN, sign bit
-// set), in which case the prefix is meaningless.
+// The k-th smallest of n distances (abc_select.cu), all on the device. In a
+// SelectWork whose first kSelectZeroBytes are zero launch_kth_bracket leaves
+// st.bad, the number of invalid keys (NaN, sign bit set), and, if there are none
+// and st.resolved is set, the k-th smallest key in st.prefix; `cand` has room
+// for `cap` = select_candidates(n, k) keys. When it leaves st.resolved at 0,
+// launch_kth_radix (which zeroes the work area itself) finds the key on any
+// input, by eight passes over the distances, or counts the invalid ones.
 struct SelectState {
     unsigned long long prefix, mask, rank, bad;
+    unsigned long long lo, hi;          // the bracket of the wanted key
+    unsigned long long below, count;    // keys below it, keys inside (the candidates)
+    unsigned long long not_least, most; // ~ the least candidate, the greatest
+    unsigned int ticket[3], n_few;
+    int stage, resolved;
 };
+constexpr int kPivotSample = 2048;
+struct SelectWork {
+    SelectState st;
+    unsigned long long hist[258];       // radix select: 256 bins, invalid keys, ticket
+    uint32_t bins[2048];
+    uint64_t few[4096];
+};
+constexpr size_t kSelectZeroBytes = offsetof(SelectWork, few);
+uint64_t select_candidates(uint64_t n, uint64_t k);
+cudaError_t launch_kth_bracket(const double* dist, uint64_t n, uint64_t k, SelectWork* w, uint64_t* cand, uint64_t cap,
+                               cudaStream_t s);
+cudaError_t launch_kth_radix(const double* dist, uint64_t n, uint64_t k, SelectWork* w, cudaStream_t s);
 // Compaction of the samples with dist[j] <= eps (theta, theta_out may both be
 // NULL); *count (zeroed by the caller) receives the number of accepts. With
 // eps_key set, eps is the value whose bit pattern is eps_key->prefix (the
@@ -166,7 +186,5 @@ struct SelectArgs {
     unsigned long long* count;
 };
 cudaError_t launch_select_below(const SelectArgs& a, cudaStream_t s);
-cudaError_t launch_kth_select(const double* dist, uint64_t n, uint64_t k, unsigned long long* hist, SelectState* st,
-                              cudaStream_t s);
 
 }  // namespace abcgb
