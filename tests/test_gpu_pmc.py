@@ -105,3 +105,26 @@ def test_pmc_posterior_matches_plain_abc():
     wa = wt.cpu().numpy()
     b = th_p.cpu().numpy().astype(np.float64)
     assert_posterior_close(a, wa, b, tag="population Monte Carlo")
+
+
+@pytest.mark.parametrize("n,m", [(1, 1), (7, 300), (127, 8), (128, 9), (129, 257), (300, 2049), (1217, 300), (2433, 300), (5000, 7)])
+def test_weights_at_the_edges_of_the_split(n, m):
+    """Rows and old particles that do not fill a cluster's rows, a slice or a
+    tile; the last rows so far away that every term is below the least normal
+    float (terms of about 2^-135, 14 bits left: 2^-13 relative)."""
+    old, w = _population(m, 10 + m)
+    new, _ = _population(n, 20 + n)
+    L = (np.eye(8) * 0.2 * (HI - LO)).astype(np.float32)
+    Li = np.linalg.inv(L.astype(np.float64))
+    far = max(1, n // 8)
+    centre = old.astype(np.float64).mean(0)
+    dist = np.sqrt(2 * 135 * np.log(2.0))
+    old[:] = (centre + 1e-3 * (old - centre)).astype(np.float32)
+    new[n - far:] = (centre + dist * L.astype(np.float64)[:, 0]).astype(np.float32)
+    got = abc.abc_pmc_weights(torch.from_numpy(new).to(DEV), torch.from_numpy(old).to(DEV),
+                              torch.from_numpy(w).to(DEV), L).cpu().numpy()
+    d2 = (((new.astype(np.float64) @ Li.T)[:, None, :] - (old.astype(np.float64) @ Li.T)[None]) ** 2).sum(2)
+    want = 1.0 / (np.exp(-0.5 * d2) @ w)
+    rel = np.abs(got / want - 1)
+    # an exponent of x bits carries x 2^-23 from FP32 distances: 1e-4 at 135, less nearer
+    assert rel[:n - far].max(initial=0) < 1e-4 and rel[n - far:].max() < 1e-3 + 2.0 ** -13
