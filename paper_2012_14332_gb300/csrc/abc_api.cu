@@ -688,29 +688,43 @@ abc_status abc_project(const float* theta, const uint64_t* sample_index, uint64_
     if (B < 1 || B > ABC_PROJECT_MAX_B) return fail(ABC_ERR_INVALID_ARG, "B must be in [1, %d]", ABC_PROJECT_MAX_B);
     if (!theta || !sample_index || !bands_out || !quantiles || n_q < 1 || n_q > 1024)
         return fail(ABC_ERR_INVALID_ARG, "NULL buffer or n_q outside [1, 1024]");
-    std::vector<float> qpos((size_t)n_q);
+    std::vector<uint32_t> qpos((size_t)n_q);
     for (int32_t k = 0; k < n_q; ++k) {
         if (!(quantiles[k] >= 0.0 && quantiles[k] <= 1.0)) return fail(ABC_ERR_INVALID_ARG, "quantile outside [0, 1]");
-        qpos[k] = (float)std::floor(quantiles[k] * (double)(B - 1));
+        qpos[k] = (uint32_t)std::floor(quantiles[k] * (double)(B - 1));
     }
     const abcgb::ModelParams p = make_params(nullptr, T, N_pop, seed, stream, init_ard);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     Scratch sc;
-    const size_t traj_bytes = sizeof(int32_t) * 6 * (size_t)(T + 1) * B;
-    if ((st = alloc_scratch(sc, traj_bytes + sizeof(float) * n_q, s)) != ABC_OK) return st;
-    int32_t* traj = (int32_t*)sc.ptr;
-    float* qd = (float*)((char*)sc.ptr + traj_bytes);
-    CUDA_TRY(cudaMemcpyAsync(qd, qpos.data(), sizeof(float) * n_q, cudaMemcpyHostToDevice, s), "cudaMemcpyAsync(q)");
-    abcgb::SimulateArgs a;
-    a.theta = theta;
-    a.sample_index = sample_index;
-    a.B = B;
-    a.traj_out = traj;
+    abcgb::ColumnArgs c;
+    c.theta = theta;
+    c.sample_index = sample_index;
+    c.B = B;
+    c.stride = (size_t)(B + 31) / 32 * 32;   // whole 128-byte lines
+    const size_t column_bytes = sizeof(int32_t) * 3 * (size_t)(T + 1) * c.stride;
+    // a few ranks go with the launch, many through device memory
+    const bool few = n_q <= abcgb::kBandRanks;
+    if ((st = alloc_scratch(sc, column_bytes + (few ? 0 : sizeof(uint32_t) * n_q), s)) != ABC_OK) return st;
+    c.out = (int32_t*)sc.ptr;
+    abcgb::BandArgs b;
+    b.columns = c.out;
+    b.stride = c.stride;
+    b.B = (uint32_t)B;
+    b.n_q = n_q;
+    b.qpos_dev = nullptr;
+    b.bands = bands_out;
+    if (few) {
+        std::copy(qpos.begin(), qpos.end(), b.qpos);
+    } else {
+        uint32_t* qd = (uint32_t*)((char*)sc.ptr + column_bytes);
+        CUDA_TRY(cudaMemcpyAsync(qd, qpos.data(), sizeof(uint32_t) * n_q, cudaMemcpyHostToDevice, s), "cudaMemcpyAsync(q)");
+        b.qpos_dev = qd;
+    }
     if (injected("launch")) return fail(ABC_ERR_CUDA, "kernel launch failed (injected)");
-    CUDA_TRY(abcgb::launch_simulate(p, a, kernel_mode(mode), s), "abc_simulate_kernel launch");
-    CUDA_TRY(abcgb::launch_bands(traj, (uint32_t)B, T, qd, n_q, bands_out, s), "band_kernel launch");
-    // qpos (host) was staged synchronously enough: wait for the copy before it leaves scope
-    CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    CUDA_TRY(abcgb::launch_columns(p, c, kernel_mode(mode), s), "trajectory kernel launch");
+    CUDA_TRY(abcgb::launch_bands(b, T, s), "band_kernel launch");
+    // the ranks on the host must outlive their copy
+    if (!few) CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
     return ok();
 }
 

@@ -3,13 +3,10 @@
 // observed series in shared memory, the accepted samples compacted with a
 // warp ballot and one atomic per warp.
 #include <cstdint>
-#include <map>
-#include <mutex>
-#include <tuple>
-#include <utility>
 #include <cuda_runtime.h>
 
 #include "abc_kernels.h"
+#include "abc_launch.h"
 #include "abc_model.cuh"
 
 namespace abcgb {
@@ -213,7 +210,7 @@ __global__ void __launch_bounds__(kBlockThreads) abc_distance_kernel(const __gri
         prior_draw(p, i, th);
         const Theta t = make_theta<MODE>(th, p.inv_p);
         const State x0 = init_state(t, p.A0, p.R0, p.D0, p.room0);
-        const uint64_t acc = simulate_sample<MODE>(p, i, t, x0, obs_s, NoVisit());
+        const uint64_t acc = simulate_sample<MODE>(p, i, t, x0, obs_s);
         a.dist_out[j] = __dsqrt_rn(__ull2double_rn(acc));
         if (a.theta_out) {
             float4* to = reinterpret_cast<float4*>(a.theta_out + 8 * j);
@@ -224,37 +221,89 @@ __global__ void __launch_bounds__(kBlockThreads) abc_distance_kernel(const __gri
 }
 
 // ---------------------------------------------------------------------------
-// K3: trajectories of given (theta, sample index) pairs.
+// K3: trajectories of given (theta, sample index) pairs, whole rows
+// [T + 1][6] (S, I, A, R, D, Ru), a thread per sample. A warp keeps kTrajDays
+// days of its 32 rows in shared memory and then writes each row's days as one
+// run of 8-byte words: a lane storing its own six values a day touched 32
+// sectors with every 4 bytes. ALU-bound now: 100,003 rows over 90 days in exact arithmetic
+// 442 -> 215 us (218 MB written). Blocks of two warps spread the rows evenly
+// over the SMs.
 // ---------------------------------------------------------------------------
-struct TrajVisit {
-    int32_t* out;
-    __device__ __forceinline__ void operator()(int32_t d, const State& x) const
-    {
-        int32_t* o = out + 6 * (size_t)d;
-        o[0] = x.S; o[1] = x.I; o[2] = x.A; o[3] = x.R; o[4] = x.D; o[5] = x.Ru;
-    }
+constexpr int kTrajDays = 8;
+constexpr int kTrajThreads = 64;
+struct TrajRows {
+    int2 s[32][3 * kTrajDays + 1];   // the odd stride (in 8 bytes) spreads lanes over the banks
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(kBlockThreads) abc_simulate_kernel(const __grid_constant__ ModelParams p,
-                                                                     const __grid_constant__ SimulateArgs a)
+// days d0 .. d0 + days - 1 of the warp's rows to global memory, 8 lanes a row
+__device__ __forceinline__ void write_days(const TrajRows& tile, int32_t* out, uint32_t rows, int32_t T, int32_t d0,
+                                           int32_t days, bool wide)
 {
-    extern __shared__ int4 obs_s[];
-    // no observed series here: a zero series keeps the distance code shared
-    for (int32_t d = threadIdx.x; d <= p.T; d += blockDim.x) obs_s[d] = make_int4(0, 0, 0, 0);
-    __syncthreads();
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < a.B; b += stride) {
+    const uint32_t lane = threadIdx.x & 31u;
+    __syncwarp();
+    for (uint32_t r = lane >> 3; r < rows; r += 4) {
+        int32_t* to = out + (size_t)r * 6 * (size_t)(T + 1) + 6 * (size_t)d0;
+        for (uint32_t c = lane & 7u; c < 3 * (uint32_t)days; c += 8) {
+            const int2 v = tile.s[r][c];
+            if (wide) {
+                *reinterpret_cast<int2*>(to + 2 * c) = v;
+            } else {
+                to[2 * c] = v.x;
+                to[2 * c + 1] = v.y;
+            }
+        }
+    }
+    __syncwarp();
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kTrajThreads) abc_simulate_kernel(const __grid_constant__ ModelParams p,
+                                                                    const __grid_constant__ SimulateArgs a)
+{
+    __shared__ TrajRows tiles[kTrajThreads / 32];
+    const uint32_t lane = threadIdx.x & 31u;
+    TrajRows& tile = tiles[threadIdx.x >> 5];
+    const bool wide = (reinterpret_cast<uintptr_t>(a.traj_out) & 7u) == 0;
+    const int32_t T = p.T;
+    const auto put = [&](int32_t slot, const State& x) {
+        int2* to = &tile.s[lane][3 * slot];
+        to[0] = make_int2(x.S, x.I);
+        to[1] = make_int2(x.A, x.R);
+        to[2] = make_int2(x.D, x.Ru);
+    };
+    const uint64_t step = (uint64_t)gridDim.x * kTrajThreads;
+    for (uint64_t b0 = (uint64_t)blockIdx.x * kTrajThreads + (threadIdx.x & ~31u); b0 < a.B; b0 += step) {
+        const uint32_t rows = (uint32_t)min(a.B - b0, (uint64_t)32);
+        const uint64_t b = b0 + min(lane, rows - 1);   // lanes past the end repeat the last row, unwritten
+        const uint64_t i = a.sample_index[b];
+        int32_t* out = a.traj_out + (size_t)b0 * 6 * (size_t)(T + 1);
         float th[8];
         const float4* ti = reinterpret_cast<const float4*>(a.theta + 8 * b);
         const float4 t0 = ti[0], t1 = ti[1];
         th[0] = t0.x; th[1] = t0.y; th[2] = t0.z; th[3] = t0.w;
         th[4] = t1.x; th[5] = t1.y; th[6] = t1.z; th[7] = t1.w;
         const Theta t = make_theta<MODE>(th, p.inv_p);
-        const State x0 = init_state(t, p.A0, p.R0, p.D0, p.room0);
-        TrajVisit v{a.traj_out + (size_t)b * 6 * (size_t)(p.T + 1)};
-        v(0, x0);
-        simulate_sample<MODE>(p, a.sample_index[b], t, x0, obs_s, v);
+        State x = init_state(t, p.A0, p.R0, p.D0, p.room0);
+        put(0, x);
+        write_days(tile, out, rows, T, 0, 1, wide);
+        const uint32_t n_pairs = (uint32_t)(T + 1) >> 1;
+        int32_t slot = 0;
+        for (uint32_t k = 1; k <= n_pairs; ++k) {
+            float z[10];
+            day_pair_normals<MODE>(p, i, k, z);
+            const int32_t d1 = (int32_t)(2 * k - 1);
+            model_day<MODE>(x, t, p.inv_p, z);
+            put(slot++, x);
+            if (d1 < T) {
+                model_day<MODE>(x, t, p.inv_p, z + 5);
+                put(slot++, x);
+            }
+            if (slot == kTrajDays || k == n_pairs) {
+                const int32_t last = min(d1 + 1, T);
+                write_days(tile, out, rows, T, last - slot + 1, slot, wide);
+                slot = 0;
+            }
+        }
     }
 }
 
@@ -285,92 +334,11 @@ __global__ void __launch_bounds__(kBlockThreads) abc_step_kernel(const __grid_co
 }
 
 // ---------------------------------------------------------------------------
-// Quantile bands of trajectories: one block per (day, compartment) column,
-// the B values sorted in shared memory by a bitonic network (padded to a power
-// of two with INT_MAX), then order statistics floor(q (B - 1)).
-// ---------------------------------------------------------------------------
-constexpr int kBandThreads = 1024;
-constexpr uint32_t kBandMaxB = 8192;   // the largest B the C ABI accepts (power of two)
-
-__global__ void __launch_bounds__(kBandThreads) band_kernel(const int32_t* __restrict__ traj, uint32_t B, int32_t T,
-                                                             const float* __restrict__ qpos, int32_t n_q,
-                                                             float* __restrict__ bands)
-{
-    extern __shared__ int32_t v[];
-    const int32_t d = blockIdx.x / 3, c = blockIdx.x % 3;
-    uint32_t n2 = 1;
-    while (n2 < B) n2 <<= 1;
-    for (uint32_t b = threadIdx.x; b < n2; b += blockDim.x)
-        v[b] = b < B ? traj[((size_t)b * (T + 1) + d) * 6 + 2 + c] : 0x7FFFFFFF;
-    __syncthreads();
-    // bitonic sort; each stage visits its n2 / 2 compare-exchange pairs
-    // (i, i + j), i with bit j clear, rather than all n2 positions
-    for (uint32_t k = 2; k <= n2; k <<= 1) {
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t q = threadIdx.x; q < n2 / 2; q += blockDim.x) {
-                const uint32_t i = ((q & ~(j - 1)) << 1) | (q & (j - 1)), p = i | j;
-                const bool up = (i & k) == 0;
-                const int32_t a = v[i], b2 = v[p];
-                if ((a > b2) == up) {
-                    v[i] = b2;
-                    v[p] = a;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    for (int32_t k = threadIdx.x; k < n_q; k += blockDim.x) {
-        const uint32_t r = (uint32_t)qpos[k];
-        bands[((size_t)k * (T + 1) + d) * 3 + c] = (float)v[r];
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-// Resident blocks per SM times the SM count, for a kernel, dynamic shared
-// memory size and device; looked up once and cached (the launch path then
-// makes no occupancy query). The kernel's dynamic shared-memory limit is one
-// value per kernel and device: it is only ever raised, to the largest size
-// launched so far, so a call with a shorter horizon never lowers it below
-// what a cached longer one needs.
-template <typename K>
-static cudaError_t grid_for(K kernel, size_t smem, int* grid)
+static int blocks_for(uint64_t n, int cap, int threads = kBlockThreads)
 {
-    static std::mutex mu;
-    static std::map<std::tuple<const void*, int, size_t>, int> cache;
-    static std::map<std::pair<const void*, int>, size_t> limit;   // largest limit set per kernel and device
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    if (smem > 48 * 1024) {
-        size_t& lim = limit[std::make_pair((const void*)kernel, dev)];
-        if (lim < smem) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            lim = smem;
-        }
-    }
-    const auto key = std::make_tuple((const void*)kernel, dev, smem);
-    auto it = cache.find(key);
-    if (it != cache.end()) {
-        *grid = it->second;
-        return cudaSuccess;
-    }
-    int sms = 0, per_sm = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlockThreads, smem);
-    if (e != cudaSuccess) return e;
-    *grid = sms * (per_sm > 0 ? per_sm : 1);
-    cache[key] = *grid;
-    return cudaSuccess;
-}
-
-static int blocks_for(uint64_t n, int cap)
-{
-    const uint64_t b = (n + kBlockThreads - 1) / kBlockThreads;
+    const uint64_t b = (n + threads - 1) / threads;
     return (int)(b < (uint64_t)cap ? (b > 0 ? b : 1) : (uint64_t)cap);
 }
 
@@ -399,14 +367,11 @@ static cudaError_t launch_reject_m(const ModelParams& p, const RejectArgs& a, cu
     return below62 ? launch_reject_t<MODE, true>(p, a, s, blocks_out) : launch_reject_t<MODE, false>(p, a, s, blocks_out);
 }
 
-#define ABC_MODE_DISPATCH(fn, mode, ...)                        \
-    ((mode) == kFast ? fn<kFast>(__VA_ARGS__)                   \
-     : (mode) == kExact ? fn<kExact>(__VA_ARGS__)               \
-     : (mode) == (kFast | kLiteral) ? fn<kFast | kLiteral>(__VA_ARGS__) \
-                                  : fn<kExact | kLiteral>(__VA_ARGS__))
-
 cudaError_t launch_reject(const ModelParams& p, const RejectArgs& a, int mode, cudaStream_t s, int* blocks_out)
 {
+    bool taken = false;
+    const cudaError_t e = launch_staged_reject(p, a, mode, s, blocks_out, &taken);
+    if (e != cudaSuccess || taken) return e;
     return ABC_MODE_DISPATCH(launch_reject_m, mode, p, a, s, blocks_out);
 }
 
@@ -424,23 +389,28 @@ static cudaError_t launch_distances_m(const ModelParams& p, const DistanceArgs& 
 
 cudaError_t launch_distances(const ModelParams& p, const DistanceArgs& a, int mode, cudaStream_t s)
 {
+    bool taken = false;
+    const cudaError_t e = launch_staged_distances(p, a, mode, s, &taken);
+    if (e != cudaSuccess || taken) return e;
     return ABC_MODE_DISPATCH(launch_distances_m, mode, p, a, s);
 }
 
 template <int MODE>
 static cudaError_t launch_simulate_m(const ModelParams& p, const SimulateArgs& a, cudaStream_t s)
 {
-    const size_t smem = sizeof(int4) * (size_t)(p.T + 1);
     int grid = 0;
-    cudaError_t e = grid_for(abc_simulate_kernel<MODE>, smem, &grid);
+    cudaError_t e = grid_for(abc_simulate_kernel<MODE>, 0, &grid, kTrajThreads);
     if (e != cudaSuccess) return e;
-    grid = blocks_for(a.B, grid);
-    abc_simulate_kernel<MODE><<<grid, kBlockThreads, smem, s>>>(p, a);
+    grid = blocks_for(a.B, grid, kTrajThreads);
+    abc_simulate_kernel<MODE><<<grid, kTrajThreads, 0, s>>>(p, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_simulate(const ModelParams& p, const SimulateArgs& a, int mode, cudaStream_t s)
 {
+    bool taken = false;
+    const cudaError_t e = launch_staged_simulate(p, a, mode, s, &taken);
+    if (e != cudaSuccess || taken) return e;
     return ABC_MODE_DISPATCH(launch_simulate_m, mode, p, a, s);
 }
 
@@ -458,32 +428,6 @@ static cudaError_t launch_step_m(const ModelParams& p, const StepArgs& a, cudaSt
 cudaError_t launch_step(const ModelParams& p, const StepArgs& a, int mode, cudaStream_t s)
 {
     return ABC_MODE_DISPATCH(launch_step_m, mode, p, a, s);
-}
-
-cudaError_t launch_bands(const int32_t* traj, uint32_t B, int32_t T, const float* qpos, int32_t n_q, float* bands,
-                         cudaStream_t s)
-{
-    if (B < 1 || B > kBandMaxB) return cudaErrorInvalidValue;
-    uint32_t n2 = 1;
-    while (n2 < B) n2 <<= 1;
-    const size_t smem = sizeof(int32_t) * n2;
-    if (smem > 48 * 1024) {
-        // set once per device to the largest size B <= ABC_PROJECT_MAX_B can need
-        static std::mutex mu;
-        static std::map<int, bool> done;
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        std::lock_guard<std::mutex> lock(mu);
-        if (!done[dev]) {
-            e = cudaFuncSetAttribute(band_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(sizeof(int32_t) * kBandMaxB));
-            if (e != cudaSuccess) return e;
-            done[dev] = true;
-        }
-    }
-    band_kernel<<<3 * (T + 1), kBandThreads, smem, s>>>(traj, B, T, qpos, n_q, bands);
-    return cudaGetLastError();
 }
 
 }  // namespace abcgb

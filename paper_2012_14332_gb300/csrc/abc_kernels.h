@@ -73,6 +73,26 @@ struct SimulateArgs {
     int32_t* traj_out;            // device [B][T+1][6]
 };
 
+// Trajectories of the observed compartments by column, [T + 1][3][stride], and
+// the order statistics of each column's B counts.
+struct ColumnArgs {
+    const float* theta;           // device [B][8]
+    const uint64_t* sample_index; // device [B]
+    uint64_t B;
+    int32_t* out;
+    size_t stride;                // >= B
+};
+constexpr int kBandRanks = 32;
+struct BandArgs {
+    const int32_t* columns;
+    size_t stride;
+    uint32_t B;                   // 1 .. 8192
+    int32_t n_q;
+    const uint32_t* qpos_dev;     // device [n_q] 0-based ranks, or NULL: the first kBandRanks in qpos
+    uint32_t qpos[kBandRanks];
+    float* bands;                 // device [n_q][T + 1][3]
+};
+
 struct StepArgs {
     const float* theta;           // device [B][8]
     const int32_t* state_in;      // device [B][6]
@@ -140,8 +160,14 @@ cudaError_t launch_reject(const ModelParams& p, const RejectArgs& a, int mode, c
 cudaError_t launch_distances(const ModelParams& p, const DistanceArgs& a, int mode, cudaStream_t s);
 cudaError_t launch_simulate(const ModelParams& p, const SimulateArgs& a, int mode, cudaStream_t s);
 cudaError_t launch_step(const ModelParams& p, const StepArgs& a, int mode, cudaStream_t s);
-cudaError_t launch_bands(const int32_t* traj, uint32_t B, int32_t T, const float* qpos, int32_t n_q, float* bands,
-                         cudaStream_t s);
+// the same for calls of at most one wave of staged blocks (abc_staged.cu):
+// *taken tells whether the call was one; the three above ask these first
+cudaError_t launch_staged_reject(const ModelParams& p, const RejectArgs& a, int mode, cudaStream_t s, int* blocks_out,
+                                 bool* taken);
+cudaError_t launch_staged_distances(const ModelParams& p, const DistanceArgs& a, int mode, cudaStream_t s, bool* taken);
+cudaError_t launch_staged_simulate(const ModelParams& p, const SimulateArgs& a, int mode, cudaStream_t s, bool* taken);
+cudaError_t launch_columns(const ModelParams& p, const ColumnArgs& a, int mode, cudaStream_t s);
+cudaError_t launch_bands(const BandArgs& a, int32_t T, cudaStream_t s);   // after launch_columns, overlapping its end
 // The k-th smallest of n distances (abc_select.cu), all on the device. In a
 // SelectWork whose first kSelectZeroBytes are zero launch_kth_bracket leaves
 // st.bad, the number of invalid keys (NaN, sign bit set), and, if there are none
