@@ -67,8 +67,11 @@ struct LaneRegion {
 // 64-bit shared-memory atomic cost 5 % of a 16-region run and 3 % of a
 // three-region one. The autotuner chooses between the two forms; it takes the
 // lean form on both workloads.
+//
+// Exact mode is bounded to the registers of 768 threads an SM: left alone, its
+// straight-line arithmetic takes 128 a thread.
 template <int MODE, int BLOCK, int PAIRS, bool BELOW62, bool OBS_S, bool LEAN>
-__global__ void __launch_bounds__(BLOCK, LEAN ? 4 : 1) abc_batch_kernel(const __grid_constant__ ModelParams p,
+__global__ void __launch_bounds__(BLOCK, LEAN ? 4 : is_fast(MODE) ? 1 : 768 / BLOCK) abc_batch_kernel(const __grid_constant__ ModelParams p,
                                                           const __grid_constant__ BatchArgs a)
 {
     __shared__ RegionDev reg_s[kMaxRegions];
