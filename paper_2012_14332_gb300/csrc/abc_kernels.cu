@@ -37,7 +37,6 @@ __device__ __forceinline__ void stage_observed(int4* obs_s, const int4* __restri
 // and one atomicAdd per warp; their theta is re-drawn from the index.
 // ---------------------------------------------------------------------------
 constexpr int kRing = 64;
-constexpr int kWarpsPerBlock = kBlockThreads / 32;
 // A warp hands new samples to its idle lanes once at least kRefillMinIdle of
 // them are idle (all 32 always qualify): the hand-out (ring read, derived
 // parameters, initial state) runs on the whole warp, while a lane left idle
@@ -222,7 +221,8 @@ __global__ void __launch_bounds__(kBlockThreads) abc_distance_kernel(const __gri
 
 // ---------------------------------------------------------------------------
 // K3: trajectories of given (theta, sample index) pairs, whole rows
-// [T + 1][6] (S, I, A, R, D, Ru), a thread per sample. A warp keeps kTrajDays
+// [T + 1][6] (S, I, A, R, D, Ru), a thread per sample (exact arithmetic only:
+// see the rule in abc_staged.cu). A warp keeps kTrajDays
 // days of its 32 rows in shared memory and then writes each row's days as one
 // run of 8-byte words: a lane storing its own six values a day touched 32
 // sectors with every 4 bytes. ALU-bound now: 100,003 rows over 90 days in exact arithmetic
@@ -342,21 +342,29 @@ static int blocks_for(uint64_t n, int cap, int threads = kBlockThreads)
     return (int)(b < (uint64_t)cap ? (b > 0 ? b : 1) : (uint64_t)cap);
 }
 
-size_t reject_smem_bytes(int32_t T) { return sizeof(int4) * (size_t)(T + 1) + sizeof(WarpRing) * kWarpsPerBlock; }
+// Threads of a block of the two kernels that stage the series: small blocks
+// deal a call of a few waves out evenly (65,536 samples are 256 blocks of 256
+// threads: two on some SMs, one on others), unless the series takes so much
+// shared memory that small blocks would not fill an SM. Distances over 90 days
+// in exact mode: 55,000 samples 103 -> 84 us, 2e6 unchanged.
+constexpr int kSmallBlock = 64;
+constexpr int32_t kSmallBlockT = 400;
+static int series_block_threads(int32_t T) { return T <= kSmallBlockT ? kSmallBlock : kBlockThreads; }
 
 template <int MODE, bool BELOW62>
 static cudaError_t launch_reject_t(const ModelParams& p, const RejectArgs& a, cudaStream_t s, int* blocks_out)
 {
-    const size_t smem = reject_smem_bytes(p.T);
+    const int threads = series_block_threads(p.T), warps = threads / 32;
+    const size_t smem = sizeof(int4) * (size_t)(p.T + 1) + sizeof(WarpRing) * warps;
     int grid = 0;
-    cudaError_t e = grid_for(abc_reject_kernel<MODE, BELOW62>, smem, &grid);
+    cudaError_t e = grid_for(abc_reject_kernel<MODE, BELOW62>, smem, &grid, threads);
     if (e != cudaSuccess) return e;
     // persistent: every resident block loops over claimed index chunks
     const uint64_t chunks = (a.n_samples + 31) / 32;
-    const uint64_t want = (chunks + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    const uint64_t want = (chunks + warps - 1) / warps;
     if (want < (uint64_t)grid) grid = (int)(want > 0 ? want : 1);
     if (blocks_out) *blocks_out = grid;
-    abc_reject_kernel<MODE, BELOW62><<<grid, kBlockThreads, smem, s>>>(p, a);
+    abc_reject_kernel<MODE, BELOW62><<<grid, threads, smem, s>>>(p, a);
     return cudaGetLastError();
 }
 
@@ -380,10 +388,11 @@ static cudaError_t launch_distances_m(const ModelParams& p, const DistanceArgs& 
 {
     const size_t smem = sizeof(int4) * (size_t)(p.T + 1);
     int grid = 0;
-    cudaError_t e = grid_for(abc_distance_kernel<MODE>, smem, &grid);
+    const int threads = series_block_threads(p.T);
+    cudaError_t e = grid_for(abc_distance_kernel<MODE>, smem, &grid, threads);
     if (e != cudaSuccess) return e;
-    grid = blocks_for(a.n_samples, grid);
-    abc_distance_kernel<MODE><<<grid, kBlockThreads, smem, s>>>(p, a);
+    grid = blocks_for(a.n_samples, grid, threads);
+    abc_distance_kernel<MODE><<<grid, threads, smem, s>>>(p, a);
     return cudaGetLastError();
 }
 
@@ -411,7 +420,8 @@ cudaError_t launch_simulate(const ModelParams& p, const SimulateArgs& a, int mod
     bool taken = false;
     const cudaError_t e = launch_staged_simulate(p, a, mode, s, &taken);
     if (e != cudaSuccess || taken) return e;
-    return ABC_MODE_DISPATCH(launch_simulate_m, mode, p, a, s);
+    // fast mode is always staged
+    return mode == kExact ? launch_simulate_m<kExact>(p, a, s) : launch_simulate_m<kExact | kLiteral>(p, a, s);
 }
 
 template <int MODE>

@@ -154,7 +154,6 @@ cudaError_t launch_batch(const ModelParams& p, const BatchArgs& a, bool fast, bo
 cudaError_t launch_advance(RegionDev* regions, int32_t n_regions, cudaStream_t s);
 cudaError_t prepare_batch(bool fast, bool below62, int32_t n_obs_smem, const BatchShape& shape);
 
-size_t reject_smem_bytes(int32_t T);
 // mode: kExact or kFast, optionally | kLiteral (see abc_model.cuh)
 cudaError_t launch_reject(const ModelParams& p, const RejectArgs& a, int mode, cudaStream_t s, int* blocks_out);
 cudaError_t launch_distances(const ModelParams& p, const DistanceArgs& a, int mode, cudaStream_t s);

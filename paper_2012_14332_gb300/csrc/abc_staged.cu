@@ -6,9 +6,9 @@
 // on a chip that is mostly idle when there are a few thousand samples. Only the
 // model day depends on the day before; the normals (Philox and Box-Muller, more
 // than half of a day's instructions) depend on the sample's index alone. So a
-// block here has 32 samples: kProducers warps draw the normals of a stage of
-// kProducers day pairs ahead, one pair each, into shared memory, and one warp
-// walks the model through them. The arithmetic of a sample is that of a thread
+// block here has 32 samples: P warps draw the normals of a stage of P day pairs
+// ahead, one pair each, into shared memory, and one warp walks the model
+// through them. The arithmetic of a sample is that of a thread
 // per sample, instruction for instruction, and so are the results.
 // Latency-bound: the model days' chain. On the device, fast arithmetic over 120
 // days: 100 trajectories 39 -> 21 us, 8192 102 -> 23 us; exact arithmetic over
@@ -25,12 +25,16 @@ namespace abcgb {
 
 namespace {
 
-constexpr int kProducers = 3;
-constexpr int kStagedThreads = 32 * (kProducers + 1);
-constexpr int kStageDays = 2 * kProducers;
+// Warps that draw: two keep up with a walk that only sums a distance, and leave
+// room for more blocks; three share the writing of trajectories (1000 of 90
+// days, fast: 12.5 us, 18.6 us with two).
+constexpr int kSumProducers = 2;
+constexpr int kWriteProducers = 3;
+constexpr int staged_threads(int producers) { return 32 * (producers + 1); }
 
+template <int P>
 struct Stage {
-    float z[kProducers][10][32];   // normals of one day pair per producer: [pair][draw][lane]
+    float z[P][10][32];   // normals of one day pair per producer: [pair][draw][lane]
 };
 
 // Runs the block's 32 samples (lane's sample index i, walked by the last warp
@@ -38,16 +42,16 @@ struct Stage {
 // walking warp (day), a call after each day pair (pair; false ends the block
 // early once no lane wants to go on, if it can stop at all), and a call from
 // the producers after each stage (drain, for the stage before).
-template <int MODE, typename Sink>
-__device__ __forceinline__ void staged_days(const ModelParams& p, uint64_t i, const Theta& t, State x, Stage (&zs)[2],
-                                            Sink& sink)
+template <int MODE, int P, typename Sink>
+__device__ __forceinline__ void staged_days(const ModelParams& p, uint64_t i, const Theta& t, State x,
+                                            Stage<P> (&zs)[2], Sink& sink)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t T = p.T;
-    const uint32_t n_pairs = (uint32_t)(T + 1) >> 1, stages = (n_pairs + kProducers - 1) / kProducers;
-    const bool walks = warp == kProducers;
+    const uint32_t n_pairs = (uint32_t)(T + 1) >> 1, stages = (n_pairs + P - 1) / P;
+    const bool walks = warp == P;
     const auto produce = [&](uint32_t st) {
-        const uint32_t k = st * kProducers + warp + 1;
+        const uint32_t k = st * P + warp + 1;
         if (k > n_pairs) return;
         float z[10];
         day_pair_normals<MODE>(p, i, k, z);
@@ -63,8 +67,8 @@ __device__ __forceinline__ void staged_days(const ModelParams& p, uint64_t i, co
             if (st > 0) sink.drain(st - 1, T);
         } else {
 #pragma unroll
-            for (int q = 0; q < kProducers; ++q) {
-                const uint32_t k = st * kProducers + q + 1;
+            for (int q = 0; q < P; ++q) {
+                const uint32_t k = st * P + q + 1;
                 if (k > n_pairs) continue;
                 float z[10];
 #pragma unroll
@@ -90,7 +94,7 @@ __device__ __forceinline__ void staged_days(const ModelParams& p, uint64_t i, co
 
 __device__ __forceinline__ void stage_series(int4* obs_s, const int4* __restrict__ obs, int32_t T)
 {
-    for (int32_t d = threadIdx.x; d <= T; d += kStagedThreads) obs_s[d] = obs[d];
+    for (int32_t d = threadIdx.x; d <= T; d += blockDim.x) obs_s[d] = obs[d];
     // read after staged_days' first barrier
 }
 
@@ -105,14 +109,14 @@ struct DistanceSink {
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(kStagedThreads) staged_distance_kernel(const __grid_constant__ ModelParams p,
+__global__ void __launch_bounds__(staged_threads(kSumProducers)) staged_distance_kernel(const __grid_constant__ ModelParams p,
                                                                          const __grid_constant__ DistanceArgs a)
 {
     extern __shared__ int4 obs_s[];
-    __shared__ Stage zs[2];
+    __shared__ Stage<kSumProducers> zs[2];
     stage_series(obs_s, a.obs, p.T);
     const uint64_t j = (uint64_t)blockIdx.x * 32 + (threadIdx.x & 31), i = a.first_index + j;
-    const bool walks = threadIdx.x >= 32 * kProducers;
+    const bool walks = threadIdx.x >= 32 * kSumProducers;
     float th[8];
     Theta t{};
     State x{};
@@ -122,7 +126,7 @@ __global__ void __launch_bounds__(kStagedThreads) staged_distance_kernel(const _
         x = init_state(t, p.A0, p.R0, p.D0, p.room0);
     }
     DistanceSink sink{obs_s};
-    staged_days<MODE>(p, i, t, x, zs, sink);
+    staged_days<MODE, kSumProducers>(p, i, t, x, zs, sink);
     if (!walks || j >= a.n_samples) return;
     a.dist_out[j] = __dsqrt_rn(__ull2double_rn(sink.acc));
     if (a.theta_out) {
@@ -167,15 +171,15 @@ struct RejectSink {
 };
 
 template <int MODE, bool BELOW62>
-__global__ void __launch_bounds__(kStagedThreads) staged_reject_kernel(const __grid_constant__ ModelParams p,
+__global__ void __launch_bounds__(staged_threads(kSumProducers)) staged_reject_kernel(const __grid_constant__ ModelParams p,
                                                                        const __grid_constant__ RejectArgs a)
 {
     extern __shared__ int4 obs_s[];
-    __shared__ Stage zs[2];
+    __shared__ Stage<kSumProducers> zs[2];
     stage_series(obs_s, a.obs, p.T);
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t j = (uint64_t)blockIdx.x * 32 + lane, i = a.first_index + j;
-    const bool walks = threadIdx.x >= 32 * kProducers;
+    const bool walks = threadIdx.x >= 32 * kSumProducers;
     float th[8];
     Theta t{};
     State x{};
@@ -187,7 +191,7 @@ __global__ void __launch_bounds__(kStagedThreads) staged_reject_kernel(const __g
     // the claim counter stands at or above n_samples afterwards, as when chunks are claimed
     if (threadIdx.x == 0) atomicAdd(a.next, 32ull);
     RejectSink<BELOW62> sink{obs_s, a.acc_max, 0, 0, 0, 0, walks && j < a.n_samples, false};
-    staged_days<MODE>(p, i, t, x, zs, sink);
+    staged_days<MODE, kSumProducers>(p, i, t, x, zs, sink);
     if (!walks) return;
     const uint32_t mask = __ballot_sync(0xFFFFFFFFu, sink.accept);
     if (mask) {
@@ -213,8 +217,9 @@ __global__ void __launch_bounds__(kStagedThreads) staged_reject_kernel(const __g
 // shared memory and the producers write them out during the next stage, a row's
 // days as one run of 8-byte words (the rows are 24 (T + 1) bytes apart; a lane
 // storing its own six values a day touched 32 sectors with every 4 bytes).
+constexpr int kTileDays = 2 * kWriteProducers;   // a stage
 struct TrajTile {
-    int2 s[32][3 * kStageDays + 1];   // one row's days; the odd stride (in 8 bytes) spreads lanes over the banks
+    int2 s[32][3 * kTileDays + 1];   // one row's days; the odd stride (in 8 bytes) spreads lanes over the banks
 };
 
 struct TrajSink {
@@ -233,14 +238,14 @@ struct TrajSink {
     }
     __device__ __forceinline__ bool pair(int32_t d1, int32_t, const State&)
     {
-        stage = (uint32_t)(d1 + 1) / kStageDays;   // the next pair's stage
+        stage = (uint32_t)(d1 + 1) / kTileDays;   // the next pair's stage
         return true;
     }
     __device__ __forceinline__ void drain(uint32_t st, int32_t T)
     {
-        const int32_t d0 = (int32_t)st * kStageDays + 1, days = min(kStageDays, T - d0 + 1);
-        if (days == kStageDays)
-            copy<3 * kStageDays>(tiles[st & 1], 0, d0, T);
+        const int32_t d0 = (int32_t)st * kTileDays + 1, days = min(kTileDays, T - d0 + 1);
+        if (days == kTileDays)
+            copy<3 * kTileDays>(tiles[st & 1], 0, d0, T);
         else
             copy<0>(tiles[st & 1], 3 * (uint32_t)days, d0, T);
     }
@@ -249,7 +254,7 @@ struct TrajSink {
     __device__ __forceinline__ void copy(const TrajTile& tile, uint32_t n, int32_t d0, int32_t T)
     {
         const uint32_t words = WORDS ? WORDS : n;
-        for (uint32_t u = threadIdx.x; u < rows * words; u += 32 * kProducers) {
+        for (uint32_t u = threadIdx.x; u < rows * words; u += 32 * kWriteProducers) {
             const uint32_t r = u / words, c = u - r * words;
             const int2 v = tile.s[r][c];
             int32_t* to = out + (size_t)r * 6 * (T + 1) + 6 * (size_t)d0 + 2 * c;
@@ -272,10 +277,10 @@ __device__ __forceinline__ void load_theta(const float* __restrict__ src, float 
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kStagedThreads) staged_simulate_kernel(const __grid_constant__ ModelParams p,
+__global__ void __launch_bounds__(staged_threads(kWriteProducers)) staged_simulate_kernel(const __grid_constant__ ModelParams p,
                                                                          const __grid_constant__ SimulateArgs a)
 {
-    __shared__ Stage zs[2];
+    __shared__ Stage<kWriteProducers> zs[2];
     __shared__ TrajTile tiles[2];
     const uint64_t b0 = (uint64_t)blockIdx.x * 32;
     const uint32_t lane = threadIdx.x & 31, rows = (uint32_t)min(a.B - b0, (uint64_t)32);
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(kStagedThreads) staged_simulate_kernel(const _
     int32_t* out = a.traj_out + (size_t)b0 * 6 * (size_t)(p.T + 1);
     Theta t{};
     State x{};
-    if (threadIdx.x >= 32 * kProducers) {
+    if (threadIdx.x >= 32 * kWriteProducers) {
         float th[8];
         load_theta(a.theta + 8 * b, th);
         t = make_theta<MODE>(th, p.inv_p);
@@ -295,7 +300,7 @@ __global__ void __launch_bounds__(kStagedThreads) staged_simulate_kernel(const _
         }
     }
     TrajSink sink{tiles, out, rows, 0, (reinterpret_cast<uintptr_t>(a.traj_out) & 7u) == 0};
-    staged_days<MODE>(p, i, t, x, zs, sink);
+    staged_days<MODE, kWriteProducers>(p, i, t, x, zs, sink);
 }
 
 // The observed compartments as columns [T + 1][3][stride], what the bands read.
@@ -316,24 +321,24 @@ struct ColumnSink {
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(kStagedThreads) staged_columns_kernel(const __grid_constant__ ModelParams p,
+__global__ void __launch_bounds__(staged_threads(kWriteProducers)) staged_columns_kernel(const __grid_constant__ ModelParams p,
                                                                         const __grid_constant__ ColumnArgs a)
 {
-    __shared__ Stage zs[2];
+    __shared__ Stage<kWriteProducers> zs[2];
     griddep_release();   // the band kernel's blocks may come in and wait
     const uint64_t row = (uint64_t)blockIdx.x * 32 + (threadIdx.x & 31), b = min(row, a.B - 1);
     const uint64_t i = a.sample_index[b];
     Theta t{};
     State x{};
     ColumnSink sink{row < a.B ? a.out + row : nullptr, a.stride};
-    if (threadIdx.x >= 32 * kProducers) {
+    if (threadIdx.x >= 32 * kWriteProducers) {
         float th[8];
         load_theta(a.theta + 8 * b, th);
         t = make_theta<MODE>(th, p.inv_p);
         x = init_state(t, p.A0, p.R0, p.D0, p.room0);
         sink.day(0, 0, x);
     }
-    staged_days<MODE>(p, i, t, x, zs, sink);
+    staged_days<MODE, kWriteProducers>(p, i, t, x, zs, sink);
 }
 
 // ---------------------------------------------------------------------------
@@ -461,18 +466,25 @@ __global__ void __launch_bounds__(THREADS) band_kernel(const __grid_constant__ B
 
 unsigned blocks_of_32(uint64_t n) { return (unsigned)((n + 31) / 32); }
 
-// The rule between the staged kernels and a thread per sample: staged while
-// all blocks are resident at once. Beyond that the chip is full either way,
-// and passing the normals through shared memory is only more work. Distances
-// over 90 days, exact arithmetic: 40,000 samples 114 us staged, 161 us with a
-// thread each; 65,536 samples (more than a wave) 188 and 167 us. Fast: 65,536
-// samples 55 and 56 us, 400,000 251 and 236 us.
+// The rule between the staged kernels and a thread per sample, in waves of
+// resident staged blocks. Once a thread per sample fills the chip, passing the
+// normals through shared memory is only more work; rejection gains longest,
+// since its blocks end with their last sample, and fast trajectories always
+// (the warps that draw also write). Both sides on the device, 90 days:
+//   distances   exact 30,000 samples 63 us staged, 65 us plain; 45,000 80 and
+//               83; 55,000 92 and 84; fast 20,000 26 and 32; 55,000 45 and 42
+//   rejection   exact 65,536 82 and 90; 150,000 143 and 150; 300,000 253 and
+//               208; fast 150,000 68 and 74; 300,000 119 and 102
+//   trajectories exact 30,000 76 and 84; 45,000 123 and 105; fast 100,003 82
+//               and 102; 300,000 230 and 303
+constexpr double kDistanceWaves = 1.0, kRejectWaves = 3.0, kExactSimulateWaves = 1.0;
+
 template <typename K>
-cudaError_t one_wave(K kernel, size_t smem, uint64_t n, bool* fits)
+cudaError_t within_waves(K kernel, size_t smem, int producers, double waves, uint64_t n, bool* fits)
 {
     int resident = 0;
-    const cudaError_t e = grid_for(kernel, smem, &resident, kStagedThreads);
-    *fits = e == cudaSuccess && n <= 32ull * resident;
+    const cudaError_t e = grid_for(kernel, smem, &resident, staged_threads(producers));
+    *fits = e == cudaSuccess && (double)n <= waves * 32.0 * resident;
     return e;
 }
 
@@ -480,9 +492,9 @@ template <int MODE>
 cudaError_t distances_m(const ModelParams& p, const DistanceArgs& a, cudaStream_t s, bool* taken)
 {
     const size_t smem = sizeof(int4) * (size_t)(p.T + 1);
-    cudaError_t e = one_wave(staged_distance_kernel<MODE>, smem, a.n_samples, taken);
+    cudaError_t e = within_waves(staged_distance_kernel<MODE>, smem, kSumProducers, kDistanceWaves, a.n_samples, taken);
     if (e != cudaSuccess || !*taken) return e;
-    staged_distance_kernel<MODE><<<blocks_of_32(a.n_samples), kStagedThreads, smem, s>>>(p, a);
+    staged_distance_kernel<MODE><<<blocks_of_32(a.n_samples), staged_threads(kSumProducers), smem, s>>>(p, a);
     return cudaGetLastError();
 }
 
@@ -490,11 +502,11 @@ template <int MODE, bool BELOW62>
 cudaError_t reject_t(const ModelParams& p, const RejectArgs& a, cudaStream_t s, int* blocks_out, bool* taken)
 {
     const size_t smem = sizeof(int4) * (size_t)(p.T + 1);
-    cudaError_t e = one_wave(staged_reject_kernel<MODE, BELOW62>, smem, a.n_samples, taken);
+    cudaError_t e = within_waves(staged_reject_kernel<MODE, BELOW62>, smem, kSumProducers, kRejectWaves, a.n_samples, taken);
     if (e != cudaSuccess || !*taken) return e;
     const unsigned blocks = blocks_of_32(a.n_samples);
     if (blocks_out) *blocks_out = (int)blocks;
-    staged_reject_kernel<MODE, BELOW62><<<blocks, kStagedThreads, smem, s>>>(p, a);
+    staged_reject_kernel<MODE, BELOW62><<<blocks, staged_threads(kSumProducers), smem, s>>>(p, a);
     return cudaGetLastError();
 }
 
@@ -508,16 +520,19 @@ cudaError_t reject_m(const ModelParams& p, const RejectArgs& a, cudaStream_t s, 
 template <int MODE>
 cudaError_t simulate_m(const ModelParams& p, const SimulateArgs& a, cudaStream_t s, bool* taken)
 {
-    cudaError_t e = one_wave(staged_simulate_kernel<MODE>, 0, a.B, taken);
-    if (e != cudaSuccess || !*taken) return e;
-    staged_simulate_kernel<MODE><<<blocks_of_32(a.B), kStagedThreads, 0, s>>>(p, a);
+    *taken = true;
+    if (!is_fast(MODE)) {
+        cudaError_t e = within_waves(staged_simulate_kernel<MODE>, 0, kWriteProducers, kExactSimulateWaves, a.B, taken);
+        if (e != cudaSuccess || !*taken) return e;
+    }
+    staged_simulate_kernel<MODE><<<blocks_of_32(a.B), staged_threads(kWriteProducers), 0, s>>>(p, a);
     return cudaGetLastError();
 }
 
 template <int MODE>
 cudaError_t columns_m(const ModelParams& p, const ColumnArgs& a, cudaStream_t s)
 {
-    staged_columns_kernel<MODE><<<blocks_of_32(a.B), kStagedThreads, 0, s>>>(p, a);
+    staged_columns_kernel<MODE><<<blocks_of_32(a.B), staged_threads(kWriteProducers), 0, s>>>(p, a);
     return cudaGetLastError();
 }
 
