@@ -6,6 +6,7 @@ stream); every step of the method runs in the CUDA library. The library must
 be built (``paper_2012_14332_gb300.build.build()``); there is no fallback.
 """
 import ctypes
+import math
 import os
 import threading
 
@@ -247,23 +248,39 @@ def prior_box(lo=PAPER_LO, hi=PAPER_HI):
     return b
 
 
+# The helpers below run on every call; a call of a few samples takes some 30 us
+# on the device, so each argument is marshalled in well under a microsecond:
+# addresses are plain integers, sizes are multiplied without numpy, and the
+# default prior box (immutable tuples) is laid out once.
+_PAPER_BOX = prior_box()
+
+
+def _box(lo, hi):
+    return ctypes.byref(_PAPER_BOX if lo is PAPER_LO and hi is PAPER_HI else prior_box(lo, hi))
+
+
 def _host_i32(a):
-    a = np.ascontiguousarray(np.asarray(a, dtype=np.int32))
-    return a, a.ctypes.data_as(ctypes.c_void_p)
+    a = np.ascontiguousarray(a, dtype=np.int32)
+    return a, a.__array_interface__["data"][0]
 
 
 def _stream(cuda_stream):
     if cuda_stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(cuda_stream, torch.cuda.Stream):
-        return ctypes.c_void_p(cuda_stream.cuda_stream)
-    return ctypes.c_void_p(int(cuda_stream))
+        return cuda_stream.cuda_stream
+    return int(cuda_stream)
 
 
 def _dev(t, dtype, shape):
     assert t.is_cuda and t.dtype == dtype and t.is_contiguous(), (t.device, t.dtype)
-    assert t.numel() >= int(np.prod(shape)), (t.shape, shape)
-    return ctypes.c_void_p(t.data_ptr())
+    assert t.numel() >= math.prod(shape), (t.shape, shape)
+    return t.data_ptr()
+
+
+def _first(t, m):
+    """t[:m], and t itself where that is all of it."""
+    return t if t.shape[0] == m else t[:m]
 
 
 def abc_sample(observed, N_pop, eps, n_samples, seed, stream=0, mode="fast", first_index=0, lo=PAPER_LO,
@@ -287,15 +304,15 @@ def abc_sample(observed, N_pop, eps, n_samples, seed, stream=0, mode="fast", fir
     else:
         theta, dist, idx = out
     nacc = ctypes.c_uint64(0)
-    b = prior_box(lo, hi)
-    st = L.abc_sample(ctypes.byref(b), obs_p, T, int(N_pop), float(eps), int(n_samples), int(seed), int(stream),
+    b = _box(lo, hi)
+    st = L.abc_sample(b, obs_p, T, int(N_pop), float(eps), int(n_samples), int(seed), int(stream),
                       _mode(mode), int(first_index), _dev(theta, torch.float32, (capacity, 8)),
                       _dev(dist, torch.float64, (capacity,)), _dev(idx, torch.int64, (capacity,)), int(capacity),
                       ctypes.byref(nacc), _stream(cuda_stream))
     _check(L, st, allow=(ABC_ERR_CAPACITY,) if allow_overflow else ())
     n = int(nacc.value)
     m = min(n, capacity)
-    return theta[:m], dist[:m], idx[:m], n
+    return _first(theta, m), _first(dist, m), _first(idx, m), n
 
 
 class Observed:
@@ -350,8 +367,8 @@ def abc_sample_async(obs, eps, n_samples, seed, out, counters, stream=0, mode="f
     capacity = theta.shape[0]
     if counters.dtype != torch.int64 or not counters.is_cuda or counters.numel() < 3 or not counters.is_contiguous():
         raise ValueError("counters must be a contiguous CUDA int64 tensor of >= 3 entries")
-    b = prior_box(lo, hi)
-    _check(L, L.abc_sample_async(ctypes.byref(b), obs.handle, float(eps), int(n_samples), int(seed), int(stream),
+    b = _box(lo, hi)
+    _check(L, L.abc_sample_async(b, obs.handle, float(eps), int(n_samples), int(seed), int(stream),
                                  _mode(mode), int(first_index), _dev(theta, torch.float32, (capacity, 8)),
                                  _dev(dist, torch.float64, (capacity,)), _dev(idx, torch.int64, (capacity,)),
                                  int(capacity), counters.data_ptr(), _stream(cuda_stream)))
@@ -377,8 +394,8 @@ def abc_sample_until(obs, eps, n_target, seed, batch=1 << 22, max_samples=1 << 4
         theta, dist, idx = out
         capacity = theta.shape[0]
     nacc, used = ctypes.c_uint64(0), ctypes.c_uint64(0)
-    b = prior_box(lo, hi)
-    st = L.abc_sample_until(ctypes.byref(b), obs.handle, float(eps), int(n_target), int(batch), int(max_samples),
+    b = _box(lo, hi)
+    st = L.abc_sample_until(b, obs.handle, float(eps), int(n_target), int(batch), int(max_samples),
                             int(seed), int(stream), _mode(mode), int(first_index),
                             _dev(theta, torch.float32, (capacity, 8)), _dev(dist, torch.float64, (capacity,)),
                             _dev(idx, torch.int64, (capacity,)), int(capacity), ctypes.byref(nacc), ctypes.byref(used),
@@ -386,7 +403,7 @@ def abc_sample_until(obs, eps, n_target, seed, batch=1 << 22, max_samples=1 << 4
     _check(L, st, allow=(ABC_ERR_CAPACITY,) if allow_overflow else ())
     n = int(nacc.value)
     m = min(n, capacity)
-    return theta[:m], dist[:m], idx[:m], n, int(used.value)
+    return _first(theta, m), _first(dist, m), _first(idx, m), n, int(used.value)
 
 
 def abc_sample_noalloc(observed, N_pop, eps, n_samples, seed, out, stream=0, mode="fast", first_index=0,
@@ -403,15 +420,15 @@ def abc_sample_noalloc(observed, N_pop, eps, n_samples, seed, out, stream=0, mod
     theta, dist, idx = out
     capacity = theta.shape[0]
     nacc = ctypes.c_uint64(0)
-    b = prior_box(lo, hi)
-    st = L.abc_sample_noalloc(ctypes.byref(b), obs_p, T, int(N_pop), float(eps), int(n_samples), int(seed),
+    b = _box(lo, hi)
+    st = L.abc_sample_noalloc(b, obs_p, T, int(N_pop), float(eps), int(n_samples), int(seed),
                               int(stream), _mode(mode), int(first_index), _dev(theta, torch.float32, (capacity, 8)),
                               _dev(dist, torch.float64, (capacity,)), _dev(idx, torch.int64, (capacity,)),
                               int(capacity), ctypes.byref(nacc), _stream(cuda_stream))
     _check(L, st, allow=(ABC_ERR_CAPACITY,) if allow_overflow else ())
     n = int(nacc.value)
     m = min(n, capacity)
-    return theta[:m], dist[:m], idx[:m], n
+    return _first(theta, m), _first(dist, m), _first(idx, m), n
 
 
 def abc_distances(observed, N_pop, n_samples, seed, stream=0, mode="fast", first_index=0, lo=PAPER_LO, hi=PAPER_HI,
@@ -426,8 +443,8 @@ def abc_distances(observed, N_pop, n_samples, seed, stream=0, mode="fast", first
         theta = torch.empty((n_samples, 8), dtype=torch.float32, device=dev) if want_theta else None
     else:
         dist, theta = out
-    b = prior_box(lo, hi)
-    st = L.abc_distances(ctypes.byref(b), obs_p, T, int(N_pop), int(n_samples), int(seed), int(stream), _mode(mode),
+    b = _box(lo, hi)
+    st = L.abc_distances(b, obs_p, T, int(N_pop), int(n_samples), int(seed), int(stream), _mode(mode),
                          int(first_index), _dev(dist, torch.float64, (n_samples,)),
                          _dev(theta, torch.float32, (n_samples, 8)) if theta is not None else None,
                          _stream(cuda_stream))
@@ -520,8 +537,8 @@ def abc_sample_quantile(observed, N_pop, n_samples, k, seed, stream=0, mode="fas
         capacity = dist.shape[0]
     nacc = ctypes.c_uint64(0)
     eps = ctypes.c_double(0.0)
-    b = prior_box(lo, hi)
-    st = L.abc_sample_quantile(ctypes.byref(b), obs_p, T, int(N_pop), int(n_samples), int(k), int(seed), int(stream),
+    b = _box(lo, hi)
+    st = L.abc_sample_quantile(b, obs_p, T, int(N_pop), int(n_samples), int(k), int(seed), int(stream),
                                _mode(mode), int(first_index), _dev(theta, torch.float32, (capacity, 8)),
                                _dev(dist, torch.float64, (capacity,)), _dev(idx, torch.int64, (capacity,)),
                                int(capacity), ctypes.byref(eps), ctypes.byref(nacc), _stream(cuda_stream))
@@ -561,9 +578,9 @@ class Plan:
                                th.data_ptr() if th is not None else None)
         self.capacity = [int(r.get("capacity", 4096)) for r in regions]
         self.n_regions = len(regions)
-        b = prior_box(lo, hi)
+        b = _box(lo, hi)
         h = ctypes.c_void_p()
-        _check(L, L.abc_plan_create(ctypes.byref(b), arr, len(regions), int(seed), _mode(mode), ctypes.byref(h)))
+        _check(L, L.abc_plan_create(b, arr, len(regions), int(seed), _mode(mode), ctypes.byref(h)))
         self._h = h
 
     def reset(self, cuda_stream=None):
@@ -683,8 +700,8 @@ class Flow:
         L = load()
         self._L = L
         h = ctypes.c_void_p()
-        b = prior_box(lo, hi)
-        _check(L, L.abc_maf_create_multi(int(n_flows), int(n_blocks), int(hidden), ctypes.byref(b), ctypes.byref(h)))
+        b = _box(lo, hi)
+        _check(L, L.abc_maf_create_multi(int(n_flows), int(n_blocks), int(hidden), b, ctypes.byref(h)))
         self._h = h
         self.n_blocks, self.hidden, self.n_flows = int(n_blocks), int(hidden), int(n_flows)
         self.n_params = int(L.abc_maf_param_count(h))
@@ -905,8 +922,8 @@ def abc_smc_run(observed, N_pop, eps0, rounds=5, sims_per_round=1 << 22, eps_fac
     n = ctypes.c_uint64()
     s = cuda_stream if cuda_stream is not None else torch.cuda.Stream()
     torch.cuda.current_stream().synchronize()
-    b = prior_box(lo, hi)
-    _check(L, L.abc_smc_run(ctypes.byref(b), obs_p, T, int(N_pop), ctypes.byref(cfg), rr, theta.data_ptr(),
+    b = _box(lo, hi)
+    _check(L, L.abc_smc_run(b, obs_p, T, int(N_pop), ctypes.byref(cfg), rr, theta.data_ptr(),
                             w.data_ptr(), dist.data_ptr(), ctypes.byref(n), _stream(s)))
     out = [dict((f, getattr(r, f)) for f, _ in AbcSmcRound._fields_) for r in rr]
     m = int(n.value)
@@ -940,7 +957,7 @@ def abc_smc_run_regions(regions, rounds=16, shrink_rounds=4, sims_per_round=1 <<
         w = torch.empty((max(pool, 1),), dtype=torch.float64, device=dev)
         d = torch.empty((max(pool, 1),), dtype=torch.float64, device=dev)
         outs.append((th, w, d))
-        arr[g] = AbcSmcRegion(ctypes.cast(obs_p, ctypes.c_void_p), obs.shape[1] - 1, int(reg["N_pop"]),
+        arr[g] = AbcSmcRegion(obs_p, obs.shape[1] - 1, int(reg["N_pop"]),
                               float(reg["eps"]), th.data_ptr(), w.data_ptr(), d.data_ptr(), pool, 0, 0)
     base = AbcSmcConfig(int(rounds), int(sims_per_round), 0.0, float(eps_factor), float(ess_min), int(flow_blocks),
                         int(flow_hidden), int(train_steps), int(train_batch), float(train_lr), int(seed),
@@ -950,8 +967,8 @@ def abc_smc_run_regions(regions, rounds=16, shrink_rounds=4, sims_per_round=1 <<
     rr = (AbcSmcRound * (int(rounds) * R))()
     s = cuda_stream if cuda_stream is not None else torch.cuda.Stream()
     torch.cuda.current_stream().synchronize()
-    b = prior_box(lo, hi)
-    _check(L, L.abc_smc_run_regions(ctypes.byref(b), arr, R, ctypes.byref(cfg), rr, _stream(s)))
+    b = _box(lo, hi)
+    _check(L, L.abc_smc_run_regions(b, arr, R, ctypes.byref(cfg), rr, _stream(s)))
     info = [[dict((f, getattr(rr[r * R + g], f)) for f, _ in AbcSmcRound._fields_) for g in range(R)]
             for r in range(int(rounds))]
     res = []
@@ -995,8 +1012,8 @@ def abc_pmc_run(observed, N_pop, eps0, rounds=4, n_particles=4096, batch=1 << 20
     n = ctypes.c_uint64()
     s = cuda_stream if cuda_stream is not None else torch.cuda.Stream()
     torch.cuda.current_stream().synchronize()
-    b = prior_box(lo, hi)
-    _check(L, L.abc_pmc_run(ctypes.byref(b), obs_p, T, int(N_pop), ctypes.byref(cfg), rr, theta.data_ptr(),
+    b = _box(lo, hi)
+    _check(L, L.abc_pmc_run(b, obs_p, T, int(N_pop), ctypes.byref(cfg), rr, theta.data_ptr(),
                             w.data_ptr(), dist.data_ptr(), ctypes.byref(n), _stream(s)))
     out = [dict((f, getattr(r, f)) for f, _ in AbcPmcRound._fields_) for r in rr]
     m = int(n.value)
@@ -1009,8 +1026,8 @@ def abc_pmc_propose(theta_old, w_old, Lmat, n, seed=0, first_index=0, lo=PAPER_L
     L = load()
     Lh = np.ascontiguousarray(np.asarray(Lmat, dtype=np.float32).reshape(8, 8))
     out = torch.empty((n, 8), dtype=torch.float32, device=theta_old.device)
-    b = prior_box(lo, hi)
-    _check(L, L.abc_pmc_propose(ctypes.byref(b), theta_old.data_ptr(), w_old.data_ptr(), theta_old.shape[0],
+    b = _box(lo, hi)
+    _check(L, L.abc_pmc_propose(b, theta_old.data_ptr(), w_old.data_ptr(), theta_old.shape[0],
                                 Lh.ctypes.data, int(seed), int(first_index), int(n), out.data_ptr(),
                                 _stream(cuda_stream)))
     return out

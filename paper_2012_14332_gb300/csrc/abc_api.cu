@@ -865,19 +865,16 @@ abc_status abc_sample_quantile(const abc_prior_box* prior, const int32_t* observ
     if ((st = alloc_select(big, dist_bytes + sizeof(float) * 8 * n_samples, cap, s, &w, &cand)) != ABC_OK) return st;
     double* dist_d = (double*)big.ptr;
     float* theta_d = (float*)((char*)big.ptr + dist_bytes);
-    // the accept counter, then the observed series: uploaded in one copy from
-    // pinned staging; the selection's state comes back behind the counter
+    // the observed series, uploaded from pinned staging; the selection's state
+    // and the accept counter behind it come back to the same place
     struct Tail {
-        unsigned long long count;
         abcgb::SelectState sel;
+        unsigned long long count;
     };
-    const size_t obs_off = 256;
-    static_assert(sizeof(Tail) <= 256, "the staged state overlaps the series");
+    static_assert(offsetof(abcgb::SelectWork, accepted) == offsetof(Tail, count), "copied back together");
     SampleScratch* sc = nullptr;
-    if ((st = sample_scratch(obs_off + sizeof(int4) * obs.size(), &sc)) != ABC_OK) return st;
-    std::memset(sc->host, 0, obs_off);
-    std::memcpy((char*)sc->host + obs_off, obs.data(), sizeof(int4) * obs.size());
-    unsigned long long* count_d = (unsigned long long*)sc->dev;
+    if ((st = sample_scratch(std::max(sizeof(int4) * obs.size(), sizeof(Tail)), &sc)) != ABC_OK) return st;
+    std::memcpy(sc->host, obs.data(), sizeof(int4) * obs.size());
     Tail* tail_h = (Tail*)sc->host;
     if (injected("launch")) return fail(ABC_ERR_CUDA, "kernel launch failed (injected)");
     // from here on the pinned staging buffer may be in use by the stream: every
@@ -886,10 +883,10 @@ abc_status abc_sample_quantile(const abc_prior_box* prior, const int32_t* observ
         cudaStreamSynchronize(s);
         return e;
     };
-    cudaError_t ce = cudaMemcpyAsync(sc->dev, sc->host, obs_off + sizeof(int4) * obs.size(), cudaMemcpyHostToDevice, s);
-    if (ce != cudaSuccess) return drain(cuda_fail(ce, "cudaMemcpyAsync(observed, counters)"));
+    cudaError_t ce = cudaMemcpyAsync(sc->dev, sc->host, sizeof(int4) * obs.size(), cudaMemcpyHostToDevice, s);
+    if (ce != cudaSuccess) return drain(cuda_fail(ce, "cudaMemcpyAsync(observed)"));
     abcgb::DistanceArgs da;
-    da.obs = (const int4*)((char*)sc->dev + obs_off);
+    da.obs = (const int4*)sc->dev;
     da.first_index = first_index;
     da.n_samples = n_samples;
     da.dist_out = dist_d;
@@ -907,22 +904,19 @@ abc_status abc_sample_quantile(const abc_prior_box* prior, const int32_t* observ
     a.dist_out = dist_out;
     a.idx_out = idx_out;
     a.capacity = capacity;
-    a.count = count_d;
+    a.count = &w->accepted;
     // the key by the bracket; by the radix select where that left it open
     for (int pass = cand ? 0 : 1; pass < 2; ++pass) {
         if (pass == 0) {
             ce = cudaMemsetAsync(w, 0, abcgb::kSelectZeroBytes, s);
             if (ce == cudaSuccess) ce = abcgb::launch_kth_bracket(dist_d, n_samples, k, w, cand, cap, s);
         } else {
-            ce = cudaMemsetAsync(count_d, 0, sizeof *count_d, s);
-            if (ce == cudaSuccess) ce = abcgb::launch_kth_radix(dist_d, n_samples, k, w, s);
+            ce = abcgb::launch_kth_radix(dist_d, n_samples, k, w, s);   // zeroes the counter too
         }
         if (ce != cudaSuccess) return drain(cuda_fail(ce, "k-th smallest launch"));
         ce = abcgb::launch_select_below(a, s);
         if (ce != cudaSuccess) return drain(cuda_fail(ce, "select_below launch"));
-        ce = cudaMemcpyAsync(&tail_h->count, count_d, sizeof *count_d, cudaMemcpyDeviceToHost, s);
-        if (ce == cudaSuccess)
-            ce = cudaMemcpyAsync(&tail_h->sel, &w->st, sizeof tail_h->sel, cudaMemcpyDeviceToHost, s);
+        ce = cudaMemcpyAsync(tail_h, w, sizeof *tail_h, cudaMemcpyDeviceToHost, s);
         if (ce != cudaSuccess) return drain(cuda_fail(ce, "cudaMemcpyAsync(select state)"));
         CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
         if (tail_h->sel.resolved) break;

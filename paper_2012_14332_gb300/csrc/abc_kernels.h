@@ -185,6 +185,7 @@ struct SelectState {
 constexpr int kPivotSample = 2048;
 struct SelectWork {
     SelectState st;
+    unsigned long long accepted;        // counter for the accept step that follows
     unsigned long long hist[258];       // radix select: 256 bins, invalid keys, ticket
     uint32_t bins[2048];
     uint64_t few[4096];
