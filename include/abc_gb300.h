@@ -457,7 +457,10 @@ abc_status abc_maf_get_params(abc_maf maf, float* params);
  * (i_lo, i_hi, 0, 4 stream + c / 4), whose uniform (2m + 1) 2^-24 (m its low
  * 23 bits) gives the draw log(u / (1 - u))), the sequential
  * inverse of the flow, theta = lo + (hi - lo) sigmoid(y). theta_out DEVICE
- * float [n][8]; logq_out DEVICE float [n] (log q(theta)) or NULL. Async. */
+ * float [n][8]; logq_out DEVICE float [n] (log q(theta)) or NULL. Async.
+ * Sampling and density run in one of two kernel forms by n (both round the same
+ * values to BF16, with FP32 sums in another order), so one index drawn in calls
+ * of different n agrees to rounding, not always to the bit. */
 abc_status abc_maf_sample(abc_maf maf, uint64_t n, const float* base_draws, uint64_t seed, uint32_t stream,
                           uint64_t first_index, float* theta_out, float* logq_out, void* cuda_stream);
 abc_status abc_maf_sample_at(abc_maf maf, int32_t flow, uint64_t n, const float* base_draws, uint64_t seed,

@@ -1,10 +1,11 @@
 // abc_maf.cu -- masked autoregressive flow proposal for sequential ABC:
 // density, sampling (sequential inverse), weighted maximum-likelihood
-// gradient and Adam, with BF16 tensor-core products (mma.sync m16n8k8 and
-// m16n8k16 per warp tile; tcgen05.mma with TMEM accumulators for the weight
-// gradients; FP32 accumulation).
+// gradient and Adam, with BF16 tensor-core products and FP32 accumulation:
+// density and sampling of many points on tcgen05.mma, a thread per row; of few
+// points, and the gradient's per-row passes, on mma.sync m16n8k8 and m16n8k16
+// per warp tile; the weight gradients on tcgen05.mma.
 //
-// A warp owns 16 rows (samples). A row's eight coordinates sit in the
+// In the mma.sync form a warp owns 16 rows (samples). A row's eight coordinates sit in the
 // accumulator layout of an m16n8 tile: lane (g = lane / 4, t = lane % 4) holds
 // columns 2t, 2t+1 of rows g and g+8. That is also the A-operand layout of an
 // m16n8k8 product, so a MADE block runs entirely in registers:
@@ -32,6 +33,7 @@
 #include "../../include/abc_gb300.h"
 #include "abc_kernels.h"
 #include "abc_model.cuh"
+#include "abc_tc.cuh"
 
 namespace abcgb {
 abc_status plan_fail(abc_status st, const char* msg);
@@ -51,29 +53,45 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 // Master (FP32) parameters of one block: W1 [H][8], b1 [H], W2 [16][H], b2 [16].
 __host__ __device__ inline int master_block(int H) { return 25 * H + 16; }
 
-// Published BF16 layout of one block, in 32-bit words (two bf16 per word).
-// The forward operands come first, so density and sampling kernels stage only
-// fwd_words per block; the gradient kernel stages all words. The forward
-// operands are grouped by 16-unit hidden chunk s and lane (g = lane / 4,
-// t = lane % 4) so that one chunk's fragments are one vector load per lane:
+// Published BF16 layout of one block, in 32-bit words (two bf16 per word): the
+// density's operands, the sampler's and the gradient's, each kernel staging its
+// own contiguous words.
+//
+// Density and sampler (tcgen05, B operands, K-major): core matrices of 8 rows
+// (hidden units, or outputs) x 16 bytes (8 bf16 along k), 128 bytes apart
+// along k and 256 along the rows.
+//   d1  [H/8][2][8][4]   layer 1: row = hidden unit, k = 0..7 its input weights,
+//                        k = 8..10 three bf16 that add up to its b1 (they meet
+//                        ones), k = 11..15 zero
+//   d2  [H/16][2][2][8][4] layer 2, a k-step of 16 hidden units after another:
+//                        row 2j = mu_j, row 2j + 1 = alpha_raw_j
+//   db2 [16]             FP32 b2 in the same row order
+// then s1, s2, sb2: the same for the sampler, over hidden units grouped by
+// degree: every degree d = 1..7 has the same number of 16-unit steps,
+// sampler_cpd(H) (the steps degree 1, which has the most units, needs), holding
+// units d - 1, d + 6, d + 13, ... in order, padded with zero units.
+//
+// Gradient (mma.sync fragments, grouped by 16-unit hidden chunk s and lane
+// g = lane / 4, t = lane % 4, so that one chunk's fragments are one vector load
+// per lane):
 //   w1  [H/16][8][4][2]  B operands of x W1^T (k = input j = 2t, 2t+1) for
 //                        hidden units 16s + g and 16s + 8 + g
 //   w2  [H/16][8][4][4]  B operands of h W2^T (k = hidden 16s + 2t, +1 and
 //                        16s + 8 + 2t, +1) for outputs g and 8 + g
 //   b1  [H/16][4][4]     FP32: b1 of hidden 16s + 2t, +1, 16s + 8 + 2t, +1
-//   b2  [16]             FP32
+//   b2  [16]             FP32 (w1 to b2 also serve the density of few points)
 //   w1t [8][H/2+4]       B operand of g_a1 W1     (n = j, k = l)
 //   w2t [H][8]           B operand of g_out W2    (n = l, k = o); rows l with
 //                        l & 4 hold their two 4-word halves swapped, so the
 //                        warp's fragment loads meet 32 distinct banks
-// then the sampler's copy of the forward operands (sw1, sw2, sb1 in the w1,
-// w2, b1 layouts, and sb2 = b2), whose 16-unit chunks hold the hidden units
-// grouped by degree: every degree d = 1..7 has the same number of chunks,
-// sampler_cpd(H) (the chunks degree 1, which has the most units, needs),
-// holding units d - 1, d + 6, d + 13, ... in order, padded with zero units.
+//
+// then the fragments of the sampler of few points (m1, m2, mb1, mb2 in the w1,
+// w2, b1, b2 layouts), over the same degree-grouped units as s1 and s2.
 struct Layout {
-    int w1, w2, b1, b2, w1t, w2t, fwd_words, grad_words;
-    int sw1, sw2, sb1, sb2, samp_words, words;
+    int d1, d2, db2, dens_words;
+    int s1, s2, sb2, samp_words;
+    int w1, w2, b1, b2, fwd_words, w1t, w2t, grad_words;
+    int m1, m2, mb1, mb2, msamp_words, words;
 };
 
 // MADE masks (Germain et al.): hidden degree (l mod 7) + 1; input j and output
@@ -97,23 +115,39 @@ __host__ __device__ inline int sampler_unit(int H, int s, int u)
 __host__ __device__ inline Layout layout(int H)
 {
     Layout L;
+    const int C = sampler_chunks(H);
     int o = 0;
+    L.d1 = o; o += H * 8;
+    L.d2 = o; o += H * 8;
+    L.db2 = o; o += 16;
+    L.dens_words = o - L.d1;
+    L.s1 = o; o += C * 128;
+    L.s2 = o; o += C * 128;
+    L.sb2 = o; o += 16;
+    L.samp_words = o - L.s1;
     L.w1 = o; o += H * 4;
     L.w2 = o; o += H * 8;
     L.b1 = o; o += H;
     L.b2 = o; o += 16;
-    L.fwd_words = o;
+    L.fwd_words = o - L.w1;
     L.w1t = o; o += 8 * (H / 2 + 4);
     L.w2t = o; o += H * 8;
-    L.grad_words = o;
-    const int C = sampler_chunks(H);
-    L.sw1 = o; o += C * 64;
-    L.sw2 = o; o += C * 128;
-    L.sb1 = o; o += C * 16;
-    L.sb2 = o; o += 16;
-    L.samp_words = o - L.sw1;
+    L.grad_words = o - L.w1;
+    L.m1 = o; o += C * 64;
+    L.m2 = o; o += C * 128;
+    L.mb1 = o; o += C * 16;
+    L.mb2 = o; o += 16;
+    L.msamp_words = o - L.m1;
     L.words = o;
     return L;
+}
+
+// Part k (0..2) of b as bf16: each part is the rounding of what the ones before
+// left, so the three add up to b to its last bit (24 bits of significand).
+__device__ __forceinline__ float bias_part(float b, int k)
+{
+    for (int i = 0; i < k; ++i) b -= __bfloat162float(__float2bfloat16_rn(b));
+    return b;
 }
 
 struct Box {
@@ -179,8 +213,10 @@ struct BlockView {
     const float* b2;
 };
 
-__device__ __forceinline__ BlockView view(const uint32_t* base, const Layout& L)
+// the gradient's operands of one block, staged from layout word w1 on
+__device__ __forceinline__ BlockView view(const uint32_t* staged, const Layout& L)
 {
+    const uint32_t* base = staged - L.w1;
     BlockView v;
     v.w1 = base + L.w1;
     v.w2 = base + L.w2;
@@ -206,24 +242,19 @@ __device__ __forceinline__ void reverse_cols(float (&v)[4])
     v[0] = n0; v[1] = n1; v[2] = n2; v[3] = n3;
 }
 
+// exp and the reciprocal of 1 + e as single SFU operations, results below 2^-126
+// flushed to 0 (__expf and __fdividef keep them, at about ten instructions
+// more for an alpha and its exponential).
+__device__ __forceinline__ float exp_sfu(float x) { return fast::ex2(1.44269504f * x); }
+
 // alpha = A tanh(ar / A) from one exponential: tanh|y| = (1 - e) / (1 + e) with
-// e = exp(-2 |y|) in (0, 1], so nothing overflows; the fast exponential and
-// division leave an absolute error of a few 1e-7 in alpha
+// e = exp(-2 |y|) in (0, 1], so nothing overflows; the SFU operations leave an
+// absolute error of a few 1e-7 in alpha
 __device__ __forceinline__ float soft_alpha(float ar)
 {
-    const float e = __expf((-2.f / kAlphaMax) * fabsf(ar));
-    return copysignf(kAlphaMax * __fdividef(1.f - e, 1.f + e), ar);
+    const float e = fast::ex2((-2.f * 1.44269504f / kAlphaMax) * fabsf(ar));
+    return copysignf(kAlphaMax * ((1.f - e) * fast::rcp(1.f + e)), ar);
 }
-
-// Density and sampling CTAs: 8 warps share one staged copy of the forward
-// operands (about 41 KB at 3 x 256), at most 64 registers so that 4 CTAs
-// (32 warps) fit on an SM to hide the tensor-core chains' latency.
-constexpr int kFwdThreads = 256;
-constexpr int kFwdMinBlocks = 4;
-// The sampler's longer passes run better at 3 CTAs per SM (80 registers,
-// 16 bytes spilled, against 64 and 32): 1.182 -> 1.157 ms per 0.9 x 2^22
-// proposals at 3 x 256.
-constexpr int kSampMinBlocks = 3;
 
 // The base density: independent standard logistic coordinates,
 // log p(z) = -|z| - 2 log(1 + exp(-|z|)); d(-log p)/dz = tanh(z / 2). The logit
@@ -336,6 +367,130 @@ __device__ __forceinline__ void to_theta(const Box& b, int j, float y, float& th
     jac = b.logw[j] + ls + l1s;
 }
 
+// ---------------------------------------------------------------------------
+// publish: masked BF16 copies (and biases) from the FP32 master parameters
+// ---------------------------------------------------------------------------
+// Every word of each block's published operands, padding included (a
+// training step's Adam launch republishes the gradient's operands of the
+// parameters it updates, one parameter per thread, and never writes the padding).
+__global__ void publish_kernel(const float* __restrict__ master, uint32_t* __restrict__ pub, int K, int H)
+{
+    const Layout L = layout(H);
+    const int per = L.words, mb = master_block(H), hw = H / 2 + 4;
+    master += (size_t)blockIdx.y * K * mb;   // flow blockIdx.y
+    pub += (size_t)blockIdx.y * K * per;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < K * per; i += gridDim.x * blockDim.x) {
+        const int b = i / per, w = i % per;
+        const float* M = master + (size_t)b * mb;
+        const float* W1 = M;
+        const float* b1 = M + 8 * H;
+        const float* W2 = M + 9 * H;
+        const float* b2 = M + 25 * H;
+        // masked weights; unit -1 is padding
+        const auto w1_of = [&](int l, int j) { return l >= 0 && mask1(l, j) ? W1[l * 8 + j] : 0.f; };
+        const auto w2_of = [&](int o, int l) { return l >= 0 && mask2(o, l) ? W2[o * H + l] : 0.f; };
+        // word r of a d1 section: ((unit / 8 * 2 + k / 8) 8 + unit % 8) 4 + k % 8 / 2
+        const auto layer1 = [&](int r, int l) {
+            const int k = 8 * (r >> 5 & 1) + 2 * (r & 3);
+            if (k < 8) return pack2(w1_of(l, k), w1_of(l, k + 1));
+            if (l < 0 || k > 10) return 0u;
+            return k == 8 ? pack2(bias_part(b1[l], 0), bias_part(b1[l], 1)) : pack2(bias_part(b1[l], 2), 0.f);
+        };
+        const auto layer1_unit = [](int r) { return 8 * (r >> 6) + (r >> 2 & 7); };
+        // word r of a d2 section: (((step 2 + row / 8) 2 + k / 8) 8 + row % 8) 4 + k % 8 / 2;
+        // row 2j is mu_j (output j), row 2j + 1 alpha_raw_j (output 8 + j)
+        const auto layer2_row = [](int r) { return 8 * (r >> 6 & 1) + (r >> 2 & 7); };
+        const auto layer2_unit = [](int r) { return 16 * (r >> 7) + 8 * (r >> 5 & 1) + 2 * (r & 3); };
+        const auto output_of = [](int row) { return (row >> 1) + 8 * (row & 1); };
+        uint32_t out = 0;
+        if (w < L.d2) {
+            out = layer1(w - L.d1, layer1_unit(w - L.d1));
+        } else if (w < L.db2) {
+            const int r = w - L.d2, o = output_of(layer2_row(r)), l = layer2_unit(r);
+            out = pack2(w2_of(o, l), w2_of(o, l + 1));
+        } else if (w < L.s1) {
+            out = __float_as_uint(b2[output_of(w - L.db2)]);
+        } else if (w < L.s2) {
+            const int r = w - L.s1, u = layer1_unit(r);
+            out = layer1(r, sampler_unit(H, u >> 4, u & 15));
+        } else if (w < L.sb2) {
+            const int r = w - L.s2, o = output_of(layer2_row(r)), u = layer2_unit(r);
+            out = pack2(w2_of(o, sampler_unit(H, u >> 4, u & 15)), w2_of(o, sampler_unit(H, u >> 4, (u & 15) + 1)));
+        } else if (w < L.w1) {
+            out = __float_as_uint(b2[output_of(w - L.sb2)]);
+        } else if (w < L.w2) {
+            // r = ((s 8 + g) 4 + t) 2 + h: hidden l = 16 s + g + 8 h, inputs 2t, 2t+1
+            const int r = w - L.w1, h = r & 1, t = (r >> 1) & 3, g = (r >> 3) & 7, sc = r >> 6;
+            const int l = 16 * sc + g + 8 * h;
+            out = pack2(w1_of(l, 2 * t), w1_of(l, 2 * t + 1));
+        } else if (w < L.b1) {
+            // r = ((s 8 + g) 4 + t) 4 + q: output g + 8 (q / 2), hidden 16 s + 8 (q % 2) + 2t, +1
+            const int r = w - L.w2, q = r & 3, t = (r >> 2) & 3, g = (r >> 4) & 7, sc = r >> 7;
+            const int o = g + 8 * (q >> 1), l0 = 16 * sc + 8 * (q & 1) + 2 * t;
+            out = pack2(w2_of(o, l0), w2_of(o, l0 + 1));
+        } else if (w < L.b2) {
+            // r = (s 4 + t) 4 + q: b1 of hidden 16 s + 8 (q / 2) + 2t + q % 2
+            const int r = w - L.b1, q = r & 3, t = (r >> 2) & 3, sc = r >> 4;
+            out = __float_as_uint(b1[16 * sc + 8 * (q >> 1) + 2 * t + (q & 1)]);
+        } else if (w < L.w1t) {
+            out = __float_as_uint(b2[w - L.b2]);
+        } else if (w < L.w2t) {
+            const int r = w - L.w1t, j = r / hw, c = r % hw;
+            if (c < H / 2) out = pack2(w1_of(2 * c, j), w1_of(2 * c + 1, j));
+        } else if (w < L.m1) {
+            const int r = w - L.w2t, l = r / 8, o0 = 2 * ((r % 8) ^ (l & 4));
+            out = pack2(w2_of(o0, l), w2_of(o0 + 1, l));
+        } else if (w < L.m2) {
+            // as w1, over the degree-grouped units
+            const int r = w - L.m1, h = r & 1, t = (r >> 1) & 3, g = (r >> 3) & 7, sc = r >> 6;
+            const int l = sampler_unit(H, sc, g + 8 * h);
+            out = pack2(w1_of(l, 2 * t), w1_of(l, 2 * t + 1));
+        } else if (w < L.mb1) {
+            const int r = w - L.m2, q = r & 3, t = (r >> 2) & 3, g = (r >> 4) & 7, sc = r >> 7;
+            const int o = g + 8 * (q >> 1), u = 8 * (q & 1) + 2 * t;
+            out = pack2(w2_of(o, sampler_unit(H, sc, u)), w2_of(o, sampler_unit(H, sc, u + 1)));
+        } else if (w < L.mb2) {
+            const int r = w - L.mb1, q = r & 3, t = (r >> 2) & 3, sc = r >> 4;
+            const int l = sampler_unit(H, sc, 8 * (q >> 1) + 2 * t + (q & 1));
+            out = __float_as_uint(l >= 0 ? b1[l] : 0.f);
+        } else {
+            out = __float_as_uint(b2[w - L.mb2]);
+        }
+        pub[(size_t)b * per + w] = out;
+    }
+}
+
+// The K blocks' words [off, off + n) of the published operands, copied into
+// sm (K x n words, packed) by the bulk-copy engine: thread 0 sets the
+// barrier's transaction count and issues one copy per block. The barrier was
+// initialised (count 1) and that made visible to the CTA before the call.
+// Offsets and sizes are multiples of 4 words (16 bytes), as the bulk copy
+// requires: every section of the layout is, since H is a multiple of 16.
+__device__ __forceinline__ void stage_blocks_bulk(uint32_t* sm, const uint32_t* pub, int K, int off, int n,
+                                                  const Layout& L, uint32_t bar)
+{
+    if (threadIdx.x != 0) return;
+    mbar_arrive_expect_tx(bar, (uint32_t)(K * n) * 4u);
+    for (int b = 0; b < K; ++b) bulk_g2s(smem_addr(sm + b * n), pub + (size_t)b * L.words + off, (uint32_t)n * 4u, bar);
+}
+
+// ---------------------------------------------------------------------------
+// Density and sampling of few points: mma.sync, a warp per 16 rows. With few
+// rows an SM the time is the length of the chain, and a pass of the sampler
+// takes a warp about half as long as a group of 128 rows in the form below (two
+// commits a pass): 12.7 us for 3000 proposals at 4 x 176, 24.7 there; with expf
+// and divisions for its sigmoids and softplus this form took 18.9.
+// ---------------------------------------------------------------------------
+// Density and sampling CTAs: 8 warps share one staged copy of the forward
+// operands (about 41 KB at 3 x 256), at most 64 registers so that 4 CTAs
+// (32 warps) fit on an SM to hide the tensor-core chains' latency.
+constexpr int kFwdThreads = 256;
+constexpr int kFwdMinBlocks = 4;
+// The sampler's longer passes run better at 3 CTAs per SM (80 registers,
+// 16 bytes spilled, against 64 and 32): 1.182 -> 1.157 ms per 0.9 x 2^22
+// proposals at 3 x 256.
+constexpr int kSampMinBlocks = 3;
+
 // words [off, off + n) of each of K published blocks, packed block after
 // block in shared memory (stride n). Every offset and length is a multiple of
 // 4 words (H is a multiple of 16), so the copy moves 16-byte vectors.
@@ -349,97 +504,15 @@ __device__ __forceinline__ void stage_blocks(uint32_t* sm, const uint32_t* pub, 
     }
 }
 
-// ---------------------------------------------------------------------------
-// publish: masked BF16 copies (and biases) from the FP32 master parameters
-// ---------------------------------------------------------------------------
-// Every word of each block's published operands, padding included (a
-// training step's Adam launch republishes the parameters it updates, one
-// parameter per thread, and never writes the padding).
-__global__ void publish_kernel(const float* __restrict__ master, uint32_t* __restrict__ pub, int K, int H)
-{
-    const Layout L = layout(H);
-    const int per = L.words, limit = L.words, mb = master_block(H), hw = H / 2 + 4;
-    master += (size_t)blockIdx.y * K * mb;   // flow blockIdx.y
-    pub += (size_t)blockIdx.y * K * per;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < K * limit; i += gridDim.x * blockDim.x) {
-        const int b = i / limit, w = i % limit, idx = b * per + w;
-        const float* M = master + (size_t)b * mb;
-        const float* W1 = M;
-        const float* b1 = M + 8 * H;
-        const float* W2 = M + 9 * H;
-        const float* b2 = M + 25 * H;
-        uint32_t out = 0;
-        if (w < L.w2) {
-            // r = ((s 8 + g) 4 + t) 2 + h: hidden l = 16 s + g + 8 h, inputs 2t, 2t+1
-            const int r = w - L.w1, h = r & 1, t = (r >> 1) & 3, g = (r >> 3) & 7, sc = r >> 6;
-            const int l = 16 * sc + g + 8 * h, j0 = 2 * t;
-            __nv_bfloat162 v = __floats2bfloat162_rn(mask1(l, j0) ? W1[l * 8 + j0] : 0.f,
-                                                     mask1(l, j0 + 1) ? W1[l * 8 + j0 + 1] : 0.f);
-            out = *reinterpret_cast<uint32_t*>(&v);
-        } else if (w < L.b1) {
-            // r = ((s 8 + g) 4 + t) 4 + q: output g + 8 (q / 2), hidden 16 s + 8 (q % 2) + 2t, +1
-            const int r = w - L.w2, q = r & 3, t = (r >> 2) & 3, g = (r >> 4) & 7, sc = r >> 7;
-            const int o = g + 8 * (q >> 1), l0 = 16 * sc + 8 * (q & 1) + 2 * t;
-            __nv_bfloat162 v = __floats2bfloat162_rn(mask2(o, l0) ? W2[o * H + l0] : 0.f,
-                                                     mask2(o, l0 + 1) ? W2[o * H + l0 + 1] : 0.f);
-            out = *reinterpret_cast<uint32_t*>(&v);
-        } else if (w < L.b2) {
-            // r = (s 4 + t) 4 + q: b1 of hidden 16 s + 8 (q / 2) + 2t + q % 2
-            const int r = w - L.b1, q = r & 3, t = (r >> 2) & 3, sc = r >> 4;
-            out = __float_as_uint(b1[16 * sc + 8 * (q >> 1) + 2 * t + (q & 1)]);
-        } else if (w < L.w1t) {
-            out = __float_as_uint(b2[w - L.b2]);
-        } else if (w < L.w2t) {
-            const int r = w - L.w1t, j = r / hw, c = r % hw;
-            if (c < H / 2) {
-                const int l0 = 2 * c;
-                __nv_bfloat162 v = __floats2bfloat162_rn(mask1(l0, j) ? W1[l0 * 8 + j] : 0.f,
-                                                         mask1(l0 + 1, j) ? W1[(l0 + 1) * 8 + j] : 0.f);
-                out = *reinterpret_cast<uint32_t*>(&v);
-            }
-        } else if (w < L.grad_words) {
-            const int r = w - L.w2t, l = r / 8, o0 = 2 * ((r % 8) ^ (l & 4));
-            __nv_bfloat162 v = __floats2bfloat162_rn(mask2(o0, l) ? W2[o0 * H + l] : 0.f,
-                                                     mask2(o0 + 1, l) ? W2[(o0 + 1) * H + l] : 0.f);
-            out = *reinterpret_cast<uint32_t*>(&v);
-        } else if (w < L.sw2) {
-            // as w1, over the degree-grouped chunks: unit at position g + 8 h of chunk s
-            const int r = w - L.sw1, h = r & 1, t = (r >> 1) & 3, g = (r >> 3) & 7, sc = r >> 6;
-            const int l = sampler_unit(H, sc, g + 8 * h), j0 = 2 * t;
-            __nv_bfloat162 v = __floats2bfloat162_rn(l >= 0 && mask1(l, j0) ? W1[l * 8 + j0] : 0.f,
-                                                     l >= 0 && mask1(l, j0 + 1) ? W1[l * 8 + j0 + 1] : 0.f);
-            out = *reinterpret_cast<uint32_t*>(&v);
-        } else if (w < L.sb1) {
-            const int r = w - L.sw2, q = r & 3, t = (r >> 2) & 3, g = (r >> 4) & 7, sc = r >> 7;
-            const int o = g + 8 * (q >> 1), u0 = 8 * (q & 1) + 2 * t;
-            const int l0 = sampler_unit(H, sc, u0), l1 = sampler_unit(H, sc, u0 + 1);
-            __nv_bfloat162 v = __floats2bfloat162_rn(l0 >= 0 && mask2(o, l0) ? W2[o * H + l0] : 0.f,
-                                                     l1 >= 0 && mask2(o, l1) ? W2[o * H + l1] : 0.f);
-            out = *reinterpret_cast<uint32_t*>(&v);
-        } else if (w < L.sb2) {
-            const int r = w - L.sb1, q = r & 3, t = (r >> 2) & 3, sc = r >> 4;
-            const int l = sampler_unit(H, sc, 8 * (q >> 1) + 2 * t + (q & 1));
-            out = __float_as_uint(l >= 0 ? b1[l] : 0.f);
-        } else {
-            out = __float_as_uint(b2[w - L.sb2]);
-        }
-        pub[idx] = out;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// density: log q(theta)
-// ---------------------------------------------------------------------------
-// The proposal may use a broadened base, z = tau * (standard logistic), with
-// density log p(z / tau) - log tau per coordinate (tau = 1: the trained flow).
 template <int K>
-__global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) logq_kernel(const uint32_t* __restrict__ pub, int H, Box box,
+__global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) logq_few_kernel(const uint32_t* __restrict__ pub, int H,
+                                                   const __grid_constant__ Box box,
                                                    const float* __restrict__ theta, uint64_t n, float inv_tau,
                                                    float log_tau, float* __restrict__ logq)
 {
     extern __shared__ __align__(16) uint32_t sm[];
     const Layout L = layout(H);
-    stage_blocks(sm, pub, K, 0, L.fwd_words, L);
+    stage_blocks(sm, pub, K, L.w1, L.fwd_words, L);
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const uint64_t tiles = (n + 15) / 16;
@@ -463,7 +536,7 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) logq_kernel(const 
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float al = soft_alpha(ar[e]);
-                x[e] = (x[e] - mu[e]) * __expf(-al);
+                x[e] = (x[e] - mu[e]) * exp_sfu(-al);
                 ld[e] -= al;
             }
             reverse_cols(x);
@@ -510,8 +583,8 @@ __device__ __forceinline__ void inverse_column(int t, const float (&z)[4], float
     constexpr int e = D & 1;
     if (t == D / 2) {
         const float al0 = soft_alpha(o1[e] + p1[e]), al1 = soft_alpha(o1[2 + e] + p1[2 + e]);
-        xin[e] = z[e] * __expf(al0) + (o0[e] + p0[e]);
-        xin[2 + e] = z[2 + e] * __expf(al1) + (o0[2 + e] + p0[2 + e]);
+        xin[e] = z[e] * exp_sfu(al0) + (o0[e] + p0[e]);
+        xin[2 + e] = z[2 + e] * exp_sfu(al1) + (o0[2 + e] + p0[2 + e]);
         lq[e] -= al0;
         lq[2 + e] -= al1;
     }
@@ -532,7 +605,7 @@ __device__ __forceinline__ void inverse_passes(const BlockView& v, int g, int t,
 template <int K, int CPD>
 // box: read in place from the parameter space (indexing a by-value copy by
 // the lane's column put it in local memory)
-__global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_kernel(const uint32_t* __restrict__ pub, int H,
+__global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_few_kernel(const uint32_t* __restrict__ pub, int H,
                                                      const __grid_constant__ Box box,
                                                      const float* __restrict__ u_in, const __grid_constant__ ModelParams p,
                                                      uint32_t ctr3, uint64_t first, uint64_t n, float tau,
@@ -541,7 +614,7 @@ __global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_kernel(con
 {
     extern __shared__ __align__(16) uint32_t sm[];
     const Layout L = layout(H);
-    stage_blocks(sm, pub, K, L.sw1, L.samp_words, L);
+    stage_blocks(sm, pub, K, L.m1, L.msamp_words, L);
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const uint64_t tiles = (n + 15) / 16;
@@ -577,12 +650,12 @@ __global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_kernel(con
         // 1..j have added to the accumulators by then.
 #pragma unroll 1
         for (int bb = K - 1; bb >= 0; --bb) {
-            const uint32_t* base = sm + bb * L.samp_words;
+            const uint32_t* base = sm + bb * L.msamp_words;
             BlockView v;
             v.w1 = base;
-            v.w2 = base + (L.sw2 - L.sw1);
-            v.b1 = reinterpret_cast<const float*>(base + (L.sb1 - L.sw1));
-            v.b2 = reinterpret_cast<const float*>(base + (L.sb2 - L.sw1));
+            v.w2 = base + (L.m2 - L.m1);
+            v.b1 = reinterpret_cast<const float*>(base + (L.mb1 - L.m1));
+            v.b2 = reinterpret_cast<const float*>(base + (L.mb2 - L.m1));
             v.w1t = v.w2t = nullptr;
             float z[4] = {x[0], x[1], x[2], x[3]};
             reverse_cols(z);
@@ -594,8 +667,8 @@ __global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_kernel(con
             if (t == 0) {
                 // column 0 has degree 1: every weight into mu_0, alpha_0 is masked
                 const float al0 = soft_alpha(bs.x);
-                xin[0] = z[0] * __expf(al0) + bm.x;
-                xin[2] = z[2] * __expf(al0) + bm.x;
+                xin[0] = z[0] * exp_sfu(al0) + bm.x;
+                xin[2] = z[2] * exp_sfu(al0) + bm.x;
                 lq[0] -= al0;
                 lq[2] -= al0;
             }
@@ -616,6 +689,378 @@ __global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_kernel(con
             if (r1 < n) logq_out[r1] = q1;
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// Density and sampling on tcgen05: a thread per row.
+//
+// A group of 128 threads owns 128 rows, one a thread, and a tensor-memory
+// quarter or eighth of an SM. Layer 1 is one product of M = 128 rows x N
+// hidden units x K = 16 (8 inputs, 3 ones against b1's three bf16 parts, the
+// rest zero), the rows' inputs from shared memory; each thread reads its row's
+// pre-activations from tensor memory, applies the ReLU as it rounds them to
+// bf16, and writes them back as the A operand of layer 2 (N = 16 outputs,
+// K = 16 a step), which accumulates in tensor memory too. Everything between
+// the products (the box map, alpha, its exponential, the log-determinant) is
+// plain arithmetic on the thread's own row, no lane idle, no shuffle.
+//
+// In the mma.sync form above the products alone keep the legacy tensor path
+// busy for 405 of the sampler's 829 us per 0.9 x 2^22 proposals at 3 x 256 (8
+// cycles each, m16n8k8 as much as m16n8k16), a pass's elementwise work runs on
+// 8 of 32 lanes, and its fragments go through shared memory once per 16 rows.
+// This form: sampler 829 -> 535 us there, 188 -> 125 us for 10^6 at 3 x 128;
+// density 540 -> 484 us and (419,431 points) 69 -> 60 us. It is bound by issue
+// (60 % of the cycles issue) in the conversions and the tensor-memory reads of
+// the hidden units; a chain of 14 commits a block hides behind the other groups.
+//
+// One thread of a group issues its products and commits them to the group's
+// mbarrier; the group's own named barrier orders its threads' shared and tensor
+// memory writes before the issue. Every wait is bounded: one that runs out sets
+// the flow's error word, later waits are skipped, and the kernel ends as usual.
+// ---------------------------------------------------------------------------
+constexpr int kRowGroup = 128;
+
+// instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
+// K-major, N >> 3 (bits 17-22), M >> 4 (bits 24-28)
+__host__ __device__ constexpr uint32_t row_idesc(int n)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kRowGroup >> 4) << 24);
+}
+
+// A group's products: its barrier, its tensor memory (column base), its rows'
+// layer-1 operand in shared memory ([16 row groups][2][8 rows][16 bytes]).
+struct RowGroup {
+    uint32_t bar, tmem, lane_tmem, a1;   // lane_tmem: tmem at this warp's lane quarter
+    int id, row;
+    uint32_t phase;
+    bool ok;
+    int* err;
+
+    __device__ __forceinline__ uint32_t a1_row() const { return a1 + (row >> 3) * 256 + (row & 7) * 16; }
+    // shared and tensor memory writes of every thread before the next issue
+    __device__ __forceinline__ void before_issue()
+    {
+        tc_fence_before();
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + id), "n"(kRowGroup) : "memory");
+    }
+    __device__ __forceinline__ bool issues() const { return row == 0; }
+    // the committed products are complete
+    __device__ __forceinline__ void after_commit()
+    {
+        if (ok && !mbar_wait(bar, phase)) {
+            ok = false;
+            atomicExch(err, 1);
+        }
+        phase ^= 1u;
+        __syncwarp();
+        tc_fence_after();
+    }
+};
+
+// COLS (16, 32, 48 or 64) pre-activations of this thread's row from column
+// `from`, through the ReLU, as COLS / 2 columns of bf16 pairs at column `to`.
+// COLS > 16 may write over what it has read.
+template <int COLS>
+__device__ __forceinline__ void relu_to_operand(uint32_t from, uint32_t to)
+{
+#pragma unroll
+    for (int c = 0; c + 32 <= COLS; c += 32) {
+        uint32_t v[32], h[16];
+        tc_ld32(from + c, v);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) h[e] = pack2_relu(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+        tc_st8(to + c / 2, h);
+        tc_st8(to + c / 2 + 8, h + 8);
+    }
+    if constexpr (COLS % 32 != 0) {
+        constexpr int c = COLS - 16;
+        uint32_t v[16], h[8];
+        tc_ld16(from + c, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) h[e] = pack2_relu(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+        tc_st8(to + c / 2, h);
+    }
+    tc_wait_st();
+}
+
+// Set-up shared by the two kernels: tensor memory, barriers, the published
+// operands by bulk copy, the constant half of the rows' layer-1 operand.
+template <int GROUPS, int COLUMNS>
+__device__ __forceinline__ RowGroup row_setup(uint32_t* sm, const uint32_t* pub, int K, int from, int words, const Layout& L,
+                                              int* err, uint64_t (&bar)[GROUPS], uint64_t& bar_stage, uint32_t& tmem_s)
+{
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        for (int g = 0; g < GROUPS; ++g) mbar_init(smem_addr(&bar[g]), 1);
+        mbar_init(smem_addr(&bar_stage), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_s)),
+                     "r"(GROUPS * COLUMNS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    RowGroup g;
+    g.id = threadIdx.x / kRowGroup;
+    g.row = threadIdx.x % kRowGroup;
+    g.a1 = smem_addr(sm + K * words) + g.id * (kRowGroup * 32);
+    // inputs 8..15 of every row: three ones for b1, then zeros
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %3};" ::"r"(g.a1_row() + 128), "r"(0x3F803F80u), "r"(0x3F80u), "r"(0u)
+                 : "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    stage_blocks_bulk(sm, pub, K, from, words, L, smem_addr(&bar_stage));
+    g.bar = smem_addr(&bar[g.id]);
+    g.tmem = tmem_s + g.id * COLUMNS;
+    g.lane_tmem = g.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    g.phase = 0;
+    g.err = err;
+    g.ok = mbar_wait(smem_addr(&bar_stage), 0);
+    if (!g.ok) atomicExch(err, 1);
+    __syncwarp();
+    return g;
+}
+
+template <int GROUPS, int COLUMNS>
+__device__ __forceinline__ void row_teardown(uint32_t tmem_s)
+{
+    tc_fence_before();
+    __syncthreads();   // every group has waited for its last products
+    tc_fence_after();
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_s), "r"(GROUPS * COLUMNS) : "memory");
+}
+
+// log q of one row: the base's and the box map's 16 terms, whose sum is an order
+// larger than any of them, with the rounding errors carried along (Knuth's
+// two-sum). Plain sums in one thread would round at the total's size each time;
+// the mma.sync form spreads a row's over 4 lanes.
+struct LogSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float t = __fadd_rn(hi, v), w = __fsub_rn(t, hi);
+        lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, w)), __fsub_rn(v, w));
+        hi = t;
+    }
+    __device__ __forceinline__ float plus(float v) const { return hi + (lo + v); }
+};
+
+// Density: two groups a CTA, two CTAs an SM. Hidden units go through in chunks
+// of 64 (tensor-memory columns 0..63; their bf16 64..95; outputs 96..111): a
+// chunk's layer 2 and the next chunk's layer 1 are one commit. (Four groups of
+// 64 columns and chunks of 32: 1 % faster for 3.8e6 points, 10 % slower for
+// 419,431.)
+// The proposal may use a broadened base, z = tau * (standard logistic), with
+// density log p(z / tau) - log tau per coordinate (tau = 1: the trained flow).
+constexpr int kDensGroups = 2, kDensColumns = 128, kDensChunk = 64;
+
+template <int K>
+__global__ void __launch_bounds__(kDensGroups * kRowGroup, 2) logq_kernel(const uint32_t* __restrict__ pub, int H,
+                                                                          const __grid_constant__ Box box,
+                                                                          const float* __restrict__ theta, uint64_t n,
+                                                                          float inv_tau, float log_tau,
+                                                                          float* __restrict__ logq, int* __restrict__ err)
+{
+    extern __shared__ __align__(128) uint32_t row_sm[];
+    __shared__ __align__(8) uint64_t bar[kDensGroups], bar_stage;
+    __shared__ uint32_t tmem_s;
+    const Layout L = layout(H);
+    RowGroup g = row_setup<kDensGroups, kDensColumns>(row_sm, pub, K, L.d1, L.dens_words, L, err, bar, bar_stage, tmem_s);
+    const int chunks = (H + kDensChunk - 1) / kDensChunk;
+    const uint64_t tiles = (n + kRowGroup - 1) / kRowGroup;
+    for (uint64_t tile = (uint64_t)blockIdx.x * kDensGroups + g.id; tile < tiles; tile += (uint64_t)gridDim.x * kDensGroups) {
+        const uint64_t r = tile * kRowGroup + g.row;
+        LogSum lq;
+        float x[8], sum_al = 0.f;
+        const float2* src = reinterpret_cast<const float2*>(theta + 8 * (r < n ? r : n - 1));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 v = src[j];
+            float jac;
+            to_y(box, 2 * j, v.x, x[2 * j], jac);
+            lq.add(-jac);
+            to_y(box, 2 * j + 1, v.y, x[2 * j + 1], jac);
+            lq.add(-jac);
+        }
+#pragma unroll 1
+        for (int b = 0; b < K; ++b) {
+            const uint32_t* base = row_sm + b * L.dens_words;
+            const uint32_t w1 = smem_addr(base), w2 = smem_addr(base + L.d2 - L.d1);
+            const float2* b2 = reinterpret_cast<const float2*>(base + L.db2 - L.d1);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(g.a1_row()), "r"(pack2(x[0], x[1])),
+                         "r"(pack2(x[2], x[3])), "r"(pack2(x[4], x[5])), "r"(pack2(x[6], x[7]))
+                         : "memory");
+            fence_async_smem();
+            g.before_issue();
+            const auto layer1 = [&](int c) {   // 32 bytes of w1 a unit
+                const uint32_t units = min(kDensChunk, H - kDensChunk * c);
+                tc_mma(g.tmem, tc_desc(g.a1), tc_desc(w1 + 32 * kDensChunk * c), row_idesc(0) | (units >> 3) << 17, 0);
+            };
+            if (g.issues()) {
+                tc_fence_after();
+                layer1(0);
+                tc_commit(g.bar);
+            }
+            for (int c = 0; c < chunks; ++c) {
+                g.after_commit();
+                const int steps = min(kDensChunk, H - kDensChunk * c) / 16;
+                if (steps == 4)
+                    relu_to_operand<64>(g.lane_tmem, g.lane_tmem + 64);
+                else if (steps == 3)
+                    relu_to_operand<48>(g.lane_tmem, g.lane_tmem + 64);
+                else if (steps == 2)
+                    relu_to_operand<32>(g.lane_tmem, g.lane_tmem + 64);
+                else
+                    relu_to_operand<16>(g.lane_tmem, g.lane_tmem + 64);
+                g.before_issue();
+                if (g.issues()) {
+                    tc_fence_after();
+                    for (int s = 0; s < steps; ++s)
+                        tc_mma_ta(g.tmem + 96, g.tmem + 64 + 8 * s, tc_desc(w2 + 512 * (4 * c + s)), row_idesc(16), c + s > 0);
+                    if (c + 1 < chunks) layer1(c + 1);
+                    tc_commit(g.bar);
+                }
+            }
+            g.after_commit();
+            uint32_t o[16];   // mu_j, alpha_raw_j
+            tc_ld16(g.lane_tmem + 96, o);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float2 bj = b2[j];
+                const float al = soft_alpha(__uint_as_float(o[2 * j + 1]) + bj.y);
+                x[j] = (x[j] - (__uint_as_float(o[2 * j]) + bj.x)) * exp_sfu(-al);
+                sum_al += al;
+            }
+            // the order reversed for the next block
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float v = x[j];
+                x[j] = x[7 - j];
+                x[7 - j] = v;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) lq.add(log_base(x[j] * inv_tau));
+        if (r < n) logq[r] = lq.plus(-sum_al - 8.f * log_tau);
+    }
+    row_teardown<kDensGroups, kDensColumns>(tmem_s);
+}
+
+// Sampling: the sequential inverse. Column j of a block depends on the hidden
+// units of degree <= j alone, and those on the inputs below j: pass D = 1..7
+// computes the CPD 16-unit steps of degree-D units (all their inputs final),
+// adds their layer-2 contribution to every output, and column D follows. Four
+// groups a CTA, two CTAs an SM; tensor-memory columns 0..47 hold a pass's
+// pre-activations, then (0..23) their bf16, 48..63 the outputs.
+constexpr int kSampGroups = 4, kSampColumns = 64;
+
+template <int K, int CPD>
+__global__ void __launch_bounds__(kSampGroups * kRowGroup, 2) sample_kernel(
+    const uint32_t* __restrict__ pub, int H, const __grid_constant__ Box box, const float* __restrict__ u_in,
+    const __grid_constant__ ModelParams p, uint32_t ctr3, uint64_t first, uint64_t n, float tau, float log_tau,
+    float* __restrict__ theta_out, float* __restrict__ logq_out, int* __restrict__ err)
+{
+    extern __shared__ __align__(128) uint32_t row_sm[];
+    __shared__ __align__(8) uint64_t bar[kSampGroups], bar_stage;
+    __shared__ uint32_t tmem_s;
+    const Layout L = layout(H);
+    RowGroup g = row_setup<kSampGroups, kSampColumns>(row_sm, pub, K, L.s1, L.samp_words, L, err, bar, bar_stage, tmem_s);
+    const uint64_t tiles = (n + kRowGroup - 1) / kRowGroup;
+    for (uint64_t tile = (uint64_t)blockIdx.x * kSampGroups + g.id; tile < tiles; tile += (uint64_t)gridDim.x * kSampGroups) {
+        const uint64_t r = tile * kRowGroup + g.row;
+        LogSum lq;
+        float x[8], sum_al = 0.f;
+        if (u_in) {
+            const float2* src = reinterpret_cast<const float2*>(u_in + 8 * (r < n ? r : n - 1));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 v = src[j];
+                x[2 * j] = v.x;
+                x[2 * j + 1] = v.y;
+            }
+        } else {
+            const uint4 a = rng_block_s(p, first + r, 0, ctr3, 0), c = rng_block_s(p, first + r, 0, ctr3, 1);
+            x[0] = logistic_draw(a.x); x[1] = logistic_draw(a.y); x[2] = logistic_draw(a.z); x[3] = logistic_draw(a.w);
+            x[4] = logistic_draw(c.x); x[5] = logistic_draw(c.y); x[6] = logistic_draw(c.z); x[7] = logistic_draw(c.w);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            lq.add(log_base(x[j]));
+            x[j] *= tau;
+        }
+#pragma unroll 1
+        for (int b = K - 1; b >= 0; --b) {
+            const uint32_t* base = row_sm + b * L.samp_words;
+            const uint32_t w1 = smem_addr(base), w2 = smem_addr(base + L.s2 - L.s1);
+            const float2* b2 = reinterpret_cast<const float2*>(base + L.sb2 - L.s1);
+            // z = x reversed becomes the block's input column by column
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float v = x[j];
+                x[j] = x[7 - j];
+                x[7 - j] = v;
+            }
+            // column 0: every weight into mu_0, alpha_0 is masked
+            {
+                const float2 bj = b2[0];
+                const float al = soft_alpha(bj.y);
+                x[0] = x[0] * exp_sfu(al) + bj.x;
+                sum_al += al;
+            }
+#pragma unroll
+            for (int D = 1; D < 8; ++D) {
+                // input D - 1 is final; the ones above it are still 0
+                if (D == 1)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %2, %2};" ::"r"(g.a1_row()), "r"(pack2(x[0], 0.f)), "r"(0u)
+                                 : "memory");
+                else
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(g.a1_row() + 2 * (D - 1)),
+                                 "h"(__bfloat16_as_ushort(__float2bfloat16_rn(x[D - 1])))
+                                 : "memory");
+                fence_async_smem();
+                g.before_issue();
+                if (g.issues()) {
+                    tc_fence_after();
+                    tc_mma(g.tmem, tc_desc(g.a1), tc_desc(w1 + 512 * CPD * (D - 1)), row_idesc(16 * CPD), 0);
+                    tc_commit(g.bar);
+                }
+                g.after_commit();
+                relu_to_operand<16 * CPD>(g.lane_tmem, g.lane_tmem);
+                g.before_issue();
+                if (g.issues()) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int s = 0; s < CPD; ++s)
+                        tc_mma_ta(g.tmem + 48, g.tmem + 8 * s, tc_desc(w2 + 512 * (CPD * (D - 1) + s)), row_idesc(16), D + s > 1);
+                    tc_commit(g.bar);
+                }
+                g.after_commit();
+                uint32_t o[2];
+                tc_ld2(g.lane_tmem + 48 + 2 * D, o);
+                const float2 bj = b2[D];
+                const float al = soft_alpha(__uint_as_float(o[1]) + bj.y);
+                x[D] = x[D] * exp_sfu(al) + (__uint_as_float(o[0]) + bj.x);
+                sum_al += al;
+            }
+        }
+        float th[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float jac;
+            to_theta(box, j, x[j], th[j], jac);
+            lq.add(-jac);
+        }
+        if (r < n) {
+            float2* to = reinterpret_cast<float2*>(theta_out + 8 * r);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) to[j] = make_float2(th[2 * j], th[2 * j + 1]);
+            if (logq_out) logq_out[r] = lq.plus(-sum_al - 8.f * log_tau);
+        }
+    }
+    row_teardown<kSampGroups, kSampColumns>(tmem_s);
 }
 
 // ---------------------------------------------------------------------------
@@ -683,125 +1128,11 @@ constexpr int kTcM = 128;                          // hidden units per product
 constexpr int kTcHalf = 4096;                      // one A operand: 128 units x 16 rows, bf16
 constexpr int kTcB = 1024;                         // the B slot: g_out (512 B), [x | 1] (512 B)
 constexpr int kTcSlot = 2 * kTcHalf + kTcB;        // shared memory per compute warp
-constexpr uint32_t kTcLBO = 128, kTcSBO = 256;
 // instruction descriptor of kind::f16: FP32 accumulator (bits 4-5), BF16 A
 // and B (bits 7-9, 10-12), both MN-major (bits 15, 16), N >> 3 (bits 17-22),
 // M >> 4 (bits 24-28)
 constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((16u >> 3) << 17) |
                               ((uint32_t)(kTcM >> 4) << 24);
-constexpr unsigned long long kTcWaitNs = 2000000000ull;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void st_u32(unsigned char* p, uint32_t v) { *reinterpret_cast<uint32_t*>(p) = v; }
-
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}" ::"r"(bar) : "memory");
-}
-
-// has the phase of this parity completed (no waiting)
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    return ok != 0;
-}
-
-// waits for the phase of this parity to complete, for at most kTcWaitNs. The
-// clock (a long-latency read of the global timer) starts only once a first
-// try has failed, and is read every 8th try after that: the issuing thread
-// meets mostly completed phases, and a timer read per wait had cost it
-// hundreds of cycles per job.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
-{
-    if (mbar_try(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (uint32_t i = 1;; ++i) {
-        if (mbar_try(bar, parity)) return true;
-        if ((i & 7u) == 0 && global_ns() - t0 > kTcWaitNs) return false;
-    }
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// this thread's shared-memory stores become visible to the tensor cores
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// shared-memory matrix descriptor: start address, leading and stride byte
-// offsets (all >> 4), descriptor version 1 (bit 46), no swizzle
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr)
-{
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(kTcLBO >> 4) << 16) | ((uint64_t)(kTcSBO >> 4) << 32) |
-           (1ull << 46);
-}
-
-// D (TMEM) = A B + (accumulate ? D : 0)
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate)
-{
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d), "l"(a), "l"(b), "r"(kTcIdesc), "r"(accumulate)
-                 : "memory");
-}
-
-// arrives on the barrier once every product this thread issued has completed
-__device__ __forceinline__ void tc_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// 16 consecutive 32-bit columns of this warp's 32 TMEM lanes (lane i: thread i)
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-                 "tcgen05.wait::ld.sync.aligned;"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                   "=r"(v[15])
-                 : "r"(taddr)
-                 : "memory");
-}
-
-// 32 consecutive 32-bit columns of this warp's 32 TMEM lanes (lane i: thread i)
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-                 "tcgen05.wait::ld.sync.aligned;"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                   "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-                   "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-                   "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                 : "r"(taddr)
-                 : "memory");
-}
-
 // one hidden unit's dW1 row (eight inputs, masked) as two 16-byte stores
 __device__ __forceinline__ void store_dw1(float* __restrict__ row, int l, const uint32_t* v)
 {
@@ -811,38 +1142,6 @@ __device__ __forceinline__ void store_dw1(float* __restrict__ row, int l, const 
     float4* r4 = reinterpret_cast<float4*>(row);
     r4[0] = make_float4(w[0], w[1], w[2], w[3]);
     r4[1] = make_float4(w[4], w[5], w[6], w[7]);
-}
-
-// mbarrier arrival that also adds `bytes` to the transaction count of the
-// current phase (the bytes bulk copies will complete on it)
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
-
-// bulk copy (no tensor map) of `bytes` from global to this CTA's shared
-// memory, completing on the mbarrier; both addresses and the size are
-// multiples of 16 bytes
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
-// The K blocks' words [off, off + n) of the published operands, copied into
-// sm (K x n words, packed) by the bulk-copy engine: thread 0 sets the
-// barrier's transaction count and issues one copy per block. The barrier was
-// initialised (count 1) and that made visible to the CTA before the call.
-// Offsets and sizes are multiples of 4 words (16 bytes), as the bulk copy
-// requires: every section of the layout is, since H is a multiple of 16.
-__device__ __forceinline__ void stage_blocks_bulk(uint32_t* sm, const uint32_t* pub, int K, int off, int n,
-                                                  const Layout& L, uint32_t bar)
-{
-    if (threadIdx.x != 0) return;
-    mbar_arrive_expect_tx(bar, (uint32_t)(K * n) * 4u);
-    for (int b = 0; b < K; ++b) bulk_g2s(smem_addr(sm + b * n), pub + (size_t)b * L.words + off, (uint32_t)n * 4u, bar);
 }
 
 // The two warps of a pair add their partial sums: each stores its N values per
@@ -998,7 +1297,7 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
     if (warp < W && tile0 < tiles)
         first = tile_rows(tile0, lane >> 2, lane & 3, lane, n_rows, ticket != nullptr, rp, step_now, f, slot);
     griddep_wait();
-    stage_blocks_bulk(wsm, pub, K, 0, L.grad_words, L, smem_addr(&bar_stage));
+    stage_blocks_bulk(wsm, pub, K, L.w1, L.grad_words, L, smem_addr(&bar_stage));
     griddep_release();
     // the operands staged (a wait that runs out sets the error word; the
     // CTA's result is then not used, but it still runs to its end)
@@ -1216,8 +1515,8 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
                     const uint32_t sb = sa + 2 * kTcHalf;
                     const uint32_t acc = (init >> d) & 1u;
                     init |= 1u << d;
-                    tc_mma(tmem + 32 * d, tc_desc(sa), tc_desc(sb), acc);
-                    tc_mma(tmem + 32 * d + 16, tc_desc(sa + kTcHalf), tc_desc(sb + 512), acc);
+                    tc_mma(tmem + 32 * d, tc_desc(sa), tc_desc(sb), kTcIdesc, acc);
+                    tc_mma(tmem + 32 * d + 16, tc_desc(sa + kTcHalf), tc_desc(sb + 512), kTcIdesc, acc);
                 }
                 pending = 0;
             };
@@ -1484,16 +1783,15 @@ __global__ void __launch_bounds__(256) early_stop_kernel(const float* __restrict
 }
 
 // Master parameter r of one block (W1 [H][8], b1 [H], W2 [16][H], b2 [16]),
-// value val, written to every place the published layout holds it: the
-// forward and backward operands and the sampler's copy, as BF16 halves of
-// their words (masked weights as 0) or whole FP32 words. The words of a layout
+// value val, written to every place the gradient's operands hold it, as BF16
+// halves of their words (masked weights as 0) or whole FP32 words. The words
 // hold two parameters each; storing each half separately lets one thread per
-// parameter publish without the other. The layout's padding is never written
-// here (a full publish zeroes it).
+// parameter publish without the other. The padding is never written here (a
+// full publish zeroes it), nor are the density's and the sampler's operands:
+// no step of a training run reads them, and the run ends with a full publish.
 __device__ __forceinline__ void publish_param(uint32_t* __restrict__ pb, int H, const Layout& L, int r, float val)
 {
     unsigned short* h16 = reinterpret_cast<unsigned short*>(pb);
-    const int cpd = sampler_cpd(H);
     if (r < 8 * H) {
         const int l = r >> 3, j = r & 7;
         const unsigned short bf = mask1(l, j) ? __bfloat16_as_ushort(__float2bfloat16_rn(val)) : (unsigned short)0;
@@ -1502,15 +1800,10 @@ __device__ __forceinline__ void publish_param(uint32_t* __restrict__ pb, int H, 
         h16[2 * (L.w1 + (((l >> 4) * 8 + (l & 7)) * 4 + t) * 2 + ((l >> 3) & 1)) + (j & 1)] = bf;
         // w1t: word [j][l / 2]
         h16[2 * (L.w1t + j * (H / 2 + 4) + (l >> 1)) + (l & 1)] = bf;
-        // sampler copy: unit l sits at position u of chunk sc
-        const int i = l / 7, sc = (l % 7) * cpd + (i >> 4), u = i & 15;
-        h16[2 * (L.sw1 + ((sc * 8 + (u & 7)) * 4 + t) * 2 + (u >> 3)) + (j & 1)] = bf;
     } else if (r < 9 * H) {
         const int l = r - 8 * H, rem = l & 15;
         // b1: word (s 4 + t) 4 + q for hidden 16 s + 8 (q / 2) + 2 t + q % 2
         pb[L.b1 + ((l >> 4) * 4 + ((rem & 7) >> 1)) * 4 + ((rem >> 3) << 1 | (rem & 1))] = __float_as_uint(val);
-        const int i = l / 7, sc = (l % 7) * cpd + (i >> 4), u = i & 15;
-        pb[L.sb1 + (sc * 4 + ((u & 7) >> 1)) * 4 + ((u >> 3) << 1 | (u & 1))] = __float_as_uint(val);
     } else if (r < 25 * H) {
         const int o = (r - 9 * H) / H, l = (r - 9 * H) - o * H, rem = l & 15;
         const unsigned short bf = mask2(o, l) ? __bfloat16_as_ushort(__float2bfloat16_rn(val)) : (unsigned short)0;
@@ -1520,12 +1813,8 @@ __device__ __forceinline__ void publish_param(uint32_t* __restrict__ pb, int H, 
             (l & 1)] = bf;
         // w2t: word l 8 + ((o / 2) ^ (l & 4)), output o / 2 * 2 low, +1 high
         h16[2 * (L.w2t + l * 8 + ((o >> 1) ^ (l & 4))) + (o & 1)] = bf;
-        const int i = l / 7, sc = (l % 7) * cpd + (i >> 4), u = i & 15;
-        h16[2 * (L.sw2 + ((sc * 8 + (o & 7)) * 4 + ((u & 7) >> 1)) * 4 + ((o >> 3) << 1 | (u >> 3))) + (u & 1)] = bf;
     } else {
-        const int o = r - 25 * H;
-        pb[L.b2 + o] = __float_as_uint(val);
-        pb[L.sb2 + o] = __float_as_uint(val);
+        pb[L.b2 + r - 25 * H] = __float_as_uint(val);
     }
 }
 
@@ -1705,8 +1994,11 @@ abc_status take_err(abc_maf f)
     return ABC_OK;
 }
 
-size_t fwd_smem(const abc_maf_s* f) { return sizeof(uint32_t) * (size_t)f->K * maf::layout(f->H).fwd_words; }
-size_t samp_smem(const abc_maf_s* f) { return sizeof(uint32_t) * (size_t)f->K * maf::layout(f->H).samp_words; }
+// the K blocks' operands and every group's layer-1 rows
+size_t row_smem(const abc_maf_s* f, int words, int groups)
+{
+    return sizeof(uint32_t) * (size_t)f->K * words + (size_t)groups * maf::kRowGroup * 32;
+}
 
 size_t grad_smem(const abc_maf_s* f, int warps)
 {
@@ -1786,16 +2078,53 @@ cudaError_t publish(abc_maf f, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// CTAs of the density and sampling kernels: one for each CTA's worth of rows, at
+// most the two an SM's tensor memory holds (fewer where shared memory for two
+// is lacking). Not from the occupancy query: it says one CTA per SM for any
+// kernel that allocates tensor memory, and two run at once all the same.
+int row_grid(int threads, size_t smem, uint64_t n)
+{
+    constexpr size_t kStaticAndReserved = 2 * 1024;   // a CTA's static shared memory and what the system takes
+    int dev = 0, sm_smem = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const uint64_t per_sm = 2 * (smem + kStaticAndReserved) <= (size_t)sm_smem ? 2 : 1;
+    const uint64_t want = (n + threads - 1) / threads, cap = per_sm * (uint64_t)sm_count();
+    return (int)(want < cap ? want : cap);
+}
+
+// Points from which the density and the sampler run in the tcgen05 form (us,
+// this form against the mma.sync one, blocks x hidden units):
+//              3 x 256           4 x 176           2 x 64
+//   sampler  60,000  23.5 / 21.8   25.4 / 23.4   15.4 / 13.1
+//           100,000  29.2 / 29.9   29.8 / 31.5   18.0 / 15.8
+//           150,000  29.5 / 42.0   30.4 / 44.0   18.5 / 21.3
+//           300,000  51.0 / 71.0   54.3 / 72.7   29.8 / 34.3
+//   density 100,000  23.2 / 21.7   23.1 / 22.7   12.4 / 10.2
+//           200,000  35.2 / 34.7   35.4 / 35.6   15.2 / 15.1
+//           300,000  45.1 / 49.2   45.8 / 50.0   19.1 / 19.3
+//           500,000  68.5 / 76.6   70.4 / 78.4   27.1 / 29.4
+constexpr uint64_t kSampleRows = 100000, kLogqRows = 300000;
+
 template <int K>
 cudaError_t launch_logq(abc_maf f, int r, uint64_t n, const float* theta, float* logq, cudaStream_t s)
 {
-    const size_t smem = fwd_smem(f);
+    const float inv_tau = 1.f / f->tau, log_tau = logf(f->tau);
+    if (n < kLogqRows) {
+        const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).fwd_words;
+        cudaError_t e = allow_smem(maf::logq_few_kernel<K>, smem);
+        if (e != cudaSuccess) return e;
+        const int grid = fill_grid(maf::logq_few_kernel<K>, maf::kFwdThreads, smem, (n + 127) / 128);
+        maf::logq_few_kernel<K><<<grid, maf::kFwdThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n, inv_tau, log_tau,
+                                                                     logq);
+        return cudaGetLastError();
+    }
+    constexpr int kThreads = maf::kDensGroups * maf::kRowGroup;
+    const size_t smem = row_smem(f, maf::layout(f->H).dens_words, maf::kDensGroups);
     cudaError_t e = allow_smem(maf::logq_kernel<K>, smem);
     if (e != cudaSuccess) return e;
-    const uint64_t tiles = (n + 15) / 16;
-    const int grid = fill_grid(maf::logq_kernel<K>, maf::kFwdThreads, smem, (tiles + 7) / 8);
-    maf::logq_kernel<K><<<grid, maf::kFwdThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n, 1.f / f->tau, logf(f->tau),
-                                                logq);
+    maf::logq_kernel<K><<<row_grid(kThreads, smem, n), kThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n, inv_tau,
+                                                                           log_tau, logq, f->d_err);
     return cudaGetLastError();
 }
 
@@ -1803,13 +2132,22 @@ template <int K, int CPD>
 cudaError_t launch_sample_c(abc_maf f, int r, uint64_t n, const float* u, const ModelParams& p, uint32_t ctr3,
                             uint64_t first, float* theta, float* logq, cudaStream_t s)
 {
-    const size_t smem = samp_smem(f);
+    const float log_tau = logf(f->tau);
+    if (n < kSampleRows) {
+        const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).msamp_words;
+        cudaError_t e = allow_smem(maf::sample_few_kernel<K, CPD>, smem);
+        if (e != cudaSuccess) return e;
+        const int grid = fill_grid(maf::sample_few_kernel<K, CPD>, maf::kFwdThreads, smem, (n + 127) / 128);
+        maf::sample_few_kernel<K, CPD><<<grid, maf::kFwdThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n,
+                                                                            f->tau, log_tau, theta, logq);
+        return cudaGetLastError();
+    }
+    constexpr int kThreads = maf::kSampGroups * maf::kRowGroup;
+    const size_t smem = row_smem(f, maf::layout(f->H).samp_words, maf::kSampGroups);
     cudaError_t e = allow_smem(maf::sample_kernel<K, CPD>, smem);
     if (e != cudaSuccess) return e;
-    const uint64_t tiles = (n + 15) / 16;
-    const int grid = fill_grid(maf::sample_kernel<K, CPD>, maf::kFwdThreads, smem, (tiles + 7) / 8);
-    maf::sample_kernel<K, CPD><<<grid, maf::kFwdThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau,
-                                                  logf(f->tau), theta, logq);
+    maf::sample_kernel<K, CPD><<<row_grid(kThreads, smem, n), kThreads, smem, s>>>(
+        flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, log_tau, theta, logq, f->d_err);
     return cudaGetLastError();
 }
 
@@ -2425,9 +2763,10 @@ abc_status abc_maf_train_flows(abc_maf f, const float* const* theta, const float
         return plan_ok();
     }
     if (n_steps > 0) {
-        // each step publishes every parameter it updates, the sampler's
-        // operands included
+        // each step publishes the gradient's operands of every parameter it
+        // updates; the density's and the sampler's follow here
         MAF_TRY(run_steps(f, n_steps, s), "cudaGraphLaunch");
+        MAF_TRY(publish(f, s), "publish");
     }
     if (loss_out) {
         MAF_TRY(full_gradient(f, max_n, s), "flow loss");

@@ -83,6 +83,54 @@ def test_sample_matches_oracle_inverse(K, H):
     f.close()
 
 
+# one, two and three 16-unit steps a degree; one to four chunks of 64 units, the
+# last one of 16, 32, 48 or 64; a last tile of 1, 31, 127 and 128 rows
+@pytest.mark.parametrize("K,H,extra", [(1, 16, 1), (2, 64, 31), (2, 112, 128), (3, 208, 127), (4, 256, 0), (3, 160, 129)])
+def test_many_points_match_few_and_the_oracle(K, H, extra):
+    """From a number of points on, sampling and density run in another form
+    (tcgen05, a thread per row). It is held against the form for few points, row
+    by row in tiles of 128, and against the oracle on the last rows. Both forms
+    round the same values to bf16, so a row differs by a few float32 steps but
+    where one falls on a bf16 boundary (2^-9 of an input): the median of every
+    tile and the last rows' quantiles carry the bounds of the oracle tests."""
+    f, params = _flow(K, H, 60 + K, 0.3)
+    n = 128 * 2400 + extra                  # above both forms' lines; a last wave that is not full
+    g = torch.Generator(device="cpu").manual_seed(K)
+    u = torch.rand(n, 8, generator=g).clamp(1e-6, 1 - 1e-6)
+    u = torch.log(u / (1 - u)).to(DEV)
+    pad = torch.empty(8 * n + 2, device=DEV)
+    base = pad[2:].view(n, 8)               # 8-byte aligned rows
+    base.copy_(u)
+    few = 128 * 640
+
+    def parts(fn):
+        return [torch.cat(c) for c in zip(*(fn(slice(i, min(i + few, n))) for i in range(0, n, few)))]
+
+    def per_tile(err):
+        err = err.flatten(1).amax(1) if err.dim() > 1 else err
+        m = n // 128 * 128
+        return err[:m].view(-1, 128).median(1).values.max().item()
+
+    width = torch.tensor(HI - LO, dtype=torch.float32, device=DEV)
+    th, lq = f.sample(n, base=base)
+    th2, lq2 = parts(lambda i: f.sample(i.stop - i.start, base=u[i]))
+    d = f.log_q(th)
+    d2, = parts(lambda i: (f.log_q(th[i]),))
+    e_th, e_lq, e_d = per_tile((th - th2).abs() / width), per_tile((lq - lq2).abs()), per_tile((d - d2).abs())
+    print("many points K=%d H=%d: largest tile median theta %.1e logq %.1e density %.1e" % (K, H, e_th, e_lq, e_d))
+    assert e_th < 1e-5 and e_lq < 1e-4 and e_d < 1e-4
+    s1, l1 = f.sample(n, seed=3, stream=2, first_index=(1 << 32) - 7)
+    s2, _ = f.sample(few - 5, seed=3, stream=2, first_index=(1 << 32) - 2)
+    assert ((s1[5:few] - s2).abs() / width).flatten(1).amax(1).median().item() < 1e-5
+    tail = slice(n - 200, n)
+    y, lqy = mo.inverse(u[tail].cpu().numpy().astype(np.float64), params, bf16=True)
+    ref = mo.to_theta(y, LO, HI)
+    rel = np.abs(th[tail].cpu().numpy() - ref) / (HI - LO)
+    errq = np.abs(lq[tail].cpu().numpy() - (lqy - mo.log_jacobian_y(y, LO, HI)))
+    assert np.median(rel) < 1e-5 and np.quantile(rel, 0.95) < 1e-3
+    assert np.median(errq) < 1e-4 and np.quantile(errq, 0.95) < 5e-3
+    f.close()
+
 def test_zero_flow_draws_the_prior_from_the_documented_words():
     """A flow with zero parameters is the uniform prior: base coordinate c of
     sample j is logit(u), u = (2m + 1) 2^-24 from word c mod 4 of the Philox
