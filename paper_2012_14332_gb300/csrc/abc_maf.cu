@@ -24,6 +24,7 @@
 #include <map>
 #include <mutex>
 #include <random>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -323,25 +324,57 @@ __device__ __forceinline__ void made_fwd(const BlockView& v, int H, const float 
 }
 
 // The partial MADE outputs (without b2) of hidden chunks [s0, s1) on the
-// warp's 16 rows: the contributions to mu and alpha_raw, even and odd chunks in
-// separate chains added at the end.
+// warp's 16 rows: the contributions to mu and alpha_raw. Four chunks at a time,
+// stage by stage (four independent chains of products); even and odd chunks
+// accumulate separately, summed at the end.
 __device__ __forceinline__ void made_part(const BlockView& v, int s0, int s1, const float (&x)[4], float (&pm)[4],
                                           float (&pa)[4])
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const uint32_t a0 = pack2(x[0], x[1]), a1 = pack2(x[2], x[3]);
-    float o0[4] = {0.f, 0.f, 0.f, 0.f}, o1[4] = {0.f, 0.f, 0.f, 0.f};
-    float p0[4] = {0.f, 0.f, 0.f, 0.f}, p1[4] = {0.f, 0.f, 0.f, 0.f};
+    float o[2][2][4] = {};
+    const auto group = [&](auto nb, int s) {
+        constexpr int NB = decltype(nb)::value;
+        uint2 wa[NB];
+        uint4 wb[NB];
+        float c[NB][2][4];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            wa[i] = reinterpret_cast<const uint2*>(v.w1)[((s + i) * 8 + g) * 4 + t];
+            wb[i] = reinterpret_cast<const uint4*>(v.w2)[((s + i) * 8 + g) * 4 + t];
+            const float4 bb = reinterpret_cast<const float4*>(v.b1)[(s + i) * 4 + t];
+            c[i][0][0] = c[i][0][2] = bb.x;
+            c[i][0][1] = c[i][0][3] = bb.y;
+            c[i][1][0] = c[i][1][2] = bb.z;
+            c[i][1][1] = c[i][1][3] = bb.w;
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            mma_k8_p(c[i][0], a0, a1, wa[i].x);
+            mma_k8_p(c[i][1], a0, a1, wa[i].y);
+        }
+        uint32_t A[NB][4];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                A[i][2 * h] = pack2_relu(c[i][h][0], c[i][h][1]);
+                A[i][2 * h + 1] = pack2_relu(c[i][h][2], c[i][h][3]);
+            }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            mma_k16_p(o[i & 1][0], A[i][0], A[i][1], A[i][2], A[i][3], wb[i].x, wb[i].y);
+            mma_k16_p(o[i & 1][1], A[i][0], A[i][1], A[i][2], A[i][3], wb[i].z, wb[i].w);
+        }
+    };
     int s = s0;
-    for (; s + 1 < s1; s += 2) {
-        made_chunk(v, s, g, t, a0, a1, o0, o1);
-        made_chunk(v, s + 1, g, t, a0, a1, p0, p1);
-    }
-    if (s < s1) made_chunk(v, s, g, t, a0, a1, o0, o1);
+    for (; s + 4 <= s1; s += 4) group(std::integral_constant<int, 4>{}, s);
+    for (; s + 2 <= s1; s += 2) group(std::integral_constant<int, 2>{}, s);
+    if (s < s1) group(std::integral_constant<int, 1>{}, s);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        pm[e] = o0[e] + p0[e];
-        pa[e] = o1[e] + p1[e];
+        pm[e] = o[0][0][e] + o[1][0][e];
+        pa[e] = o[0][1][e] + o[1][1][e];
     }
 }
 
@@ -1228,7 +1261,7 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
     static_assert(!PAIR || W % 2 == 0, "whole pairs");
     constexpr int TPC = PAIR ? W / 2 : W;   // tiles a CTA works on at once
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bar_full[W], bar_round, bar_done, bar_stage;
+    __shared__ __align__(8) uint64_t bar_full[W], bar_round, bar_done, bar_stage[K];
     __shared__ uint32_t tmem_s, init_s;
     __shared__ float ssum_w[W][2];       // per compute warp: weighted loss sum, weight sum
     __shared__ float gb2_w[W][K * 16];   // per compute warp: db2 sums
@@ -1252,7 +1285,7 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
     uint32_t* wsm = reinterpret_cast<uint32_t*>(smem + W * kTcSlot);
     // the published operands arrive by bulk copy while the CTA sets up
     if (threadIdx.x == 0) {
-        mbar_init(smem_addr(&bar_stage), 1);
+        for (int b = 0; b < K; ++b) mbar_init(smem_addr(&bar_stage[b]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -1297,11 +1330,14 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
     if (warp < W && tile0 < tiles)
         first = tile_rows(tile0, lane >> 2, lane & 3, lane, n_rows, ticket != nullptr, rp, step_now, f, slot);
     griddep_wait();
-    stage_blocks_bulk(wsm, pub, K, L.w1, L.grad_words, L, smem_addr(&bar_stage));
+    // block b's operands on a barrier of their own, so the first block's forward
+    // pass starts when they are in (warp 0 always has a tile: its forward pass
+    // waits for every block's copy before the CTA can end)
+#pragma unroll
+    for (int b = 0; b < K; ++b)
+        stage_blocks_bulk(wsm + b * L.grad_words, pub + (size_t)b * L.words, 1, L.w1, L.grad_words, L,
+                          smem_addr(&bar_stage[b]));
     griddep_release();
-    // the operands staged (a wait that runs out sets the error word; the
-    // CTA's result is then not used, but it still runs to its end)
-    if (!mbar_wait(smem_addr(&bar_stage), 0) && lane == 0) atomicExch(err, 1);
     const uint32_t tmem = tmem_s;
     if (warp < W) {
         const int g = lane >> 2, t = lane & 3, rg = 16 * g + 4 * t, sw = g & 4;
@@ -1331,6 +1367,9 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
 #pragma unroll
             for (int b = 0; b < K; ++b) {
                 float mu[4], ar[4];
+                // the block's operands staged (a wait that runs out sets the error
+                // word; the CTA's result is then not used, but it runs to its end)
+                if (tile == tile0 && !mbar_wait(smem_addr(&bar_stage[b]), 0) && lane == 0) atomicExch(err, 1);
                 if constexpr (PAIR) {
                     const BlockView v = view(wsm + b * L.grad_words, L);
                     float pm[4], pa[4];
@@ -1408,36 +1447,64 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
                         gb2_w[warp][16 * b + 9 + 2 * t] += d[3];
                     }
                 }
-                // one 16-unit chunk; even and odd chunks keep separate g_x sums
-                // (independent chains the compiler can interleave)
-                auto chunk = [&](int s, float (&accx)[4]) {
-                    const int q = s & 7;   // chunk within the 128-unit half
-                    // recompute the pre-activations of hidden units 16s .. 16s+15
-                    const uint2 wa = reinterpret_cast<const uint2*>(v.w1)[(s * 8 + g) * 4 + t];
-                    const float4 bq = reinterpret_cast<const float4*>(v.b1)[s * 4 + t];
-                    float c0[4] = {bq.x, bq.y, bq.x, bq.y}, c1[4] = {bq.z, bq.w, bq.z, bq.w};
-                    mma_k8_p(c0, xa0, xa1, wa.x);
-                    mma_k8_p(c1, xa0, xa1, wa.y);
-                    // g_h = g_out W2 for these units, then through the ReLU
-                    const uint32_t* w2r0 = v.w2t + (16 * s + g) * 8;
-                    const uint32_t* w2r1 = w2r0 + 64;
-                    float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma_k16_p(d0, A0, A1, A2, A3, w2r0[t ^ sw], w2r0[(4 ^ sw) + t]);
-                    mma_k16_p(d1, A0, A1, A2, A3, w2r1[t ^ sw], w2r1[(4 ^ sw) + t]);
+                // NB 16-unit chunks s .. s + NB - 1 together: their loads, then
+                // their products stage by stage, so NB independent chains are in
+                // flight (the stores into the A slot end a group: no later load
+                // moves above them). Even and odd chunks keep separate g_x sums.
+                float ax[2][4] = {};
+                const auto group = [&](auto nb, int s) {
+                    constexpr int NB = decltype(nb)::value;
+                    uint2 wa[NB];
+                    float4 bq[NB];
+                    uint32_t wt[NB][4], wx[NB][2];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        d0[e] = c0[e] > 0.f ? d0[e] : 0.f;
-                        d1[e] = c1[e] > 0.f ? d1[e] : 0.f;
+                    for (int i = 0; i < NB; ++i) {
+                        wa[i] = reinterpret_cast<const uint2*>(v.w1)[((s + i) * 8 + g) * 4 + t];
+                        bq[i] = reinterpret_cast<const float4*>(v.b1)[(s + i) * 4 + t];
+                        const uint32_t* w2r0 = v.w2t + (16 * (s + i) + g) * 8;
+                        const uint32_t* w2r1 = w2r0 + 64;
+                        wt[i][0] = w2r0[t ^ sw];
+                        wt[i][1] = w2r0[(4 ^ sw) + t];
+                        wt[i][2] = w2r1[t ^ sw];
+                        wt[i][3] = w2r1[(4 ^ sw) + t];
+                        wx[i][0] = v.w1t[g * hw + 8 * (s + i) + t];
+                        wx[i][1] = v.w1t[g * hw + 8 * (s + i) + 4 + t];
                     }
-                    const uint32_t P0 = pack2(d0[0], d0[1]), P1 = pack2(d0[2], d0[3]);
-                    const uint32_t P2 = pack2(d1[0], d1[1]), P3 = pack2(d1[2], d1[3]);
-                    // g_x += g_a1 W1 (this chunk's 16 hidden units as k)
-                    mma_k16_p(accx, P0, P1, P2, P3, v.w1t[g * hw + 8 * s + t], v.w1t[g * hw + 8 * s + 4 + t]);
+                    float c[NB][2][4], d[NB][2][4] = {};
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {   // the pre-activations again
+                        c[i][0][0] = c[i][0][2] = bq[i].x;
+                        c[i][0][1] = c[i][0][3] = bq[i].y;
+                        c[i][1][0] = c[i][1][2] = bq[i].z;
+                        c[i][1][1] = c[i][1][3] = bq[i].w;
+                        mma_k8_p(c[i][0], xa0, xa1, wa[i].x);
+                        mma_k8_p(c[i][1], xa0, xa1, wa[i].y);
+                    }
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {   // g_h = g_out W2
+                        mma_k16_p(d[i][0], A0, A1, A2, A3, wt[i][0], wt[i][1]);
+                        mma_k16_p(d[i][1], A0, A1, A2, A3, wt[i][2], wt[i][3]);
+                    }
+                    uint32_t P[NB][4];
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {   // through the ReLU
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) d[i][h][e] = c[i][h][e] > 0.f ? d[i][h][e] : 0.f;
+                            P[i][2 * h] = pack2(d[i][h][0], d[i][h][1]);
+                            P[i][2 * h + 1] = pack2(d[i][h][2], d[i][h][3]);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < NB; ++i)   // g_x += g_a1 W1 (a chunk's 16 hidden units as k)
+                        mma_k16_p(ax[i & 1], P[i][0], P[i][1], P[i][2], P[i][3], wx[i][0], wx[i][1]);
                     // h and g_a1 of these units into the A slot (core matrices
                     // 2q and 2q + 1 along M); a job's first chunk waits until the
                     // products of the warp's previous job have read the slot;
                     // after one wait has run out the warp skips the rest, so a
                     // failed call returns within about one wait limit
+                    const int q = s & 7;   // chunk within the 128-unit half
                     if (q == 0 && job > 0 && ok) ok = mbar_wait(empty, (job - 1) & 1u);
                     if (s == s_lo) {
                         // the previous job was the previous block's last: the B slot is free
@@ -1448,31 +1515,37 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
                         st_u32(sB + 512 + rg, xa0);
                         st_u32(sB + 640 + rg, xa1);
                     }
-                    unsigned char* a = sA + 512 * q + rg;
-                    st_u32(a, pack2_relu(c0[0], c0[1]));
-                    st_u32(a + 128, pack2_relu(c0[2], c0[3]));
-                    st_u32(a + 256, pack2_relu(c1[0], c1[1]));
-                    st_u32(a + 384, pack2_relu(c1[2], c1[3]));
-                    st_u32(a + kTcHalf, P0);
-                    st_u32(a + kTcHalf + 128, P1);
-                    st_u32(a + kTcHalf + 256, P2);
-                    st_u32(a + kTcHalf + 384, P3);
-                    if (q == 7 || s == chunks - 1) {
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        unsigned char* a = sA + 512 * (q + i) + rg;
+                        st_u32(a, pack2_relu(c[i][0][0], c[i][0][1]));
+                        st_u32(a + 128, pack2_relu(c[i][0][2], c[i][0][3]));
+                        st_u32(a + 256, pack2_relu(c[i][1][0], c[i][1][1]));
+                        st_u32(a + 384, pack2_relu(c[i][1][2], c[i][1][3]));
+                        st_u32(a + kTcHalf, P[i][0]);
+                        st_u32(a + kTcHalf + 128, P[i][1]);
+                        st_u32(a + kTcHalf + 256, P[i][2]);
+                        st_u32(a + kTcHalf + 384, P[i][3]);
+                    }
+                    if (q + NB == 8 || s + NB == chunks) {
                         fence_async_smem();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(full);
                         ++job;
                     }
                 };
-                float ax0[4] = {0.f, 0.f, 0.f, 0.f}, ax1[4] = {0.f, 0.f, 0.f, 0.f};
+                // Chunk by chunk a step of 4096 rows at 3 x 256 takes 18.1 us, two
+                // together 17.0, four 16.6, eight 16.6 (and 19.0 instead of 17.5 for
+                // 2048 at 4 x 256); the wide form has 128 registers a thread.
+                constexpr int GROUP = W <= 8 ? 4 : 2;
                 int s = s_lo;
-                for (; s + 1 < s_hi; s += 2) {
-                    chunk(s, ax0);
-                    chunk(s + 1, ax1);
-                }
-                if (s < s_hi) chunk(s, ax0);
+                for (; s + GROUP <= s_hi; s += GROUP) group(std::integral_constant<int, GROUP>{}, s);
+                if constexpr (GROUP > 2)
+                    for (; s + 2 <= s_hi; s += 2) group(std::integral_constant<int, 2>{}, s);
+                if (s < s_hi) group(std::integral_constant<int, 1>{}, s);
+                float ax0[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) ax0[e] += ax1[e];
+                for (int e = 0; e < 4; ++e) ax0[e] = ax[0][e] + ax[1][e];
                 if constexpr (PAIR) pair_add<4>(xbuf, xc, member, 1 + pair, lane, ax0);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) gx[e] = gxd[e] + ax0[e];
@@ -1616,6 +1689,73 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
+// The weighted loss sums alone over all points of every flow's slot (a training
+// run's validation checks), for grad_reduce_kernel: the gradient
+// kernel's forward pass, a warp per 16 rows and several CTAs an SM, each CTA's two
+// sums in its slot of the partials, its warps' in warp order: 9.5 us for 8000 points
+// at 3 x 256. The gradient kernel gives them too, at the price of the backward pass
+// (most of a step on 8192 rows, 23.6 us).
+template <int K>
+__global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) loss_kernel(const uint32_t* __restrict__ pub, int H,
+                                                                          const __grid_constant__ Box box,
+                                                                          const TrainSlot* __restrict__ slots,
+                                                                          float* __restrict__ part, uint32_t part_stride)
+{
+    extern __shared__ __align__(16) uint32_t sm[];
+    constexpr int kWarps = kFwdThreads / 32;
+    __shared__ float sums_w[kWarps][2];
+    const Layout L = layout(H);
+    const int f = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const TrainSlot slot = slots[f];
+    if (slot.n == 0) return;   // uniform over the block
+    stage_blocks(sm, pub + (size_t)f * K * L.words, K, L.w1, L.fwd_words, L);
+    __syncthreads();
+    const uint64_t tiles = (slot.n + 15) / 16;
+    float contrib = 0.f, wsum = 0.f;   // lanes t = 0: their rows'
+    for (uint64_t tile = (uint64_t)blockIdx.x * kWarps + warp; tile < tiles; tile += (uint64_t)gridDim.x * kWarps) {
+        const TileRows rows = tile_rows(tile, g, t, lane, slot.n, false, ModelParams{}, 0u, f, slot);
+        float x[4], jac, ld0 = 0.f, ld1 = 0.f;
+        to_y(box, 2 * t, rows.ta.x, x[0], jac);
+        to_y(box, 2 * t + 1, rows.ta.y, x[1], jac);
+        to_y(box, 2 * t, rows.tb.x, x[2], jac);
+        to_y(box, 2 * t + 1, rows.tb.y, x[3], jac);
+#pragma unroll 1
+        for (int b = 0; b < K; ++b) {
+            float mu[4], ar[4], al[4];
+            made_fwd(view(sm + b * L.fwd_words, L), H, x, mu, ar);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                al[e] = soft_alpha(ar[e]);
+                x[e] = (x[e] - mu[e]) * __expf(-al[e]);
+            }
+            ld0 += al[0] + al[1];
+            ld1 += al[2] + al[3];
+            reverse_cols(x);
+        }
+        const float n0 = quad_sum(ld0 - log_base(x[0]) - log_base(x[1]));
+        const float n1 = quad_sum(ld1 - log_base(x[2]) - log_base(x[3]));
+        if (t == 0) {
+            contrib += rows.w0 * n0 + rows.w1 * n1;
+            wsum += rows.w0 + rows.w1;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        contrib += __shfl_xor_sync(kFull, contrib, off);
+        wsum += __shfl_xor_sync(kFull, wsum, off);
+    }
+    if (lane == 0) {
+        sums_w[warp][0] = contrib;
+        sums_w[warp][1] = wsum;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        float a = 0.f;
+        for (int w = 0; w < kWarps; ++w) a += sums_w[w][threadIdx.x];
+        part[((size_t)f * gridDim.x + blockIdx.x) * part_stride + (size_t)K * master_block(H) + threadIdx.x] = a;
+    }
+}
+
 // The CTAs' partials are added in a fixed tree. A 256-thread block covers
 // E = 256 / G consecutive entries in G groups: thread (q, e) adds the partials
 // of CTAs q, q + G, q + 2G, ... of entry e in that order, with a chunk's loads
@@ -1635,7 +1775,7 @@ __device__ __forceinline__ float group_sum(const float* __restrict__ q, int nblk
 #pragma unroll
         for (int k = 0; k < kRedUnroll; ++k) {
             const int c = c0 + G * k;
-            x[k] = c < nblk ? q[(size_t)c * stride] : 0.f;
+            x[k] = c < nblk ? __ldcg(q + (size_t)c * stride) : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < kRedUnroll; ++k) a += x[k];
@@ -1656,8 +1796,8 @@ __device__ __forceinline__ void group_sum2(const float* __restrict__ q, int off,
 #pragma unroll
         for (int k = 0; k < kRedUnroll; ++k) {
             const int c = c0 + G * k;
-            x[k] = has0 && c < nblk ? q[(size_t)c * stride] : 0.f;
-            y[k] = has1 && c < nblk ? q[(size_t)c * stride + off] : 0.f;
+            x[k] = has0 && c < nblk ? __ldcg(q + (size_t)c * stride) : 0.f;
+            y[k] = has1 && c < nblk ? __ldcg(q + (size_t)c * stride + off) : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < kRedUnroll; ++k) {
@@ -1688,22 +1828,19 @@ __device__ __forceinline__ float block_groups_total(float (*gs)[256 / G], float 
 // The flows' gradients and loss sums from the CTAs' partials, in the fixed
 // tree above: grad[f][p] (p < np), then the two loss sums, for the entries
 // from p_first on (np: the loss sums alone). A flow without rows gets zeros
-// (its CTAs returned before writing). drawn: the gradient was over `batch`
-// drawn rows per flow, else over all of each flow's points.
+// (its CTAs returned before writing).
 template <int G>
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const float* __restrict__ part, int nblk,
                                                           uint32_t part_stride, int np, int p_first,
                                                           const TrainSlot* __restrict__ slots,
-                                                          int drawn, uint32_t batch, float* __restrict__ grad,
-                                                          float* __restrict__ sums)
+                                                          float* __restrict__ grad, float* __restrict__ sums)
 {
     constexpr int E = 256 / G;
     __shared__ float gs[G][E];
     const int f = blockIdx.y, e = threadIdx.x % E, q = threadIdx.x / E;
     const int p = p_first + blockIdx.x * E + e;
-    const uint64_t n_rows = drawn ? (slots[f].n ? batch : 0) : slots[f].n;
     const float mine =
-        n_rows && p < np + 2 ? group_sum<G>(part + (size_t)f * nblk * part_stride + p, nblk, part_stride, q) : 0.f;
+        slots[f].n && p < np + 2 ? group_sum<G>(part + (size_t)f * nblk * part_stride + p, nblk, part_stride, q) : 0.f;
     const float a = block_groups_total<G>(gs, mine, q, e);
     if (q != 0 || p >= np + 2) return;
     if (p < np)
@@ -1750,7 +1887,11 @@ struct StopState {
     int bad;
 };
 
-__global__ void __launch_bounds__(256) early_stop_kernel(const float* __restrict__ sums,
+// a copy of 3 x 256's 19,248 parameters in five rounds of 16 bytes a thread: 6 us a
+// check (256 threads, a word each time: 15.2)
+constexpr int kStopThreads = 1024;
+
+__global__ void __launch_bounds__(kStopThreads) early_stop_kernel(const float* __restrict__ sums,
                                                          const TrainSlot* __restrict__ val, StopState* st,
                                                          TrainSlot* tr, const float* __restrict__ params,
                                                          float* __restrict__ best, int64_t n_params, int patience,
@@ -1777,9 +1918,13 @@ __global__ void __launch_bounds__(256) early_stop_kernel(const float* __restrict
         if (r == 0) flags[1] = *err;
     }
     __syncthreads();
-    if (keep)
-        for (int64_t i = threadIdx.x; i < n_params; i += blockDim.x)
-            best[(size_t)r * n_params + i] = params[(size_t)r * n_params + i];
+    if (keep) {
+        // n_params is a multiple of 16 (25 H + 16 a block), both arrays are allocations
+        const float4* from = reinterpret_cast<const float4*>(params + (size_t)r * n_params);
+        float4* to = reinterpret_cast<float4*>(best + (size_t)r * n_params);
+#pragma unroll 4
+        for (int64_t i = threadIdx.x; i < n_params / 4; i += kStopThreads) to[i] = from[i];
+    }
 }
 
 // Master parameter r of one block (W1 [H][8], b1 [H], W2 [16][H], b2 [16]),
@@ -1823,16 +1968,20 @@ __device__ __forceinline__ void publish_param(uint32_t* __restrict__ pb, int H, 
 // group_sum; each updated parameter is published at once (publish_param). A
 // block updates ROWS x 256 / G parameters of flow blockIdx.y (launched with
 // two rows: a launch of 16 flows fits one wave, and a one-flow launch leaves
-// room on the SMs for the next step's gradient CTAs, which start during it);
-// a flow without rows this step keeps its parameters, moments and published
+// room on the SMs for the next step's gradient CTAs, which start during it). 64
+// registers a thread (the partials in flight take 80 if let): 4 blocks an SM,
+// 46.0 us a step of 16 flows against 47.9, 16.3 against 16.7 of one.
+// A flow without rows this step keeps its parameters, moments and published
 // words. The step t is the gradient launch's ticket count over its CTA count
 // (grad_kernel): the counter stands at t grad_ctas after the gradient launch
 // of step t - 1, so no launch has to advance a step counter. Launched to
 // start during the gradient kernel, the kernel reads its partials and the
 // ticket only after that kernel has completed, and releases the next step's
-// gradient launch only once the whole block has read the ticket.
+// gradient launch as soon as the block has read the ticket: that launch's set-up
+// (about 2 us: slots, ticket, tensor memory, the first rows) overlaps the
+// partials' loads, which its own first use of the parameters waits for.
 template <int G, int ROWS>
-__global__ void __launch_bounds__(256) adam_publish_kernel(float* __restrict__ params, const float* __restrict__ part,
+__global__ void __launch_bounds__(256, 4) adam_publish_kernel(float* __restrict__ params, const float* __restrict__ part,
                                                            int nblk, uint32_t part_stride,
                                                            const TrainSlot* __restrict__ slots, float* __restrict__ m,
                                                            float* __restrict__ v, const unsigned* __restrict__ ticket,
@@ -1844,14 +1993,32 @@ __global__ void __launch_bounds__(256) adam_publish_kernel(float* __restrict__ p
     constexpr int E = 256 / G;
     __shared__ float gs[ROWS][G][E];
     __shared__ float w_s, c_s[2];
+    const int f = blockIdx.y, e = threadIdx.x % E, q = threadIdx.x / E;
+    const int64_t p0 = (int64_t)blockIdx.x * ROWS * E + e;
+    // The parameters and moments this thread updates. They are the previous
+    // step's Adam's, which the gradient kernel waited for before it let this
+    // launch start; the slots change between steps' launches alone.
+    const bool has_rows = __ldcg(&slots[f].n) != 0;   // uniform over the block
+    float pi[ROWS], mi[ROWS], vi[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const int64_t p = p0 + r * E, i = (int64_t)f * n_params + p;
+        const bool mine = has_rows && q == 0 && p < n_params;
+        pi[r] = mine ? __ldcg(params + i) : 0.f;
+        mi[r] = mine ? __ldcg(m + i) : 0.f;
+        vi[r] = mine ? __ldcg(v + i) : 0.f;
+    }
     // launched to start during the gradient kernel: its partials and ticket
     // are read only after it has completed
     griddep_wait();
-    const int f = blockIdx.y, e = threadIdx.x % E, q = threadIdx.x / E;
-    const int64_t p0 = (int64_t)blockIdx.x * ROWS * E + e;
-    const int t_step = (int)(*ticket / grad_ctas);
-    if (threadIdx.x == 32) adam_bias(t_step, b1, b2, c_s[0], c_s[1]);
-    const bool has_rows = slots[f].n != 0;   // uniform over the block
+    if (threadIdx.x == 32) {
+        // the block's one read of the ticket; the next step's gradient kernel
+        // may launch and take its tickets once every block has its value (the
+        // release depends on it: t_step is at least 1)
+        const int t_step = (int)(__ldcg(ticket) / grad_ctas);
+        if (t_step > 0) griddep_release();
+        adam_bias(t_step, b1, b2, c_s[0], c_s[1]);
+    }
     const float* base = part + (size_t)f * nblk * part_stride;
     if (threadIdx.x < 32) {
         // the weight sum: lane j adds CTAs j, j + 32, ... (all loads of a
@@ -1864,7 +2031,7 @@ __global__ void __launch_bounds__(256) adam_publish_kernel(float* __restrict__ p
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int c = c0 + 32 * k;
-                    x[k] = c < nblk ? base[(size_t)c * part_stride + n_params + 1] : 0.f;
+                    x[k] = c < nblk ? __ldcg(base + (size_t)c * part_stride + n_params + 1) : 0.f;
                 }
 #pragma unroll
                 for (int k = 0; k < 8; ++k) w += x[k];
@@ -1872,17 +2039,6 @@ __global__ void __launch_bounds__(256) adam_publish_kernel(float* __restrict__ p
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(kFull, w, off);
         if (threadIdx.x == 0) w_s = w;
-    }
-    // the parameters and moments this thread updates, loaded with the
-    // partials (one round trip for both)
-    float pi[ROWS], mi[ROWS], vi[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        const int64_t p = p0 + r * E, i = (int64_t)f * n_params + p;
-        const bool mine = has_rows && q == 0 && p < n_params;
-        pi[r] = mine ? params[i] : 0.f;
-        mi[r] = mine ? m[i] : 0.f;
-        vi[r] = mine ? v[i] : 0.f;
     }
     float g[ROWS];
     if constexpr (ROWS == 1) {
@@ -1896,9 +2052,6 @@ __global__ void __launch_bounds__(256) adam_publish_kernel(float* __restrict__ p
         g[1] = block_groups_total<G>(gs[1], mine1, q, e);
     }
     __syncthreads();
-    // the block has read the ticket (its bias corrections are in c_s): the
-    // next step's gradient kernel may launch and take its tickets
-    griddep_release();
     const float W = w_s;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
@@ -2247,12 +2400,11 @@ int red_groups(int nblk)
 }
 
 template <int G>
-void launch_reduce(abc_maf f, const maf::TrainSlot* slots, bool drawn, uint32_t batch, int nblk, uint32_t stride,
-                   bool sums_only, cudaStream_t s)
+void launch_reduce(abc_maf f, const maf::TrainSlot* slots, int nblk, int p_first, cudaStream_t s)
 {
-    const int np = (int)f->n_params, p_first = sums_only ? np : 0;
+    const int np = (int)f->n_params;
     maf::grad_reduce_kernel<G><<<dim3((np + 2 - p_first + 256 / G - 1) / (256 / G), f->R), 256, 0, s>>>(
-        f->d_part, nblk, stride, np, p_first, slots, drawn ? 1 : 0, batch, f->d_grad, f->d_sums);
+        f->d_part, nblk, part_stride(f), np, p_first, slots, f->d_grad, f->d_sums);
 }
 
 // a training run's ticket counter (grad_kernel), zeroed when the run starts
@@ -2274,7 +2426,7 @@ cudaError_t launch_adam_publish(abc_maf f, int nblk, float lr, cudaStream_t s)
 // in a fixed tree into d_grad and d_sums.
 template <int K, int W, bool PAIR>
 cudaError_t launch_grad_w(abc_maf f, const maf::TrainSlot* slots, unsigned* ticket, const ModelParams& rp,
-                          uint32_t batch, int grid, bool reduce, bool sums_only, cudaStream_t s)
+                          uint32_t batch, int grid, bool reduce, cudaStream_t s)
 {
     const size_t smem = grad_smem(f, W);
     cudaError_t e = allow_smem(maf::grad_kernel<K, W, PAIR>, smem);
@@ -2294,10 +2446,10 @@ cudaError_t launch_grad_w(abc_maf f, const maf::TrainSlot* slots, unsigned* tick
     e = cudaGetLastError();
     if (e != cudaSuccess || !reduce) return e;
     switch (red_groups(grid)) {
-    case 1: launch_reduce<1>(f, slots, ticket != nullptr, batch, grid, stride, sums_only, s); break;
-    case 2: launch_reduce<2>(f, slots, ticket != nullptr, batch, grid, stride, sums_only, s); break;
-    case 4: launch_reduce<4>(f, slots, ticket != nullptr, batch, grid, stride, sums_only, s); break;
-    default: launch_reduce<8>(f, slots, ticket != nullptr, batch, grid, stride, sums_only, s); break;
+    case 1: launch_reduce<1>(f, slots, grid, 0, s); break;
+    case 2: launch_reduce<2>(f, slots, grid, 0, s); break;
+    case 4: launch_reduce<4>(f, slots, grid, 0, s); break;
+    default: launch_reduce<8>(f, slots, grid, 0, s); break;
     }
     return cudaGetLastError();
 }
@@ -2306,14 +2458,14 @@ cudaError_t launch_grad_w(abc_maf f, const maf::TrainSlot* slots, unsigned* tick
 // them itself instead)
 template <int K>
 cudaError_t launch_grad(abc_maf f, const maf::TrainSlot* slots, unsigned* ticket, const ModelParams& rp, uint32_t batch,
-                        uint64_t max_n, bool reduce, bool sums_only, cudaStream_t s)
+                        uint64_t max_n, bool reduce, cudaStream_t s)
 {
     const uint64_t tiles = ((ticket ? batch : max_n) + 15) / 16;
     const GradForm g = grad_form(f, tiles);
     if (g.W == maf::kGradWarpsWide)
-        return launch_grad_w<K, maf::kGradWarpsWide, false>(f, slots, ticket, rp, batch, g.grid, reduce, sums_only, s);
-    if (g.pair) return launch_grad_w<K, maf::kGradWarpsNarrow, true>(f, slots, ticket, rp, batch, g.grid, reduce, sums_only, s);
-    return launch_grad_w<K, maf::kGradWarpsNarrow, false>(f, slots, ticket, rp, batch, g.grid, reduce, sums_only, s);
+        return launch_grad_w<K, maf::kGradWarpsWide, false>(f, slots, ticket, rp, batch, g.grid, reduce, s);
+    if (g.pair) return launch_grad_w<K, maf::kGradWarpsNarrow, true>(f, slots, ticket, rp, batch, g.grid, reduce, s);
+    return launch_grad_w<K, maf::kGradWarpsNarrow, false>(f, slots, ticket, rp, batch, g.grid, reduce, s);
 }
 
 #define MAF_DISPATCH(fn, ...)                      \
@@ -2339,16 +2491,36 @@ cudaError_t upload_slots(abc_maf f, const float* const* theta, const float* cons
 }
 
 // full-data gradients of the flows described by the slot table
-// full-data gradients (sums_only: the loss sums alone reduced, d_grad left as
-// it was)
-cudaError_t full_gradient(abc_maf f, uint64_t max_n, cudaStream_t s, const maf::TrainSlot* slots = nullptr,
-                          bool sums_only = false)
+// full-data gradients and loss sums of the uploaded slots, into d_grad and d_sums
+cudaError_t full_gradient(abc_maf f, uint64_t max_n, cudaStream_t s)
 {
     cudaError_t e = ensure_part(f, (max_n + 15) / 16);
-    if (e == cudaSuccess)
-        e = MAF_DISPATCH(launch_grad, f, slots ? slots : f->d_slots, nullptr, ModelParams{}, 0u, max_n, true, sums_only,
-                         s);
+    if (e == cudaSuccess) e = MAF_DISPATCH(launch_grad, f, f->d_slots, nullptr, ModelParams{}, 0u, max_n, true, s);
     return e;
+}
+
+// the loss sums alone of the given slots (max_n points at most) into d_sums; the
+// grid does not depend on the number of flows, so a flow's sums do not either
+template <int K>
+cudaError_t launch_loss(abc_maf f, const maf::TrainSlot* slots, uint64_t max_n, cudaStream_t s)
+{
+    const uint64_t tiles = (max_n + 15) / 16;
+    const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).fwd_words;
+    cudaError_t e = allow_smem(maf::loss_kernel<K>, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = grad_grid(tiles, maf::kFwdThreads / 32);
+    maf::loss_kernel<K><<<dim3(grid, f->R), maf::kFwdThreads, smem, s>>>(f->d_pub, f->H, f->box, slots, f->d_part,
+                                                                        part_stride(f));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    launch_reduce<8>(f, slots, grid, (int)f->n_params, s);
+    return cudaGetLastError();
+}
+
+cudaError_t full_loss(abc_maf f, const maf::TrainSlot* slots, uint64_t max_n, cudaStream_t s)
+{
+    // grad_grid's CTAs at 8 tiles each: never more than ensure_part allows for
+    cudaError_t e = ensure_part(f, (max_n + 15) / 16);
+    return e == cudaSuccess ? MAF_DISPATCH(launch_loss, f, slots, max_n, s) : e;
 }
 
 cudaError_t launch_adam(abc_maf f, float lr, float b1, float b2, float eps, cudaStream_t s)
@@ -2367,7 +2539,7 @@ cudaError_t launch_adam(abc_maf f, float lr, float b1, float b2, float eps, cuda
 // finishes and waits for it before touching its results.
 cudaError_t launch_train_step(abc_maf f, uint32_t batch, const ModelParams& p, float lr, cudaStream_t s)
 {
-    cudaError_t e = MAF_DISPATCH(launch_grad, f, f->d_slots, train_ticket(f), p, batch, 0, false, false, s);
+    cudaError_t e = MAF_DISPATCH(launch_grad, f, f->d_slots, train_ticket(f), p, batch, 0, false, s);
     if (e != cudaSuccess) return e;
     const int grid = grad_form(f, ((uint64_t)batch + 15) / 16).grid;
     switch (red_groups(grid)) {
@@ -2717,10 +2889,12 @@ abc_status abc_maf_train_flows(abc_maf f, const float* const* theta, const float
         int checks = 0;
         auto check = [&]() -> abc_status {
             const int slot = checks & 1;
-            MAF_TRY(full_gradient(f, max_va, s, f->d_slots_val, true), "validation loss");
+            MAF_TRY(full_loss(f, f->d_slots_val, max_va, s), "validation loss");
             MAF_TRY(cudaMemsetAsync(d_flags + 2 * slot, 0, 2 * sizeof(int), s), "cudaMemsetAsync(flags)");
-            maf::early_stop_kernel<<<R, 256, 0, s>>>(f->d_sums, f->d_slots_val, d_st, f->d_slots, f->d_params,
-                                                     f->d_best, f->n_params, kPatience, f->d_err, d_flags + 2 * slot);
+            maf::early_stop_kernel<<<R, maf::kStopThreads, 0, s>>>(f->d_sums, f->d_slots_val, d_st, f->d_slots,
+                                                                  f->d_params,
+                                                                  f->d_best, f->n_params, kPatience, f->d_err,
+                                                                  d_flags + 2 * slot);
             MAF_TRY(cudaGetLastError(), "early stopping launch");
             MAF_TRY(cudaMemcpyAsync(flags_h + 2 * slot, d_flags + 2 * slot, 2 * sizeof(int), cudaMemcpyDeviceToHost, s),
                     "cudaMemcpyAsync(flags)");
@@ -2769,7 +2943,7 @@ abc_status abc_maf_train_flows(abc_maf f, const float* const* theta, const float
         MAF_TRY(publish(f, s), "publish");
     }
     if (loss_out) {
-        MAF_TRY(full_gradient(f, max_n, s), "flow loss");
+        MAF_TRY(full_gradient(f, max_n, s), "flow loss");   // the flows' current gradient, too
         std::vector<float> sums(2 * (size_t)f->R);
         MAF_TRY(cudaMemcpyAsync(sums.data(), f->d_sums, sizeof(float) * sums.size(), cudaMemcpyDeviceToHost, s),
                 "cudaMemcpyAsync(sums)");

@@ -329,6 +329,31 @@ def test_training_fits_a_known_density():
     f.close()
 
 
+@pytest.mark.parametrize("K,H,n", [(1, 16, 20), (3, 256, 4001), (2, 112, 257), (4, 160, 30001)])
+def test_validation_loss_matches_oracle(K, H, n):
+    """A training run's validation loss (its own kernel: forward pass only) over
+    the held-out last points, ragged 16-row tiles and unequal flows, against the
+    oracle: lr is so small that the parameters stay what they were. The bound is
+    the gradient tests' on a loss."""
+    flows = [mo.init_params(np.random.default_rng(70 + r), K=K, H=H, scale=0.3) for r in range(2)]
+    v = np.concatenate([mo.flat(p).astype(np.float32) for p in flows])
+    f = abc.Flow(K, H, n_flows=2)
+    f.set_params(v)
+    ns = [n, max(20, n // 3)]
+    th = [_thetas(m, 5 + r) for r, m in enumerate(ns)]
+    w = [np.random.default_rng(9 + r).uniform(0.1, 2.0, m).astype(np.float32) for r, m in enumerate(ns)]
+    got = f.train_flows([torch.from_numpy(t).to(DEV) for t in th], [torch.from_numpy(a).to(DEV) for a in w], n_steps=50,
+                        batch=64, lr=1e-12, val_fraction=0.4)
+    for r, m in enumerate(ns):
+        k = min(int(np.floor(float(np.float32(0.4)) * m)), 8192)
+        t, a = th[r][m - k:].astype(np.float64), w[r][m - k:].astype(np.float64)
+        P = mo.unflat(mo.flat(flows[r]).astype(np.float32).astype(np.float64), K, H)
+        y = mo.to_y(t, LO, HI)
+        nll = -(mo.log_q_theta(t, P, LO, HI, bf16=True) + mo.log_jacobian_y(y, LO, HI))
+        want = (a * nll).sum() / a.sum()
+        assert abs(got[r] - want) < 2e-3 * abs(want) + 1e-3, (r, got[r], want)
+    f.close()
+
 def test_flow_set_members_equal_single_flows():
     """Flow r of a set evaluates and samples exactly like a one-flow object
     holding the same parameters (the same kernels on flow r's copy)."""
