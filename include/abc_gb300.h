@@ -190,8 +190,10 @@ abc_status abc_step(const float* theta, const int32_t* state_in, const uint64_t*
  * (DEVICE double [n], e.g. from abc_distances), returned in *eps_out (HOST).
  * Used to set eps to a distance quantile. +infinity is allowed; any NaN,
  * negative value or -0 returns ABC_ERR_INVALID_ARG (their bit patterns do not
- * order like values). Synchronizes cuda_stream. Uses device scratch (a
- * histogram) allocated stream-ordered and freed before returning. */
+ * order like values). Synchronizes cuda_stream. Uses device scratch, allocated
+ * stream-ordered and freed before returning: 45 KB of counters and at most
+ * 1 GiB (and 8 n bytes) for the distances near the k-th; where these are more or
+ * there is no memory for them, a slower selection needs the counters alone. */
 abc_status abc_kth_smallest(const double* dist, uint64_t n, uint64_t k, double* eps_out,
                             void* cuda_stream);
 
@@ -237,8 +239,8 @@ abc_status abc_select_below(const double* dist, const float* theta, uint64_t n, 
  *
  * Order of the outputs and capacity overflow (ABC_ERR_CAPACITY with the true
  * count in *n_accepted) as in abc_sample. Device scratch: every distance and
- * prior draw (40 bytes per sample, stream-ordered, freed before returning),
- * and the per-thread cached scratch of abc_sample for the series and counters.
+ * prior draw (40 bytes per sample, stream-ordered, freed before returning), that
+ * of abc_kth_smallest, and the per-thread cached scratch of abc_sample for the series and counters.
  * Synchronizes cuda_stream. */
 abc_status abc_sample_quantile(const abc_prior_box* prior, const int32_t* observed, int32_t T,
                                int64_t N_pop, uint64_t n_samples, uint64_t k, uint64_t seed,

@@ -105,8 +105,9 @@ __global__ void __launch_bounds__(BLOCK, LEAN ? 4 : is_fast(MODE) ? 1 : 768 / BL
     // Chunks are claimed one refill ahead (lane 0 holds the claim), so the
     // atomic's round trip overlaps the day pairs simulated before the next
     // refill; a claim made is always consumed by this warp. Measured: 16-region
-    // stream 58.2 -> 56.8 ms, config 3 2.317 -> 2.289 ms (the single-region
-    // kernel, whose samples run longer between refills, gains nothing).
+    // stream 58.2 -> 56.8 ms, three regions of 2^22 samples 2.317 -> 2.289 ms
+    // (the single-region kernel, whose samples run longer between refills,
+    // gains nothing).
     unsigned long long claim = 0;
     if (lane == 0) claim = atomicAdd(a.next, 1ull);
     // region of the warp's last claim: a warp's claims only grow and regions
