@@ -462,7 +462,9 @@ abc_status abc_maf_get_params(abc_maf maf, float* params);
  * float [n][8]; logq_out DEVICE float [n] (log q(theta)) or NULL. Async.
  * Sampling and density run in one of two kernel forms by n (both round the same
  * values to BF16, with FP32 sums in another order), so one index drawn in calls
- * of different n agrees to rounding, not always to the bit. */
+ * of different n agrees to rounding, not always to the bit. The form for many
+ * points waits for its tensor-core products, bounded as in abc_maf_gradient: one
+ * that runs out is reported by the next gradient, training or sequential run. */
 abc_status abc_maf_sample(abc_maf maf, uint64_t n, const float* base_draws, uint64_t seed, uint32_t stream,
                           uint64_t first_index, float* theta_out, float* logq_out, void* cuda_stream);
 abc_status abc_maf_sample_at(abc_maf maf, int32_t flow, uint64_t n, const float* base_draws, uint64_t seed,

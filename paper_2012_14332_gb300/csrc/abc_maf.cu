@@ -37,6 +37,7 @@
 #include "abc_tc.cuh"
 
 namespace abcgb {
+abc_status maf_take_error(abc_maf f);
 abc_status plan_fail(abc_status st, const char* msg);
 abc_status plan_cuda_fail(cudaError_t e, const char* what);
 abc_status plan_ok();
@@ -2142,7 +2143,7 @@ abc_status take_err(abc_maf f)
     MAF_TRY(cudaMemcpy(&h, f->d_err, sizeof h, cudaMemcpyDeviceToHost), "cudaMemcpy(error word)");
     if (h) {
         MAF_TRY(cudaMemset(f->d_err, 0, sizeof h), "cudaMemset(error word)");
-        return plan_fail(ABC_ERR_TIMEOUT, "a flow gradient kernel's wait for its tensor-core products ran out of time");
+        return plan_fail(ABC_ERR_TIMEOUT, "a flow kernel's wait for its operands or tensor-core products ran out of time");
     }
     return ABC_OK;
 }
@@ -2552,6 +2553,10 @@ cudaError_t launch_train_step(abc_maf f, uint32_t batch, const ModelParams& p, f
 }
 
 }  // namespace
+
+// a wait that ran out in a sampling or density launch since the last check, for
+// callers that have synchronised and run no training after it
+abc_status abcgb::maf_take_error(abc_maf f) { return take_err(f); }
 
 extern "C" {
 

@@ -18,6 +18,7 @@ namespace abcgb {
 abc_status plan_fail(abc_status st, const char* msg);
 abc_status plan_cuda_fail(cudaError_t e, const char* what);
 abc_status plan_ok();
+abc_status maf_take_error(abc_maf f);
 bool plan_check_prior(const abc_prior_box* prior, abc_status* st);
 ModelParams plan_make_params(const abc_prior_box* prior, int32_t T, int64_t N_pop, uint64_t seed, uint32_t stream,
                              const int32_t* ard0);
@@ -805,6 +806,7 @@ extern "C" abc_status abc_smc_run(const abc_prior_box* prior, const int32_t* obs
         eps *= cfg->eps_factor;
     }
     SMC_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    SMC_ST(abcgb::maf_take_error(gd.flow));
     *n_out = last_n;
     return abcgb::plan_ok();
 }
@@ -1144,5 +1146,6 @@ extern "C" abc_status abc_smc_run_regions(const abc_prior_box* prior, abc_smc_re
         }
     }
     SMC_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    SMC_ST(abcgb::maf_take_error(gd.flows));
     return abcgb::plan_ok();
 }
