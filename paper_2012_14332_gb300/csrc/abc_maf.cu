@@ -521,8 +521,8 @@ __device__ __forceinline__ void stage_blocks_bulk(uint32_t* sm, const uint32_t* 
 constexpr int kFwdThreads = 256;
 constexpr int kFwdMinBlocks = 4;
 // The sampler's longer passes run better at 3 CTAs per SM (80 registers,
-// 16 bytes spilled, against 64 and 32): 1.182 -> 1.157 ms per 0.9 x 2^22
-// proposals at 3 x 256.
+// 16 bytes spilled, against 64 and 32): 2 % at full load, which calls of this
+// size reach at their upper end.
 constexpr int kSampMinBlocks = 3;
 
 // words [off, off + n) of each of K published blocks, packed block after
@@ -2249,16 +2249,22 @@ int row_grid(int threads, size_t smem, uint64_t n)
 
 // Points from which the density and the sampler run in the tcgen05 form (us,
 // this form against the mma.sync one, blocks x hidden units):
+//              3 x 256           2 x 224           2 x 64
+//   sampler  80,000  27.8 / 25.7   19.5 / 16.5   18.4 / 17.6
+//           100,000  29.2 / 29.8   20.1 / 19.7   18.9 / 16.8
+//           150,000  29.5 / 42.0   20.9 / 25.9   19.3 / 21.3
+//           157,000  40.6 / 42.0   27.5 / 25.7   25.1 / 21.3
+//           200,000  42.0 / 50.2   29.2 / 29.8   27.3 / 24.0
+//           340,000  61.3 / 78.9   40.6 / 46.6   37.3 / 36.1
 //              3 x 256           4 x 176           2 x 64
-//   sampler  60,000  23.5 / 21.8   25.4 / 23.4   15.4 / 13.1
-//           100,000  29.2 / 29.9   29.8 / 31.5   18.0 / 15.8
-//           150,000  29.5 / 42.0   30.4 / 44.0   18.5 / 21.3
-//           300,000  51.0 / 71.0   54.3 / 72.7   29.8 / 34.3
 //   density 100,000  23.2 / 21.7   23.1 / 22.7   12.4 / 10.2
 //           200,000  35.2 / 34.7   35.4 / 35.6   15.2 / 15.1
 //           300,000  45.1 / 49.2   45.8 / 50.0   19.1 / 19.3
 //           500,000  68.5 / 76.6   70.4 / 78.4   27.1 / 29.4
-constexpr uint64_t kSampleRows = 100000, kLogqRows = 300000;
+// One 16-unit step a degree (up to 112 hidden units) leaves little work between
+// the sampler's waits. A second wave with less than a fifth of its rows costs as
+// much as a fuller one (one wave is 155,648 rows here).
+constexpr uint64_t kSampleRows = 100000, kSampleRowsThin = 400000, kLogqRows = 300000;
 
 template <int K>
 cudaError_t launch_logq(abc_maf f, int r, uint64_t n, const float* theta, float* logq, cudaStream_t s)
@@ -2287,17 +2293,22 @@ cudaError_t launch_sample_c(abc_maf f, int r, uint64_t n, const float* u, const 
                             uint64_t first, float* theta, float* logq, cudaStream_t s)
 {
     const float log_tau = logf(f->tau);
-    if (n < kSampleRows) {
-        const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).msamp_words;
-        cudaError_t e = allow_smem(maf::sample_few_kernel<K, CPD>, smem);
-        if (e != cudaSuccess) return e;
-        const int grid = fill_grid(maf::sample_few_kernel<K, CPD>, maf::kFwdThreads, smem, (n + 127) / 128);
-        maf::sample_few_kernel<K, CPD><<<grid, maf::kFwdThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n,
-                                                                            f->tau, log_tau, theta, logq);
-        return cudaGetLastError();
-    }
     constexpr int kThreads = maf::kSampGroups * maf::kRowGroup;
     const size_t smem = row_smem(f, maf::layout(f->H).samp_words, maf::kSampGroups);
+    bool few = n < (CPD == 1 ? kSampleRowsThin : kSampleRows);
+    if (!few) {
+        const uint64_t wave = (uint64_t)row_grid(kThreads, smem, 1ull << 40) * kThreads;
+        few = n > wave && n - wave < wave / 5;
+    }
+    if (few) {
+        const size_t smem_few = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).msamp_words;
+        cudaError_t e = allow_smem(maf::sample_few_kernel<K, CPD>, smem_few);
+        if (e != cudaSuccess) return e;
+        const int grid = fill_grid(maf::sample_few_kernel<K, CPD>, maf::kFwdThreads, smem_few, (n + 127) / 128);
+        maf::sample_few_kernel<K, CPD><<<grid, maf::kFwdThreads, smem_few, s>>>(
+            flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, log_tau, theta, logq);
+        return cudaGetLastError();
+    }
     cudaError_t e = allow_smem(maf::sample_kernel<K, CPD>, smem);
     if (e != cudaSuccess) return e;
     maf::sample_kernel<K, CPD><<<row_grid(kThreads, smem, n), kThreads, smem, s>>>(

@@ -94,7 +94,7 @@ def test_many_points_match_few_and_the_oracle(K, H, extra):
     where one falls on a bf16 boundary (2^-9 of an input): the median of every
     tile and the last rows' quantiles carry the bounds of the oracle tests."""
     f, params = _flow(K, H, 60 + K, 0.3)
-    n = 128 * 2400 + extra                  # above both forms' lines; a last wave that is not full
+    n = 128 * 3200 + extra                  # above every line; a last wave that is not full
     g = torch.Generator(device="cpu").manual_seed(K)
     u = torch.rand(n, 8, generator=g).clamp(1e-6, 1 - 1e-6)
     u = torch.log(u / (1 - u)).to(DEV)
@@ -129,6 +129,22 @@ def test_many_points_match_few_and_the_oracle(K, H, extra):
     errq = np.abs(lq[tail].cpu().numpy() - (lqy - mo.log_jacobian_y(y, LO, HI)))
     assert np.median(rel) < 1e-5 and np.quantile(rel, 0.95) < 1e-3
     assert np.median(errq) < 1e-4 and np.quantile(errq, 0.95) < 5e-3
+    f.close()
+
+
+@pytest.mark.parametrize("K,H,n", [(2, 112, 399_999), (2, 112, 400_000), (1, 128, 99_999), (1, 128, 100_000),
+                                   (1, 128, 155_648), (1, 128, 155_649), (3, 256, 186_777), (3, 256, 186_778)])
+def test_sampler_forms_agree_at_the_lines_between_them(K, H, n):
+    """Both sides of every line of the rule that chooses the sampler's form: the
+    first and the last rows against calls of a few thousand, as the test above."""
+    f, _ = _flow(K, H, 80 + K, 0.3)
+    width = torch.tensor(HI - LO, dtype=torch.float32, device=DEV)
+    th, lq = f.sample(n, seed=4, stream=1, first_index=10)
+    for first in (0, n - 3001):
+        t2, l2 = f.sample(3001, seed=4, stream=1, first_index=10 + first)
+        part = slice(first, first + 3001)
+        assert ((th[part] - t2).abs() / width).amax(1).median().item() < 1e-5
+        assert (lq[part] - l2).abs().median().item() < 1e-4
     f.close()
 
 def test_zero_flow_draws_the_prior_from_the_documented_words():
