@@ -244,15 +244,23 @@ __device__ __forceinline__ void reverse_cols(float (&v)[4])
     v[0] = n0; v[1] = n1; v[2] = n2; v[3] = n3;
 }
 
-// exp and the reciprocal of 1 + e as single SFU operations, results below 2^-126
-// flushed to 0 (__expf and __fdividef keep them, at about ten instructions
-// more for an alpha and its exponential).
-__device__ __forceinline__ float exp_sfu(float x) { return fast::ex2(1.44269504f * x); }
-
 // alpha = A tanh(ar / A) from one exponential: tanh|y| = (1 - e) / (1 + e) with
-// e = exp(-2 |y|) in (0, 1], so nothing overflows; the SFU operations leave an
-// absolute error of a few 1e-7 in alpha
+// e = exp(-2 |y|) in (0, 1], so nothing overflows; the fast exponential and
+// division leave an absolute error of a few 1e-7 in alpha. Training's form: a
+// step's rounding travels through every later one, and a run's parameters and
+// losses are those this arithmetic has always given.
 __device__ __forceinline__ float soft_alpha(float ar)
+{
+    const float e = __expf((-2.f / kAlphaMax) * fabsf(ar));
+    return copysignf(kAlphaMax * __fdividef(1.f - e, 1.f + e), ar);
+}
+
+// The density's and the sampler's exp and alpha: the exponential and the
+// reciprocal of 1 + e as single SFU operations, results below 2^-126 flushed to 0
+// (__expf and __fdividef keep them, at about ten instructions more for an alpha
+// and its exponential; neither occurs for |alpha| <= 6).
+__device__ __forceinline__ float exp_sfu(float x) { return fast::ex2(1.44269504f * x); }
+__device__ __forceinline__ float soft_alpha_sfu(float ar)
 {
     const float e = fast::ex2((-2.f * 1.44269504f / kAlphaMax) * fabsf(ar));
     return copysignf(kAlphaMax * ((1.f - e) * fast::rcp(1.f + e)), ar);
@@ -569,7 +577,7 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) logq_few_kernel(co
             made_fwd(view(sm + b * L.fwd_words, L), H, x, mu, ar);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float al = soft_alpha(ar[e]);
+                const float al = soft_alpha_sfu(ar[e]);
                 x[e] = (x[e] - mu[e]) * exp_sfu(-al);
                 ld[e] -= al;
             }
@@ -616,7 +624,7 @@ __device__ __forceinline__ void inverse_column(int t, const float (&z)[4], float
 {
     constexpr int e = D & 1;
     if (t == D / 2) {
-        const float al0 = soft_alpha(o1[e] + p1[e]), al1 = soft_alpha(o1[2 + e] + p1[2 + e]);
+        const float al0 = soft_alpha_sfu(o1[e] + p1[e]), al1 = soft_alpha_sfu(o1[2 + e] + p1[2 + e]);
         xin[e] = z[e] * exp_sfu(al0) + (o0[e] + p0[e]);
         xin[2 + e] = z[2 + e] * exp_sfu(al1) + (o0[2 + e] + p0[2 + e]);
         lq[e] -= al0;
@@ -700,7 +708,7 @@ __global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_few_kernel
             float p0[4] = {0.f, 0.f, 0.f, 0.f}, p1[4] = {0.f, 0.f, 0.f, 0.f};
             if (t == 0) {
                 // column 0 has degree 1: every weight into mu_0, alpha_0 is masked
-                const float al0 = soft_alpha(bs.x);
+                const float al0 = soft_alpha_sfu(bs.x);
                 xin[0] = z[0] * exp_sfu(al0) + bm.x;
                 xin[2] = z[2] * exp_sfu(al0) + bm.x;
                 lq[0] -= al0;
@@ -964,7 +972,7 @@ __global__ void __launch_bounds__(kDensGroups * kRowGroup, 2) logq_kernel(const 
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float2 bj = b2[j];
-                const float al = soft_alpha(__uint_as_float(o[2 * j + 1]) + bj.y);
+                const float al = soft_alpha_sfu(__uint_as_float(o[2 * j + 1]) + bj.y);
                 x[j] = (x[j] - (__uint_as_float(o[2 * j]) + bj.x)) * exp_sfu(-al);
                 sum_al += al;
             }
@@ -1040,7 +1048,7 @@ __global__ void __launch_bounds__(kSampGroups * kRowGroup, 2) sample_kernel(
             // column 0: every weight into mu_0, alpha_0 is masked
             {
                 const float2 bj = b2[0];
-                const float al = soft_alpha(bj.y);
+                const float al = soft_alpha_sfu(bj.y);
                 x[0] = x[0] * exp_sfu(al) + bj.x;
                 sum_al += al;
             }
@@ -1075,7 +1083,7 @@ __global__ void __launch_bounds__(kSampGroups * kRowGroup, 2) sample_kernel(
                 uint32_t o[2];
                 tc_ld2(g.lane_tmem + 48 + 2 * D, o);
                 const float2 bj = b2[D];
-                const float al = soft_alpha(__uint_as_float(o[1]) + bj.y);
+                const float al = soft_alpha_sfu(__uint_as_float(o[1]) + bj.y);
                 x[D] = x[D] * exp_sfu(al) + (__uint_as_float(o[0]) + bj.x);
                 sum_al += al;
             }
