@@ -1340,12 +1340,15 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
         first = tile_rows(tile0, lane >> 2, lane & 3, lane, n_rows, ticket != nullptr, rp, step_now, f, slot);
     griddep_wait();
     // block b's operands on a barrier of their own, so the first block's forward
-    // pass starts when they are in (warp 0 always has a tile: its forward pass
-    // waits for every block's copy before the CTA can end)
+    // pass starts when they are in. Warp 0's first tile waits for every copy, so
+    // none is in flight when the CTA ends; a CTA past this flow's last tile (the
+    // flow has fewer points than the largest) has no such tile and copies nothing.
+    if ((uint64_t)blockIdx.x * TPC < tiles) {
 #pragma unroll
-    for (int b = 0; b < K; ++b)
-        stage_blocks_bulk(wsm + b * L.grad_words, pub + (size_t)b * L.words, 1, L.w1, L.grad_words, L,
-                          smem_addr(&bar_stage[b]));
+        for (int b = 0; b < K; ++b)
+            stage_blocks_bulk(wsm + b * L.grad_words, pub + (size_t)b * L.words, 1, L.w1, L.grad_words, L,
+                              smem_addr(&bar_stage[b]));
+    }
     griddep_release();
     const uint32_t tmem = tmem_s;
     if (warp < W) {

@@ -435,6 +435,27 @@ def test_training_steps_publish_what_a_full_publish_writes(K, H, R):
     fs.close()
 
 
+@pytest.mark.parametrize("K,H,ns", [(4, 256, (4000, 20, 300)), (3, 112, (4000, 3000, 1)), (2, 64, (17, 30001, 16))])
+def test_a_flow_with_fewer_points_than_the_largest(K, H, ns):
+    """Flows of one set with very unequal data: CTAs past a small flow's last
+    tile have no rows (and copy no operands); the losses over all points and the
+    trained parameters are those of one-flow objects, up to the order in which
+    the CTAs' sums are added."""
+    singles = [_flow(K, H, 90 + r, 0.3)[0] for r in range(len(ns))]
+    fs = abc.Flow(K, H, n_flows=len(ns))
+    p0 = np.stack([f.get_params() for f in singles])
+    fs.set_params(p0)
+    data = [torch.from_numpy(_thetas(m, 60 + r)).to(DEV) for r, m in enumerate(ns)]
+    s = torch.cuda.Stream()
+    for _ in range(3):
+        got = fs.train_flows(data, None, n_steps=0, batch=64, cuda_stream=s)
+        for f, t, loss in zip(singles, data, got):
+            assert abs(loss - f.gradient(t)[0]) < 1e-5 * abs(loss)
+    assert np.array_equal(fs.get_params(), p0)
+    for f in singles + [fs]:
+        f.close()
+
+
 def test_train_flows_fits_each_flow_to_its_own_data():
     """One set trains three flows on three different densities (y = A l + m in
     y space, l iid standard logistic) in the same launches; each reaches its own
