@@ -1702,29 +1702,40 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
 }
 
 // The weighted loss sums alone over all points of every flow's slot (a training
-// run's validation checks), for grad_reduce_kernel: the gradient
-// kernel's forward pass, a warp per 16 rows and several CTAs an SM, each CTA's two
-// sums in its slot of the partials, its warps' in warp order: 9.5 us for 8000 points
-// at 3 x 256. The gradient kernel gives them too, at the price of the backward pass
-// (most of a step on 8192 rows, 23.6 us).
-template <int K>
-__global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) loss_kernel(const uint32_t* __restrict__ pub, int H,
-                                                                          const __grid_constant__ Box box,
-                                                                          const TrainSlot* __restrict__ slots,
-                                                                          float* __restrict__ part, uint32_t part_stride)
+// run's validation checks), for grad_reduce_kernel: the gradient kernel's forward
+// pass, its sums bit for bit. tpc warps of a CTA take the tiles that as many tile
+// workers of the gradient kernel's CTA take (the grid is that kernel's too), each
+// adding its tiles' sums in turn; the CTA's two sums, its workers' in their order,
+// go to its slot of the partials. PAIR: the outputs as the two warps of a pair
+// add them, the first eight chunks' and the others'. The other warps only help to
+// stage. The gradient kernel gives the sums too, at the price of the backward pass
+// (most of a step on 8192 rows, 23.7 us); a check on 8000 points and 25 steps of 1024
+// at 3 x 256 take 382 us (383 with eight tiles a CTA, whose sums differed in their
+// last bit).
+constexpr int kLossThreads = 512;   // holds the wide form's 15 tile workers
+static_assert(kGradWarpsWide <= kLossThreads / 32, "a warp a tile worker");
+
+template <int K, bool PAIR>
+__global__ void __launch_bounds__(kLossThreads) loss_kernel(const uint32_t* __restrict__ pub, int H,
+                                                            const __grid_constant__ Box box,
+                                                            const TrainSlot* __restrict__ slots, int tpc,
+                                                            float* __restrict__ part, uint32_t part_stride)
 {
     extern __shared__ __align__(16) uint32_t sm[];
-    constexpr int kWarps = kFwdThreads / 32;
-    __shared__ float sums_w[kWarps][2];
+    __shared__ float sums_w[kLossThreads / 32][2];
     const Layout L = layout(H);
     const int f = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const TrainSlot slot = slots[f];
-    if (slot.n == 0) return;   // uniform over the block
+    const uint64_t tiles = (slot.n + 15) / 16;
+    if (blockIdx.x * (uint64_t)tpc >= tiles) {   // uniform over the block
+        if (threadIdx.x < 2 && tiles)
+            part[((size_t)f * gridDim.x + blockIdx.x) * part_stride + (size_t)K * master_block(H) + threadIdx.x] = 0.f;
+        return;
+    }
     stage_blocks(sm, pub + (size_t)f * K * L.words, K, L.w1, L.fwd_words, L);
     __syncthreads();
-    const uint64_t tiles = (slot.n + 15) / 16;
-    float contrib = 0.f, wsum = 0.f;   // lanes t = 0: their rows'
-    for (uint64_t tile = (uint64_t)blockIdx.x * kWarps + warp; tile < tiles; tile += (uint64_t)gridDim.x * kWarps) {
+    float loss = 0.f, weight = 0.f;   // the worker's (lane 0)
+    for (uint64_t tile = (uint64_t)blockIdx.x * tpc + warp; warp < tpc && tile < tiles; tile += (uint64_t)gridDim.x * tpc) {
         const TileRows rows = tile_rows(tile, g, t, lane, slot.n, false, ModelParams{}, 0u, f, slot);
         float x[4], jac, ld0 = 0.f, ld1 = 0.f;
         to_y(box, 2 * t, rows.ta.x, x[0], jac);
@@ -1733,8 +1744,22 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) loss_kernel(const 
         to_y(box, 2 * t + 1, rows.tb.y, x[3], jac);
 #pragma unroll 1
         for (int b = 0; b < K; ++b) {
+            const BlockView v = view(sm + b * L.fwd_words, L);
             float mu[4], ar[4], al[4];
-            made_fwd(view(sm + b * L.fwd_words, L), H, x, mu, ar);
+            if constexpr (PAIR) {
+                float pm[4], pa[4], qm[4], qa[4];
+                made_part(v, 0, 8, x, pm, pa);
+                made_part(v, 8, H / 16, x, qm, qa);
+                const float2 bm = *reinterpret_cast<const float2*>(v.b2 + 2 * t);
+                const float2 bs = *reinterpret_cast<const float2*>(v.b2 + 8 + 2 * t);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    mu[e] = (pm[e] + qm[e]) + ((e & 1) ? bm.y : bm.x);
+                    ar[e] = (pa[e] + qa[e]) + ((e & 1) ? bs.y : bs.x);
+                }
+            } else {
+                made_fwd(v, H, x, mu, ar);
+            }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 al[e] = soft_alpha(ar[e]);
@@ -1746,24 +1771,24 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) loss_kernel(const 
         }
         const float n0 = quad_sum(ld0 - log_base(x[0]) - log_base(x[1]));
         const float n1 = quad_sum(ld1 - log_base(x[2]) - log_base(x[3]));
-        if (t == 0) {
-            contrib += rows.w0 * n0 + rows.w1 * n1;
-            wsum += rows.w0 + rows.w1;
-        }
-    }
+        float contrib = (t == 0) ? (rows.w0 * n0 + rows.w1 * n1) : 0.f;
+        float wsum = (t == 0) ? (rows.w0 + rows.w1) : 0.f;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        contrib += __shfl_xor_sync(kFull, contrib, off);
-        wsum += __shfl_xor_sync(kFull, wsum, off);
+        for (int off = 16; off > 0; off >>= 1) {
+            contrib += __shfl_xor_sync(kFull, contrib, off);
+            wsum += __shfl_xor_sync(kFull, wsum, off);
+        }
+        loss += contrib;
+        weight += wsum;
     }
     if (lane == 0) {
-        sums_w[warp][0] = contrib;
-        sums_w[warp][1] = wsum;
+        sums_w[warp][0] = loss;
+        sums_w[warp][1] = weight;
     }
     __syncthreads();
     if (threadIdx.x < 2) {
         float a = 0.f;
-        for (int w = 0; w < kWarps; ++w) a += sums_w[w][threadIdx.x];
+        for (int w = 0; w < tpc; ++w) a += sums_w[w][threadIdx.x];
         part[((size_t)f * gridDim.x + blockIdx.x) * part_stride + (size_t)K * master_block(H) + threadIdx.x] = a;
     }
 }
@@ -2430,6 +2455,18 @@ void launch_reduce(abc_maf f, const maf::TrainSlot* slots, int nblk, int p_first
         f->d_part, nblk, part_stride(f), np, p_first, slots, f->d_grad, f->d_sums);
 }
 
+// the reduction of `grid` CTAs' partials from entry p_first on
+cudaError_t launch_reduction(abc_maf f, const maf::TrainSlot* slots, int grid, int p_first, cudaStream_t s)
+{
+    switch (red_groups(grid)) {
+    case 1: launch_reduce<1>(f, slots, grid, p_first, s); break;
+    case 2: launch_reduce<2>(f, slots, grid, p_first, s); break;
+    case 4: launch_reduce<4>(f, slots, grid, p_first, s); break;
+    default: launch_reduce<8>(f, slots, grid, p_first, s); break;
+    }
+    return cudaGetLastError();
+}
+
 // a training run's ticket counter (grad_kernel), zeroed when the run starts
 unsigned* train_ticket(abc_maf f) { return reinterpret_cast<unsigned*>(f->d_step + 1); }
 
@@ -2468,13 +2505,7 @@ cudaError_t launch_grad_w(abc_maf f, const maf::TrainSlot* slots, unsigned* tick
     if (e != cudaSuccess) return e;
     e = cudaGetLastError();
     if (e != cudaSuccess || !reduce) return e;
-    switch (red_groups(grid)) {
-    case 1: launch_reduce<1>(f, slots, grid, 0, s); break;
-    case 2: launch_reduce<2>(f, slots, grid, 0, s); break;
-    case 4: launch_reduce<4>(f, slots, grid, 0, s); break;
-    default: launch_reduce<8>(f, slots, grid, 0, s); break;
-    }
-    return cudaGetLastError();
+    return launch_reduction(f, slots, grid, 0, s);
 }
 
 // reduce: add the partials into d_grad and d_sums (a training step's Adam adds
@@ -2522,26 +2553,32 @@ cudaError_t full_gradient(abc_maf f, uint64_t max_n, cudaStream_t s)
     return e;
 }
 
-// the loss sums alone of the given slots (max_n points at most) into d_sums; the
-// grid does not depend on the number of flows, so a flow's sums do not either
+// the loss sums alone of the given slots (max_n points at most) into d_sums: the
+// CTAs, their tile workers and the reduction of the full gradient's launch, so
+// the sums are that launch's
+template <int K, bool PAIR>
+cudaError_t launch_loss_p(abc_maf f, const maf::TrainSlot* slots, const GradForm& g, int nthreads, cudaStream_t s)
+{
+    const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).fwd_words;
+    cudaError_t e = allow_smem(maf::loss_kernel<K, PAIR>, smem);
+    if (e != cudaSuccess) return e;
+    maf::loss_kernel<K, PAIR><<<dim3(g.grid, f->R), nthreads, smem, s>>>(f->d_pub, f->H, f->box, slots, PAIR ? g.W / 2 : g.W,
+                                                                         f->d_part, part_stride(f));
+    return cudaGetLastError();
+}
+
 template <int K>
 cudaError_t launch_loss(abc_maf f, const maf::TrainSlot* slots, uint64_t max_n, cudaStream_t s)
 {
-    const uint64_t tiles = (max_n + 15) / 16;
-    const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).fwd_words;
-    cudaError_t e = allow_smem(maf::loss_kernel<K>, smem);
+    const GradForm g = grad_form(f, (max_n + 15) / 16);
+    const int nthreads = g.W == maf::kGradWarpsWide ? maf::kLossThreads : 256;
+    const cudaError_t e = g.pair ? launch_loss_p<K, true>(f, slots, g, nthreads, s) : launch_loss_p<K, false>(f, slots, g, nthreads, s);
     if (e != cudaSuccess) return e;
-    const int grid = grad_grid(tiles, maf::kFwdThreads / 32);
-    maf::loss_kernel<K><<<dim3(grid, f->R), maf::kFwdThreads, smem, s>>>(f->d_pub, f->H, f->box, slots, f->d_part,
-                                                                        part_stride(f));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    launch_reduce<8>(f, slots, grid, (int)f->n_params, s);
-    return cudaGetLastError();
+    return launch_reduction(f, slots, g.grid, (int)f->n_params, s);
 }
 
 cudaError_t full_loss(abc_maf f, const maf::TrainSlot* slots, uint64_t max_n, cudaStream_t s)
 {
-    // grad_grid's CTAs at 8 tiles each: never more than ensure_part allows for
     cudaError_t e = ensure_part(f, (max_n + 15) / 16);
     return e == cudaSuccess ? MAF_DISPATCH(launch_loss, f, slots, max_n, s) : e;
 }
