@@ -28,8 +28,8 @@ namespace {
 // The last block of each step to finish (a ticket, after a memory fence) takes
 // the step's decision, and up to kFinish candidates it finishes at once. The
 // answer is exact whatever the sample was: a rank outside the bracket, more
-// candidates than the buffer holds or a bin that stays too full leave
-// st->resolved at 0, and the caller runs the radix select.
+// candidates than the buffer holds, a bin that stays too full or counts that do
+// not add up leave st->resolved at 0, and the caller runs the radix select.
 //
 // HBM-bound: the pass is the one read of the distances. The radix select read
 // them eight times, its first digits (mostly the exponent, the same few values)
@@ -116,14 +116,19 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v)
 // The rank-th smallest (1-based) of c keys in shared memory, all in [lo, hi]:
 // the range is cut into up to 1024 equal bins and the bin that holds the rank
 // becomes the range, until a warp can rank the keys left in it or it is one
-// value. Called by the whole block; bins (1024) is shared scratch.
-__device__ uint64_t block_select(const uint64_t* keys, uint32_t c, uint64_t lo, uint64_t hi, uint64_t rank,
-                                 uint32_t* bins)
+// value (64 bits of range lose ten each time). False, and no key, unless each
+// range holds as many keys as counted for it and the rank among them: a caller
+// then leaves its search unresolved. Called by the whole block, with one answer;
+// bins (1024) is shared scratch.
+__device__ bool block_select(const uint64_t* keys, uint32_t c, uint64_t lo, uint64_t hi, uint64_t rank, uint32_t* bins,
+                             uint64_t* key_out)
 {
     __shared__ uint32_t pick_bin, pick_below, pick_count, n_short;
     __shared__ uint64_t short_list[32];
+    if (rank < 1 || rank > c || lo > hi) return false;
     uint32_t r = (uint32_t)rank, left = c;
-    while (left > 32) {
+    for (int cut = 0; left > 32; ++cut) {
+        if (cut == 7) return false;
         const uint64_t span = hi - lo;
         const int sh = span < 1024 ? 0 : 54 - __clzll((long long)span);   // span >> sh < 1024
         reinterpret_cast<uint4*>(bins)[threadIdx.x] = make_uint4(0, 0, 0, 0);
@@ -142,9 +147,13 @@ __device__ uint64_t block_select(const uint64_t* keys, uint32_t c, uint64_t lo, 
             pick_below = below;
             pick_count = h[q];
         }
-        __syncthreads();
+        // with every key of the range counted, r <= left lies in one thread's bins
+        if (!__syncthreads_and(threadIdx.x != kThreads - 1 || incl == left)) return false;
         lo += (uint64_t)pick_bin << sh;
-        if (sh == 0) return lo;
+        if (sh == 0) {
+            *key_out = lo;
+            return true;
+        }
         hi = lo + ((1ull << sh) - 1);
         r -= pick_below;
         left = pick_count;
@@ -153,8 +162,12 @@ __device__ uint64_t block_select(const uint64_t* keys, uint32_t c, uint64_t lo, 
     if (threadIdx.x == 0) n_short = 0;
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < c; i += kThreads)
-        if (keys[i] >= lo && keys[i] <= hi) short_list[atomicAdd(&n_short, 1u)] = keys[i];
+        if (keys[i] >= lo && keys[i] <= hi) {
+            const uint32_t at = atomicAdd(&n_short, 1u);
+            if (at < 32) short_list[at] = keys[i];
+        }
     __syncthreads();
+    if (n_short != left) return false;
     // every warp alike: lane's key, and how many of the others come before it
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t key = lane < left ? short_list[lane] : ~0ull;
@@ -164,7 +177,8 @@ __device__ uint64_t block_select(const uint64_t* keys, uint32_t c, uint64_t lo, 
         before += v < key || (v == key && j < lane);
     }
     const uint32_t at = __ballot_sync(0xFFFFFFFFu, lane < left && before + 1 == r);
-    return short_list[__ffs(at) - 1];
+    if (at) *key_out = short_list[__ffs(at) - 1];
+    return at != 0;
 }
 
 // Whether this block is the last of the grid to reach the ticket (its memory
@@ -282,7 +296,9 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const double* __restri
         if (below) atomicAdd(&st->below, below);
         if (bad) atomicAdd(&st->bad, bad);
     }
-    if (threadIdx.x == 0 && most) {
+    // a block with candidates has a least one, perhaps of key 0 (a distance of
+    // exactly 0), which is never ~0
+    if (threadIdx.x == 0 && least != ~0ull) {
         atomicMax(&st->not_least, ~least);
         atomicMax(&st->most, most);
     }
@@ -297,8 +313,9 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const double* __restri
     } else if (c <= cap && c <= kFinish) {
         for (uint32_t i = threadIdx.x; i < c; i += kThreads) buf[i] = __ldcg(&cand[i]);
         __syncthreads();
-        const uint64_t key = block_select(buf, (uint32_t)c, ~__ldcg(&st->not_least), __ldcg(&st->most), k - b, bins);
-        if (threadIdx.x == 0) {
+        uint64_t key;
+        if (block_select(buf, (uint32_t)c, ~__ldcg(&st->not_least), __ldcg(&st->most), k - b, bins, &key) &&
+            threadIdx.x == 0) {
             st->prefix = key;
             st->resolved = 1;
         }
@@ -323,8 +340,10 @@ __global__ void __launch_bounds__(kThreads) bin_kernel(SelectState* __restrict__
     const uint64_t c = __ldcg(&st->count);
     const int sh = span < kBins ? 0 : 53 - __clzll((long long)span);   // span >> sh < kBins
 #pragma unroll 4
-    for (uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x; i < c; i += (uint64_t)gridDim.x * kThreads)
-        atomicAdd(&h[(__ldcg(&cand[i]) - lo) >> sh], 1u);
+    for (uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x; i < c; i += (uint64_t)gridDim.x * kThreads) {
+        const uint64_t bin = (__ldcg(&cand[i]) - lo) >> sh;
+        if (bin < kBins) atomicAdd(&h[bin], 1u);
+    }
     __syncthreads();
     for (int b = threadIdx.x; b < kBins; b += kThreads)
         if (h[b]) atomicAdd(&bins[b], h[b]);
@@ -335,7 +354,10 @@ __global__ void __launch_bounds__(kThreads) bin_kernel(SelectState* __restrict__
         own[q] = __ldcg(&bins[threadIdx.x * (kBins / kThreads) + q]);
         sum += own[q];
     }
-    uint64_t before = block_scan(sum) - sum;
+    const uint32_t incl = block_scan(sum);
+    // a candidate outside [least, greatest] was not counted: unresolved
+    if (!__syncthreads_and(threadIdx.x != kThreads - 1 || incl == c)) return;
+    uint64_t before = incl - sum;
     const uint64_t rank = __ldcg(&st->rank);
     if (!(before < rank && rank <= before + sum)) return;
     int q = 0;
@@ -365,14 +387,18 @@ __global__ void __launch_bounds__(kThreads) finish_kernel(SelectState* __restric
 #pragma unroll 4
     for (uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x; i < c; i += (uint64_t)gridDim.x * kThreads) {
         const uint64_t key = __ldcg(&cand[i]);
-        if (key >= lo && key <= hi) few[atomicAdd(&st->n_few, 1u)] = key;
+        if (key >= lo && key <= hi) {
+            const uint32_t at = atomicAdd(&st->n_few, 1u);
+            if (at < kFinish) few[at] = key;
+        }
     }
     if (!last_block(&st->ticket[2])) return;
     const uint32_t m = __ldcg(&st->n_few);
+    if (m > kFinish) return;
     for (uint32_t i = threadIdx.x; i < m; i += kThreads) buf[i] = __ldcg(&few[i]);
     __syncthreads();
-    const uint64_t key = block_select(buf, m, lo, hi, __ldcg(&st->rank), bins);
-    if (threadIdx.x == 0) {
+    uint64_t key;
+    if (block_select(buf, m, lo, hi, __ldcg(&st->rank), bins, &key) && threadIdx.x == 0) {
         st->prefix = key;
         st->resolved = 1;
     }
@@ -551,7 +577,7 @@ __global__ void __launch_bounds__(kThreads) select_below_kernel(const __grid_con
     }
 }
 
-// blocks for n items at `per` a block, at most `waves` per SM of the device
+// blocks for n items at `per` a block, at most `per_sm` per SM of the device
 cudaError_t blocks_of(uint64_t n, uint64_t per, int per_sm, int* blocks)
 {
     int dev = 0, sms = 0;
@@ -573,7 +599,7 @@ cudaError_t launch_select_below(const SelectArgs& a, cudaStream_t s)
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Expected share of the keys inside the bracket of ranks [r_lo, r_hi].
+// The ranks [r_lo, r_hi] of the sample that the wanted key lies between.
 static void bracket(uint64_t n, uint64_t k, int32_t* r_lo, int32_t* r_hi)
 {
     const double q = ((double)k - 0.5) / (double)n, c = q * kPivotSample;

@@ -83,3 +83,45 @@ def test_invalid_keys_are_counted_wherever_they_lie(n, bad):
         with pytest.raises(abc.AbcError) as e:
             abc.abc_kth_smallest(torch.from_numpy(x).cuda(), n // 2)
         assert e.value.status == abc.binding.ABC_ERR_INVALID_ARG and "1 distances" in e.value.message
+
+
+def _zeros(kind, n):
+    """Distances of exactly 0 in tiles of their own (a tile is 2048 keys)."""
+    rest = 1.0 + np.random.default_rng(n).random(n)
+    if kind == "all":
+        return np.zeros(n)
+    if kind == "lone_last":
+        rest[n - 1] = 0.0
+        return rest
+    if kind == "rising_after_one":      # sorted input: one 0, then rising
+        return np.arange(n, dtype=np.float64)
+    lead = {"2048_first": 2048, "4096_first": 4096, "half_first": n // 2}[kind]
+    return np.concatenate([np.zeros(min(lead, n)), np.sort(rest[min(lead, n):])])
+
+
+@pytest.mark.parametrize("kind", ["all", "lone_last", "rising_after_one", "2048_first", "4096_first", "half_first"])
+@pytest.mark.parametrize("n", [2049, 3000, 4096, 4097, 6145, 65_536, 98_305, 2_000_000])
+def test_distances_of_exactly_zero_count_like_any_other(kind, n):
+    """A block whose only candidates are zeros, few candidates (finished by one
+    block) and many (binned first), ranks among the zeros, at their end and above."""
+    v = _zeros(kind, n)
+    s, dev = np.sort(v), torch.from_numpy(v).cuda()
+    zeros = int((v == 0).sum())
+    for k in sorted({1, 2, 14, 1000, 2000, 2300, zeros - 1, zeros, zeros + 1, n // 2, n - 1, n} & set(range(1, n + 1))):
+        assert abc.abc_kth_smallest(dev, k) == s[k - 1], (kind, n, k)
+
+
+@pytest.mark.parametrize("A0,T,n", [(0, 5, 3000), (0, 5, 70_000), (1, 1, 2049), (1, 2, 70_000), (2, 1, 200_000)])
+def test_quantile_of_runs_that_match_the_series_exactly(A0, T, n):
+    """A series without infections (every distance 0) and short ones of a few
+    cases, which many runs match exactly."""
+    obs = np.ascontiguousarray(np.tile([[A0], [0], [0]], (1, T + 1)).astype(np.int32))
+    d = abc.abc_distances(obs, 10**6, n, 3, mode="exact")
+    x = d.cpu().numpy()
+    zeros = int((x == 0).sum())
+    assert zeros > 0
+    for k in sorted({1, zeros, min(zeros + 1, n), n // 2, n}):
+        want = np.sort(x)[k - 1]
+        _, _, idx, m, eps = abc.abc_sample_quantile(obs, 10**6, n, k, 3, mode="exact", capacity=n)
+        assert eps == want and m == int((x <= want).sum())
+        assert np.array_equal(np.sort(idx.cpu().numpy()), np.flatnonzero(x <= want))
