@@ -388,8 +388,9 @@ abc_status abc_plan_destroy(abc_plan plan);
  *  - log q(theta) = log p(z) - sum alpha - sum_j log((hi_j - lo_j) s_j (1 - s_j)),
  *    s = sigmoid(y).
  * Weights live in FP32 (the master copy trained by Adam) and in masked BF16
- * copies used by tensor-core products (mma.sync m16n8k8 / m16n8k16 BF16 with
- * FP32 accumulation). Activations entering a product are rounded to BF16;
+ * copies used by tensor-core products (BF16 with FP32 accumulation: tcgen05 for
+ * density, sampling and the weight gradients, mma.sync for the gradient's passes
+ * over its rows). Activations entering a product are rounded to BF16;
  * everything else is FP32.
  *
  * Parameter order (host float arrays): for each block b = 0..n_blocks-1:
@@ -460,11 +461,11 @@ abc_status abc_maf_get_params(abc_maf maf, float* params);
  * 23 bits) gives the draw log(u / (1 - u))), the sequential
  * inverse of the flow, theta = lo + (hi - lo) sigmoid(y). theta_out DEVICE
  * float [n][8]; logq_out DEVICE float [n] (log q(theta)) or NULL. Async.
- * Sampling and density run in one of two kernel forms by n (both round the same
- * values to BF16, with FP32 sums in another order), so one index drawn in calls
- * of different n agrees to rounding, not always to the bit. The form for many
- * points waits for its tensor-core products, bounded as in abc_maf_gradient: one
- * that runs out is reported by the next gradient, training or sequential run. */
+ * A draw depends on (seed, stream, i), or on its base draws, and the flow's
+ * parameters alone: any split of the indices into calls gives the same bits.
+ * The kernel's waits for its tensor-core products are bounded as in
+ * abc_maf_gradient: one that runs out is reported by the next gradient, training
+ * or sequential run. */
 abc_status abc_maf_sample(abc_maf maf, uint64_t n, const float* base_draws, uint64_t seed, uint32_t stream,
                           uint64_t first_index, float* theta_out, float* logq_out, void* cuda_stream);
 abc_status abc_maf_sample_at(abc_maf maf, int32_t flow, uint64_t n, const float* base_draws, uint64_t seed,
@@ -472,7 +473,8 @@ abc_status abc_maf_sample_at(abc_maf maf, int32_t flow, uint64_t n, const float*
                              void* cuda_stream);
 
 /* log q(theta) for n points (DEVICE float [n][8] inside the box) into logq_out
- * (DEVICE float [n]). Async. */
+ * (DEVICE float [n]); a point's value does not depend on the others of its call.
+ * Async, with bounded waits as abc_maf_sample. */
 abc_status abc_maf_log_q(abc_maf maf, uint64_t n, const float* theta, float* logq_out, void* cuda_stream);
 abc_status abc_maf_log_q_at(abc_maf maf, int32_t flow, uint64_t n, const float* theta, float* logq_out,
                             void* cuda_stream);

@@ -1,11 +1,11 @@
 // abc_maf.cu -- masked autoregressive flow proposal for sequential ABC:
 // density, sampling (sequential inverse), weighted maximum-likelihood
 // gradient and Adam, with BF16 tensor-core products and FP32 accumulation:
-// density and sampling of many points on tcgen05.mma, a thread per row; of few
-// points, and the gradient's per-row passes, on mma.sync m16n8k8 and m16n8k16
-// per warp tile; the weight gradients on tcgen05.mma.
+// density and sampling on tcgen05.mma, a thread per row; the gradient's per-row
+// passes on mma.sync m16n8k8 and m16n8k16 per warp tile, its weight gradients on
+// tcgen05.mma.
 //
-// In the mma.sync form a warp owns 16 rows (samples). A row's eight coordinates sit in the
+// In the gradient a warp owns 16 rows (samples). A row's eight coordinates sit in the
 // accumulator layout of an m16n8 tile: lane (g = lane / 4, t = lane % 4) holds
 // columns 2t, 2t+1 of rows g and g+8. That is also the A-operand layout of an
 // m16n8k8 product, so a MADE block runs entirely in registers:
@@ -81,19 +81,15 @@ __host__ __device__ inline int master_block(int H) { return 25 * H + 16; }
 //   w2  [H/16][8][4][4]  B operands of h W2^T (k = hidden 16s + 2t, +1 and
 //                        16s + 8 + 2t, +1) for outputs g and 8 + g
 //   b1  [H/16][4][4]     FP32: b1 of hidden 16s + 2t, +1, 16s + 8 + 2t, +1
-//   b2  [16]             FP32 (w1 to b2 also serve the density of few points)
+//   b2  [16]             FP32 (w1 to b2 are all that a validation loss needs)
 //   w1t [8][H/2+4]       B operand of g_a1 W1     (n = j, k = l)
 //   w2t [H][8]           B operand of g_out W2    (n = l, k = o); rows l with
 //                        l & 4 hold their two 4-word halves swapped, so the
 //                        warp's fragment loads meet 32 distinct banks
-//
-// then the fragments of the sampler of few points (m1, m2, mb1, mb2 in the w1,
-// w2, b1, b2 layouts), over the same degree-grouped units as s1 and s2.
 struct Layout {
     int d1, d2, db2, dens_words;
     int s1, s2, sb2, samp_words;
-    int w1, w2, b1, b2, fwd_words, w1t, w2t, grad_words;
-    int m1, m2, mb1, mb2, msamp_words, words;
+    int w1, w2, b1, b2, fwd_words, w1t, w2t, grad_words, words;
 };
 
 // MADE masks (Germain et al.): hidden degree (l mod 7) + 1; input j and output
@@ -135,11 +131,6 @@ __host__ __device__ inline Layout layout(int H)
     L.w1t = o; o += 8 * (H / 2 + 4);
     L.w2t = o; o += H * 8;
     L.grad_words = o - L.w1;
-    L.m1 = o; o += C * 64;
-    L.m2 = o; o += C * 128;
-    L.mb1 = o; o += C * 16;
-    L.mb2 = o; o += 16;
-    L.msamp_words = o - L.m1;
     L.words = o;
     return L;
 }
@@ -479,24 +470,9 @@ __global__ void publish_kernel(const float* __restrict__ master, uint32_t* __res
         } else if (w < L.w2t) {
             const int r = w - L.w1t, j = r / hw, c = r % hw;
             if (c < H / 2) out = pack2(w1_of(2 * c, j), w1_of(2 * c + 1, j));
-        } else if (w < L.m1) {
+        } else {
             const int r = w - L.w2t, l = r / 8, o0 = 2 * ((r % 8) ^ (l & 4));
             out = pack2(w2_of(o0, l), w2_of(o0 + 1, l));
-        } else if (w < L.m2) {
-            // as w1, over the degree-grouped units
-            const int r = w - L.m1, h = r & 1, t = (r >> 1) & 3, g = (r >> 3) & 7, sc = r >> 6;
-            const int l = sampler_unit(H, sc, g + 8 * h);
-            out = pack2(w1_of(l, 2 * t), w1_of(l, 2 * t + 1));
-        } else if (w < L.mb1) {
-            const int r = w - L.m2, q = r & 3, t = (r >> 2) & 3, g = (r >> 4) & 7, sc = r >> 7;
-            const int o = g + 8 * (q >> 1), u = 8 * (q & 1) + 2 * t;
-            out = pack2(w2_of(o, sampler_unit(H, sc, u)), w2_of(o, sampler_unit(H, sc, u + 1)));
-        } else if (w < L.mb2) {
-            const int r = w - L.mb1, q = r & 3, t = (r >> 2) & 3, sc = r >> 4;
-            const int l = sampler_unit(H, sc, 8 * (q >> 1) + 2 * t + (q & 1));
-            out = __float_as_uint(l >= 0 ? b1[l] : 0.f);
-        } else {
-            out = __float_as_uint(b2[w - L.mb2]);
         }
         pub[(size_t)b * per + w] = out;
     }
@@ -517,223 +493,6 @@ __device__ __forceinline__ void stage_blocks_bulk(uint32_t* sm, const uint32_t* 
 }
 
 // ---------------------------------------------------------------------------
-// Density and sampling of few points: mma.sync, a warp per 16 rows. With few
-// rows an SM the time is the length of the chain, and a pass of the sampler
-// takes a warp about half as long as a group of 128 rows in the form below (two
-// commits a pass): 12.7 us for 3000 proposals at 4 x 176, 24.7 there; with expf
-// and divisions for its sigmoids and softplus this form took 18.9.
-// ---------------------------------------------------------------------------
-// Density and sampling CTAs: 8 warps share one staged copy of the forward
-// operands (about 41 KB at 3 x 256), at most 64 registers so that 4 CTAs
-// (32 warps) fit on an SM to hide the tensor-core chains' latency.
-constexpr int kFwdThreads = 256;
-constexpr int kFwdMinBlocks = 4;
-// The sampler's longer passes run better at 3 CTAs per SM (80 registers,
-// 16 bytes spilled, against 64 and 32): 2 % at full load, which calls of this
-// size reach at their upper end.
-constexpr int kSampMinBlocks = 3;
-
-// words [off, off + n) of each of K published blocks, packed block after
-// block in shared memory (stride n). Every offset and length is a multiple of
-// 4 words (H is a multiple of 16), so the copy moves 16-byte vectors.
-__device__ __forceinline__ void stage_blocks(uint32_t* sm, const uint32_t* pub, int K, int off, int n,
-                                             const Layout& L)
-{
-    const int n4 = n / 4;
-    for (int i = threadIdx.x; i < K * n4; i += blockDim.x) {
-        const int b = i / n4, r = i - b * n4;
-        reinterpret_cast<uint4*>(sm)[i] = reinterpret_cast<const uint4*>(pub + (size_t)b * L.words + off)[r];
-    }
-}
-
-template <int K>
-__global__ void __launch_bounds__(kFwdThreads, kFwdMinBlocks) logq_few_kernel(const uint32_t* __restrict__ pub, int H,
-                                                   const __grid_constant__ Box box,
-                                                   const float* __restrict__ theta, uint64_t n, float inv_tau,
-                                                   float log_tau, float* __restrict__ logq)
-{
-    extern __shared__ __align__(16) uint32_t sm[];
-    const Layout L = layout(H);
-    stage_blocks(sm, pub, K, L.w1, L.fwd_words, L);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const uint64_t tiles = (n + 15) / 16;
-    const int warps = blockDim.x / 32;
-    for (uint64_t tile = (uint64_t)blockIdx.x * warps + (threadIdx.x >> 5); tile < tiles;
-         tile += (uint64_t)gridDim.x * warps) {
-        const uint64_t r0 = tile * 16 + g, r1 = r0 + 8;
-        float x[4], jac[4];
-        const float mid[2] = {box.lo[2 * t] + 0.5f * box.w[2 * t], box.lo[2 * t + 1] + 0.5f * box.w[2 * t + 1]};
-        const float2 ta = r0 < n ? *reinterpret_cast<const float2*>(theta + 8 * r0 + 2 * t) : make_float2(mid[0], mid[1]);
-        const float2 tb = r1 < n ? *reinterpret_cast<const float2*>(theta + 8 * r1 + 2 * t) : make_float2(mid[0], mid[1]);
-        to_y(box, 2 * t, ta.x, x[0], jac[0]);
-        to_y(box, 2 * t + 1, ta.y, x[1], jac[1]);
-        to_y(box, 2 * t, tb.x, x[2], jac[2]);
-        to_y(box, 2 * t + 1, tb.y, x[3], jac[3]);
-        float ld[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int b = 0; b < K; ++b) {
-            float mu[4], ar[4];
-            made_fwd(view(sm + b * L.fwd_words, L), H, x, mu, ar);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float al = soft_alpha_sfu(ar[e]);
-                x[e] = (x[e] - mu[e]) * exp_sfu(-al);
-                ld[e] -= al;
-            }
-            reverse_cols(x);
-        }
-        const float q0 = quad_sum(log_base(x[0] * inv_tau) + log_base(x[1] * inv_tau) + ld[0] + ld[1] - jac[0] -
-                                  jac[1] - 2.f * log_tau);
-        const float q1 = quad_sum(log_base(x[2] * inv_tau) + log_base(x[3] * inv_tau) + ld[2] + ld[3] - jac[2] -
-                                  jac[3] - 2.f * log_tau);
-        if (t == 0) {
-            if (r0 < n) logq[r0] = q0;
-            if (r1 < n) logq[r1] = q1;
-        }
-    }
-}
-
-// One pass of the sequential inverse: the CPD chunks of degree-D hidden units
-// (chunks (D-1) CPD .. D CPD - 1 of the sampler's copy). Their inputs (columns
-// below D) are all final, so each unit's activation is computed once, and its
-// layer-2 contribution to every output is added to the running accumulators
-// (even chunks into o, odd into p). D and CPD are compile-time, so every
-// operand load is a fixed offset from the lane's base in the block's copy.
-template <int D, int CPD>
-__device__ __forceinline__ void inverse_pass(const BlockView& v, int g, int t, const float (&xin)[4], float (&o0)[4],
-                                             float (&o1)[4], float (&p0)[4], float (&p1)[4])
-{
-    const uint32_t a0 = pack2(xin[0], xin[1]), a1 = pack2(xin[2], xin[3]);
-#pragma unroll
-    for (int c = 0; c < CPD; ++c) {
-        const int s = (D - 1) * CPD + c;
-        if (s & 1)
-            made_chunk(v, s, g, t, a0, a1, p0, p1);
-        else
-            made_chunk(v, s, g, t, a0, a1, o0, o1);
-    }
-}
-
-// Column D of the block's inverse, once pass D has added every unit of degree
-// <= D: lane t = D / 2 holds it, element D % 2 for row g and 2 + D % 2 for row g + 8.
-template <int D>
-__device__ __forceinline__ void inverse_column(int t, const float (&z)[4], float (&xin)[4], float (&lq)[4],
-                                               const float (&o0)[4], const float (&o1)[4], const float (&p0)[4],
-                                               const float (&p1)[4])
-{
-    constexpr int e = D & 1;
-    if (t == D / 2) {
-        const float al0 = soft_alpha_sfu(o1[e] + p1[e]), al1 = soft_alpha_sfu(o1[2 + e] + p1[2 + e]);
-        xin[e] = z[e] * exp_sfu(al0) + (o0[e] + p0[e]);
-        xin[2 + e] = z[2 + e] * exp_sfu(al1) + (o0[2 + e] + p0[2 + e]);
-        lq[e] -= al0;
-        lq[2 + e] -= al1;
-    }
-}
-
-template <int D, int CPD>
-__device__ __forceinline__ void inverse_passes(const BlockView& v, int g, int t, const float (&z)[4], float (&xin)[4],
-                                               float (&lq)[4], float (&o0)[4], float (&o1)[4], float (&p0)[4],
-                                               float (&p1)[4])
-{
-    if constexpr (D <= 7) {
-        inverse_pass<D, CPD>(v, g, t, xin, o0, o1, p0, p1);
-        inverse_column<D>(t, z, xin, lq, o0, o1, p0, p1);
-        inverse_passes<D + 1, CPD>(v, g, t, z, xin, lq, o0, o1, p0, p1);
-    }
-}
-
-template <int K, int CPD>
-// box: read in place from the parameter space (indexing a by-value copy by
-// the lane's column put it in local memory)
-__global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_few_kernel(const uint32_t* __restrict__ pub, int H,
-                                                     const __grid_constant__ Box box,
-                                                     const float* __restrict__ u_in, const __grid_constant__ ModelParams p,
-                                                     uint32_t ctr3, uint64_t first, uint64_t n, float tau,
-                                                     float log_tau, float* __restrict__ theta_out,
-                                                     float* __restrict__ logq_out)
-{
-    extern __shared__ __align__(16) uint32_t sm[];
-    const Layout L = layout(H);
-    stage_blocks(sm, pub, K, L.m1, L.msamp_words, L);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const uint64_t tiles = (n + 15) / 16;
-    const int warps = blockDim.x / 32;
-    for (uint64_t tile = (uint64_t)blockIdx.x * warps + (threadIdx.x >> 5); tile < tiles;
-         tile += (uint64_t)gridDim.x * warps) {
-        const uint64_t r0 = tile * 16 + g, r1 = r0 + 8;
-        float x[4];
-        if (u_in) {
-            const float2 ua = r0 < n ? *reinterpret_cast<const float2*>(u_in + 8 * r0 + 2 * t) : make_float2(0.f, 0.f);
-            const float2 ub = r1 < n ? *reinterpret_cast<const float2*>(u_in + 8 * r1 + 2 * t) : make_float2(0.f, 0.f);
-            x[0] = ua.x; x[1] = ua.y; x[2] = ub.x; x[3] = ub.y;
-        } else {
-            // row r: Philox block (t / 2) of sample first + r; lane t takes words
-            // (x, y) for even t and (z, w) for odd t, one word per column
-            const uint4 wa = rng_block_s(p, first + r0, 0, ctr3, (uint32_t)(t >> 1));
-            const uint4 wb = rng_block_s(p, first + r1, 0, ctr3, (uint32_t)(t >> 1));
-            x[0] = logistic_draw((t & 1) ? wa.z : wa.x);
-            x[1] = logistic_draw((t & 1) ? wa.w : wa.y);
-            x[2] = logistic_draw((t & 1) ? wb.z : wb.x);
-            x[3] = logistic_draw((t & 1) ? wb.w : wb.y);
-        }
-        float lq[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            lq[e] = log_base(x[e]) - log_tau;
-            x[e] *= tau;
-        }
-        // blocks are a runtime loop (a fully unrolled 3 x 7 inverse overflows
-        // the instruction cache); a block's seven passes are unrolled, so
-        // every operand offset and register index is static. Column j
-        // depends on the hidden units of degree <= j alone, which passes
-        // 1..j have added to the accumulators by then.
-#pragma unroll 1
-        for (int bb = K - 1; bb >= 0; --bb) {
-            const uint32_t* base = sm + bb * L.msamp_words;
-            BlockView v;
-            v.w1 = base;
-            v.w2 = base + (L.m2 - L.m1);
-            v.b1 = reinterpret_cast<const float*>(base + (L.mb1 - L.m1));
-            v.b2 = reinterpret_cast<const float*>(base + (L.mb2 - L.m1));
-            v.w1t = v.w2t = nullptr;
-            float z[4] = {x[0], x[1], x[2], x[3]};
-            reverse_cols(z);
-            float xin[4] = {0.f, 0.f, 0.f, 0.f};
-            const float2 bm = *reinterpret_cast<const float2*>(v.b2 + 2 * t);
-            const float2 bs = *reinterpret_cast<const float2*>(v.b2 + 8 + 2 * t);
-            float o0[4] = {bm.x, bm.y, bm.x, bm.y}, o1[4] = {bs.x, bs.y, bs.x, bs.y};
-            float p0[4] = {0.f, 0.f, 0.f, 0.f}, p1[4] = {0.f, 0.f, 0.f, 0.f};
-            if (t == 0) {
-                // column 0 has degree 1: every weight into mu_0, alpha_0 is masked
-                const float al0 = soft_alpha_sfu(bs.x);
-                xin[0] = z[0] * exp_sfu(al0) + bm.x;
-                xin[2] = z[2] * exp_sfu(al0) + bm.x;
-                lq[0] -= al0;
-                lq[2] -= al0;
-            }
-            inverse_passes<1, CPD>(v, g, t, z, xin, lq, o0, o1, p0, p1);
-            x[0] = xin[0]; x[1] = xin[1]; x[2] = xin[2]; x[3] = xin[3];
-        }
-        float th[4], jac[4];
-        to_theta(box, 2 * t, x[0], th[0], jac[0]);
-        to_theta(box, 2 * t + 1, x[1], th[1], jac[1]);
-        to_theta(box, 2 * t, x[2], th[2], jac[2]);
-        to_theta(box, 2 * t + 1, x[3], th[3], jac[3]);
-        const float q0 = quad_sum(lq[0] + lq[1] - jac[0] - jac[1]);
-        const float q1 = quad_sum(lq[2] + lq[3] - jac[2] - jac[3]);
-        if (r0 < n) *reinterpret_cast<float2*>(theta_out + 8 * r0 + 2 * t) = make_float2(th[0], th[1]);
-        if (r1 < n) *reinterpret_cast<float2*>(theta_out + 8 * r1 + 2 * t) = make_float2(th[2], th[3]);
-        if (t == 0 && logq_out) {
-            if (r0 < n) logq_out[r0] = q0;
-            if (r1 < n) logq_out[r1] = q1;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Density and sampling on tcgen05: a thread per row.
 //
 // A group of 128 threads owns 128 rows, one a thread, and a tensor-memory
@@ -746,14 +505,21 @@ __global__ void __launch_bounds__(kFwdThreads, kSampMinBlocks) sample_few_kernel
 // the products (the box map, alpha, its exponential, the log-determinant) is
 // plain arithmetic on the thread's own row, no lane idle, no shuffle.
 //
-// In the mma.sync form above the products alone keep the legacy tensor path
-// busy for 405 of the sampler's 829 us per 0.9 x 2^22 proposals at 3 x 256 (8
-// cycles each, m16n8k8 as much as m16n8k16), a pass's elementwise work runs on
-// 8 of 32 lanes, and its fragments go through shared memory once per 16 rows.
-// This form: sampler 829 -> 535 us there, 188 -> 125 us for 10^6 at 3 x 128;
-// density 540 -> 484 us and (419,431 points) 69 -> 60 us. It is bound by issue
-// (60 % of the cycles issue) in the conversions and the tensor-memory reads of
-// the hidden units; a chain of 14 commits a block hides behind the other groups.
+// With mma.sync, a warp per 16 rows, the products alone kept the legacy tensor
+// path busy for 405 of the sampler's 829 us per 0.9 x 2^22 proposals at 3 x 256 (8
+// cycles each, m16n8k8 as much as m16n8k16), a pass's elementwise work ran on 8 of
+// 32 lanes, and the fragments went through shared memory once per 16 rows. This
+// form: sampler 829 -> 532 us there, 188 -> 124 us for 10^6 at 3 x 128; density
+// 540 -> 469 us and (400,000 points) 64 -> 56 us. It is bound by issue (60 % of the
+// cycles issue) in the conversions and the tensor-memory reads of the hidden
+// units; a chain of 14 commits a block hides behind the other groups.
+//
+// A call of a few thousand rows is bound by that chain instead, and a warp's
+// mma.sync chain is shorter (3000 proposals at 3 x 256: 14.3 us here, 8.2 there;
+// density 9.7 and 6.4). It is not used: the two kinds of product round their sums
+// differently, and an index drawn, or a point evaluated, in calls of different
+// size has one result. The arithmetic of a row here depends on nothing but the
+// row, whatever the number of groups in a CTA or of rows in the call.
 //
 // One thread of a group issues its products and commits them to the group's
 // mbarrier; the group's own named barrier orders its threads' shared and tensor
@@ -890,17 +656,17 @@ struct LogSum {
     __device__ __forceinline__ float plus(float v) const { return hi + (lo + v); }
 };
 
-// Density: two groups a CTA, two CTAs an SM. Hidden units go through in chunks
+// Density: a group a CTA, four CTAs an SM. Hidden units go through in chunks
 // of 64 (tensor-memory columns 0..63; their bf16 64..95; outputs 96..111): a
-// chunk's layer 2 and the next chunk's layer 1 are one commit. (Four groups of
-// 64 columns and chunks of 32: 1 % faster for 3.8e6 points, 10 % slower for
-// 419,431.)
+// chunk's layer 2 and the next chunk's layer 1 are one commit. (Two groups a CTA,
+// two CTAs an SM: 3000 points at 3 x 256 10.7 us instead of 9.7, 200,000 33.0
+// instead of 30.5, 3.8e6 482 instead of 469.)
 // The proposal may use a broadened base, z = tau * (standard logistic), with
 // density log p(z / tau) - log tau per coordinate (tau = 1: the trained flow).
-constexpr int kDensGroups = 2, kDensColumns = 128, kDensChunk = 64;
+constexpr int kDensGroups = 1, kDensColumns = 128, kDensChunk = 64, kDensPerSm = 4;
 
 template <int K>
-__global__ void __launch_bounds__(kDensGroups * kRowGroup, 2) logq_kernel(const uint32_t* __restrict__ pub, int H,
+__global__ void __launch_bounds__(kDensGroups * kRowGroup, kDensPerSm) logq_kernel(const uint32_t* __restrict__ pub, int H,
                                                                           const __grid_constant__ Box box,
                                                                           const float* __restrict__ theta, uint64_t n,
                                                                           float inv_tau, float log_tau,
@@ -994,24 +760,24 @@ __global__ void __launch_bounds__(kDensGroups * kRowGroup, 2) logq_kernel(const 
 // Sampling: the sequential inverse. Column j of a block depends on the hidden
 // units of degree <= j alone, and those on the inputs below j: pass D = 1..7
 // computes the CPD 16-unit steps of degree-D units (all their inputs final),
-// adds their layer-2 contribution to every output, and column D follows. Four
-// groups a CTA, two CTAs an SM; tensor-memory columns 0..47 hold a pass's
-// pre-activations, then (0..23) their bf16, 48..63 the outputs.
-constexpr int kSampGroups = 4, kSampColumns = 64;
+// adds their layer-2 contribution to every output, and column D follows.
+// Tensor-memory columns 0..47 hold a pass's pre-activations, then (0..23) their
+// bf16, 48..63 the outputs. A CTA has one, two or four groups (launch_sample_c).
+constexpr int kSampColumns = 64;
 
-template <int K, int CPD>
-__global__ void __launch_bounds__(kSampGroups * kRowGroup, 2) sample_kernel(
+template <int K, int CPD, int GROUPS>
+__global__ void __launch_bounds__(GROUPS * kRowGroup, GROUPS == 1 ? 4 : 8 / GROUPS) sample_kernel(
     const uint32_t* __restrict__ pub, int H, const __grid_constant__ Box box, const float* __restrict__ u_in,
     const __grid_constant__ ModelParams p, uint32_t ctr3, uint64_t first, uint64_t n, float tau, float log_tau,
     float* __restrict__ theta_out, float* __restrict__ logq_out, int* __restrict__ err)
 {
     extern __shared__ __align__(128) uint32_t row_sm[];
-    __shared__ __align__(8) uint64_t bar[kSampGroups], bar_stage;
+    __shared__ __align__(8) uint64_t bar[GROUPS], bar_stage;
     __shared__ uint32_t tmem_s;
     const Layout L = layout(H);
-    RowGroup g = row_setup<kSampGroups, kSampColumns>(row_sm, pub, K, L.s1, L.samp_words, L, err, bar, bar_stage, tmem_s);
+    RowGroup g = row_setup<GROUPS, kSampColumns>(row_sm, pub, K, L.s1, L.samp_words, L, err, bar, bar_stage, tmem_s);
     const uint64_t tiles = (n + kRowGroup - 1) / kRowGroup;
-    for (uint64_t tile = (uint64_t)blockIdx.x * kSampGroups + g.id; tile < tiles; tile += (uint64_t)gridDim.x * kSampGroups) {
+    for (uint64_t tile = (uint64_t)blockIdx.x * GROUPS + g.id; tile < tiles; tile += (uint64_t)gridDim.x * GROUPS) {
         const uint64_t r = tile * kRowGroup + g.row;
         LogSum lq;
         float x[8], sum_al = 0.f;
@@ -1102,7 +868,7 @@ __global__ void __launch_bounds__(kSampGroups * kRowGroup, 2) sample_kernel(
             if (logq_out) logq_out[r] = lq.plus(-sum_al - 8.f * log_tau);
         }
     }
-    row_teardown<kSampGroups, kSampColumns>(tmem_s);
+    row_teardown<GROUPS, kSampColumns>(tmem_s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1701,6 +1467,19 @@ __global__ void __launch_bounds__((W + 1) * 32, 1) grad_kernel(const uint32_t* _
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
+// words [off, off + n) of each of K published blocks, packed block after
+// block in shared memory (stride n). Every offset and length is a multiple of
+// 4 words (H is a multiple of 16), so the copy moves 16-byte vectors.
+__device__ __forceinline__ void stage_blocks(uint32_t* sm, const uint32_t* pub, int K, int off, int n,
+                                             const Layout& L)
+{
+    const int n4 = n / 4;
+    for (int i = threadIdx.x; i < K * n4; i += blockDim.x) {
+        const int b = i / n4, r = i - b * n4;
+        reinterpret_cast<uint4*>(sm)[i] = reinterpret_cast<const uint4*>(pub + (size_t)b * L.words + off)[r];
+    }
+}
+
 // The weighted loss sums alone over all points of every flow's slot (a training
 // run's validation checks), for grad_reduce_kernel: the gradient kernel's forward
 // pass, its sums bit for bit. tpc warps of a CTA take the tiles that as many tile
@@ -2228,18 +2007,6 @@ int sm_count()
     return sms > 0 ? sms : 1;
 }
 
-// blocks to launch: all that fit on the GPU at once, or fewer if the work is smaller
-template <typename Kern>
-int fill_grid(Kern k, int threads, size_t smem, uint64_t want)
-{
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    const uint64_t cap = (uint64_t)sm_count() * per_sm;
-    return (int)(want < cap ? (want > 0 ? want : 1) : cap);
-}
-
-
 // The kernel's dynamic shared-memory limit (one value per kernel and device)
 // is only ever raised, so flows of different sizes used from several host
 // threads never lower it under a launch that needs more.
@@ -2268,88 +2035,75 @@ cudaError_t publish(abc_maf f, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// CTAs of the density and sampling kernels: one for each CTA's worth of rows, at
-// most the two an SM's tensor memory holds (fewer where shared memory for two
-// is lacking). Not from the occupancy query: it says one CTA per SM for any
-// kernel that allocates tensor memory, and two run at once all the same.
-int row_grid(int threads, size_t smem, uint64_t n)
+// CTAs of a density or sampling kernel that an SM holds: at most `most` (what its
+// tensor memory holds), fewer where shared memory is lacking. Not from the
+// occupancy query: it says one CTA per SM for any kernel that allocates tensor
+// memory, and more run at once all the same.
+int row_ctas_per_sm(size_t smem, int most)
 {
     constexpr size_t kStaticAndReserved = 2 * 1024;   // a CTA's static shared memory and what the system takes
     int dev = 0, sm_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    const uint64_t per_sm = 2 * (smem + kStaticAndReserved) <= (size_t)sm_smem ? 2 : 1;
-    const uint64_t want = (n + threads - 1) / threads, cap = per_sm * (uint64_t)sm_count();
-    return (int)(want < cap ? want : cap);
+    const int fit = (int)((size_t)sm_smem / (smem + kStaticAndReserved));
+    return std::max(1, std::min(most, fit));
 }
 
-// Points from which the density and the sampler run in the tcgen05 form (us,
-// this form against the mma.sync one, blocks x hidden units):
-//              3 x 256           2 x 224           2 x 64
-//   sampler  80,000  27.8 / 25.7   19.5 / 16.5   18.4 / 17.6
-//           100,000  29.2 / 29.8   20.1 / 19.7   18.9 / 16.8
-//           150,000  29.5 / 42.0   20.9 / 25.9   19.3 / 21.3
-//           157,000  40.6 / 42.0   27.5 / 25.7   25.1 / 21.3
-//           200,000  42.0 / 50.2   29.2 / 29.8   27.3 / 24.0
-//           340,000  61.3 / 78.9   40.6 / 46.6   37.3 / 36.1
-//              3 x 256           4 x 176           2 x 64
-//   density 100,000  23.2 / 21.7   23.1 / 22.7   12.4 / 10.2
-//           200,000  35.2 / 34.7   35.4 / 35.6   15.2 / 15.1
-//           300,000  45.1 / 49.2   45.8 / 50.0   19.1 / 19.3
-//           500,000  68.5 / 76.6   70.4 / 78.4   27.1 / 29.4
-// One 16-unit step a degree (up to 112 hidden units) leaves little work between
-// the sampler's waits. A second wave with less than a fifth of its rows costs as
-// much as a fuller one (one wave is 155,648 rows here).
-constexpr uint64_t kSampleRows = 100000, kSampleRowsThin = 400000, kLogqRows = 300000;
+// one CTA for each CTA's worth of 128-row tiles, at most what the SMs hold
+int row_grid(uint64_t tiles, int groups, size_t smem, int most)
+{
+    const uint64_t cap = (uint64_t)row_ctas_per_sm(smem, most) * (uint64_t)sm_count();
+    return (int)std::min((tiles + groups - 1) / groups, cap);
+}
+
+uint64_t row_tiles(uint64_t n) { return n / maf::kRowGroup + (n % maf::kRowGroup != 0); }
 
 template <int K>
 cudaError_t launch_logq(abc_maf f, int r, uint64_t n, const float* theta, float* logq, cudaStream_t s)
 {
-    const float inv_tau = 1.f / f->tau, log_tau = logf(f->tau);
-    if (n < kLogqRows) {
-        const size_t smem = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).fwd_words;
-        cudaError_t e = allow_smem(maf::logq_few_kernel<K>, smem);
-        if (e != cudaSuccess) return e;
-        const int grid = fill_grid(maf::logq_few_kernel<K>, maf::kFwdThreads, smem, (n + 127) / 128);
-        maf::logq_few_kernel<K><<<grid, maf::kFwdThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n, inv_tau, log_tau,
-                                                                     logq);
-        return cudaGetLastError();
-    }
-    constexpr int kThreads = maf::kDensGroups * maf::kRowGroup;
     const size_t smem = row_smem(f, maf::layout(f->H).dens_words, maf::kDensGroups);
     cudaError_t e = allow_smem(maf::logq_kernel<K>, smem);
     if (e != cudaSuccess) return e;
-    maf::logq_kernel<K><<<row_grid(kThreads, smem, n), kThreads, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n, inv_tau,
-                                                                           log_tau, logq, f->d_err);
+    const int grid = row_grid(row_tiles(n), maf::kDensGroups, smem, maf::kDensPerSm);
+    maf::logq_kernel<K><<<grid, maf::kDensGroups * maf::kRowGroup, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n,
+                                                                              1.f / f->tau, logf(f->tau), logq, f->d_err);
     return cudaGetLastError();
 }
 
+template <int K, int CPD, int GROUPS>
+cudaError_t launch_sample_g(abc_maf f, int r, uint64_t n, const float* u, const ModelParams& p, uint32_t ctr3,
+                            uint64_t first, float* theta, float* logq, cudaStream_t s)
+{
+    const size_t smem = row_smem(f, maf::layout(f->H).samp_words, GROUPS);
+    cudaError_t e = allow_smem(maf::sample_kernel<K, CPD, GROUPS>, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = row_grid(row_tiles(n), GROUPS, smem, 8 / GROUPS);
+    maf::sample_kernel<K, CPD, GROUPS><<<grid, GROUPS * maf::kRowGroup, smem, s>>>(
+        flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, logf(f->tau), theta, logq, f->d_err);
+    return cudaGetLastError();
+}
+
+// Groups in a CTA (the same results). While every SM has at most two tiles of 128
+// rows, a group a CTA: groups of one CTA are on one SM, where they slow each
+// other's chains. Then two while a wave of three such CTAs an SM (fewer if shared
+// memory is lacking) holds all tiles, else four, eight groups an SM. us with one,
+// two and four groups:
+//              3 x 256             4 x 176             2 x 64
+//     3,000  14.3  15.8  19.2    16.2  17.8  21.9    8.8   9.6  11.9
+//    30,000  15.4  16.2  20.6    17.0  18.0  23.1    9.7  10.0  12.7
+//    60,000  27.9  18.9  20.8    31.4  20.6  23.3   11.6  12.0  12.8
+//   100,000  30.9  23.0  26.5    34.1  24.3  28.4   18.7  13.9  16.1
+//   150,000  43.2  33.6  26.9    47.9  37.3  28.7   21.0  16.4  16.5
+// 1,000,000   243   162   144     274   177   156    110  79.7  80.2
 template <int K, int CPD>
 cudaError_t launch_sample_c(abc_maf f, int r, uint64_t n, const float* u, const ModelParams& p, uint32_t ctr3,
                             uint64_t first, float* theta, float* logq, cudaStream_t s)
 {
-    const float log_tau = logf(f->tau);
-    constexpr int kThreads = maf::kSampGroups * maf::kRowGroup;
-    const size_t smem = row_smem(f, maf::layout(f->H).samp_words, maf::kSampGroups);
-    bool few = n < (CPD == 1 ? kSampleRowsThin : kSampleRows);
-    if (!few) {
-        const uint64_t wave = (uint64_t)row_grid(kThreads, smem, 1ull << 40) * kThreads;
-        few = n > wave && n - wave < wave / 5;
-    }
-    if (few) {
-        const size_t smem_few = sizeof(uint32_t) * (size_t)K * maf::layout(f->H).msamp_words;
-        cudaError_t e = allow_smem(maf::sample_few_kernel<K, CPD>, smem_few);
-        if (e != cudaSuccess) return e;
-        const int grid = fill_grid(maf::sample_few_kernel<K, CPD>, maf::kFwdThreads, smem_few, (n + 127) / 128);
-        maf::sample_few_kernel<K, CPD><<<grid, maf::kFwdThreads, smem_few, s>>>(
-            flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, log_tau, theta, logq);
-        return cudaGetLastError();
-    }
-    cudaError_t e = allow_smem(maf::sample_kernel<K, CPD>, smem);
-    if (e != cudaSuccess) return e;
-    maf::sample_kernel<K, CPD><<<row_grid(kThreads, smem, n), kThreads, smem, s>>>(
-        flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, log_tau, theta, logq, f->d_err);
-    return cudaGetLastError();
+    const uint64_t tiles = row_tiles(n), sms = (uint64_t)sm_count();
+    if (tiles <= 2 * sms) return launch_sample_g<K, CPD, 1>(f, r, n, u, p, ctr3, first, theta, logq, s);
+    if (tiles <= 2 * sms * row_ctas_per_sm(row_smem(f, maf::layout(f->H).samp_words, 2), 3))
+        return launch_sample_g<K, CPD, 2>(f, r, n, u, p, ctr3, first, theta, logq, s);
+    return launch_sample_g<K, CPD, 4>(f, r, n, u, p, ctr3, first, theta, logq, s);
 }
 
 template <int K>

@@ -87,41 +87,28 @@ def test_sample_matches_oracle_inverse(K, H):
 # last one of 16, 32, 48 or 64; a last tile of 1, 31, 127 and 128 rows
 @pytest.mark.parametrize("K,H,extra", [(1, 16, 1), (2, 64, 31), (2, 112, 128), (3, 208, 127), (4, 256, 0), (3, 160, 129)])
 def test_many_points_match_few_and_the_oracle(K, H, extra):
-    """From a number of points on, sampling and density run in another form
-    (tcgen05, a thread per row). It is held against the form for few points, row
-    by row in tiles of 128, and against the oracle on the last rows. Both forms
-    round the same values to bf16, so a row differs by a few float32 steps but
-    where one falls on a bf16 boundary (2^-9 of an input): the median of every
-    tile and the last rows' quantiles carry the bounds of the oracle tests."""
+    """A row of a call of many points (four groups of 128 rows a CTA) is the row
+    of calls of fewer (one or two groups), bit for bit, and the last rows are the
+    oracle's: the median and the quantiles carry the bounds of the oracle tests."""
     f, params = _flow(K, H, 60 + K, 0.3)
-    n = 128 * 3200 + extra                  # above every line; a last wave that is not full
+    n = 128 * 3200 + extra                  # several waves, the last one not full
     g = torch.Generator(device="cpu").manual_seed(K)
     u = torch.rand(n, 8, generator=g).clamp(1e-6, 1 - 1e-6)
     u = torch.log(u / (1 - u)).to(DEV)
     pad = torch.empty(8 * n + 2, device=DEV)
     base = pad[2:].view(n, 8)               # 8-byte aligned rows
     base.copy_(u)
-    few = 128 * 640
-
-    def parts(fn):
-        return [torch.cat(c) for c in zip(*(fn(slice(i, min(i + few, n))) for i in range(0, n, few)))]
-
-    def per_tile(err):
-        err = err.flatten(1).amax(1) if err.dim() > 1 else err
-        m = n // 128 * 128
-        return err[:m].view(-1, 128).median(1).values.max().item()
-
-    width = torch.tensor(HI - LO, dtype=torch.float32, device=DEV)
     th, lq = f.sample(n, base=base)
-    th2, lq2 = parts(lambda i: f.sample(i.stop - i.start, base=u[i]))
     d = f.log_q(th)
-    d2, = parts(lambda i: (f.log_q(th[i]),))
-    e_th, e_lq, e_d = per_tile((th - th2).abs() / width), per_tile((lq - lq2).abs()), per_tile((d - d2).abs())
-    print("many points K=%d H=%d: largest tile median theta %.1e logq %.1e density %.1e" % (K, H, e_th, e_lq, e_d))
-    assert e_th < 1e-5 and e_lq < 1e-4 and e_d < 1e-4
+    for few in (128 * 100, 128 * 640):      # one group a CTA, two
+        for i in range(0, n, few):
+            part = slice(i, min(i + few, n))
+            t2, l2 = f.sample(part.stop - i, base=u[part])
+            assert torch.equal(t2, th[part]) and torch.equal(l2, lq[part])
+            assert torch.equal(f.log_q(th[part]), d[part])
     s1, l1 = f.sample(n, seed=3, stream=2, first_index=(1 << 32) - 7)
-    s2, _ = f.sample(few - 5, seed=3, stream=2, first_index=(1 << 32) - 2)
-    assert ((s1[5:few] - s2).abs() / width).flatten(1).amax(1).median().item() < 1e-5
+    s2, l2 = f.sample(128 * 640 - 5, seed=3, stream=2, first_index=(1 << 32) - 2)
+    assert torch.equal(s1[5:128 * 640], s2) and torch.equal(l1[5:128 * 640], l2)
     tail = slice(n - 200, n)
     y, lqy = mo.inverse(u[tail].cpu().numpy().astype(np.float64), params, bf16=True)
     ref = mo.to_theta(y, LO, HI)
@@ -135,17 +122,36 @@ def test_many_points_match_few_and_the_oracle(K, H, extra):
 @pytest.mark.parametrize("K,H,n", [(2, 112, 399_999), (2, 112, 400_000), (1, 128, 99_999), (1, 128, 100_000),
                                    (1, 128, 155_648), (1, 128, 155_649), (3, 256, 186_777), (3, 256, 186_778)])
 def test_sampler_forms_agree_at_the_lines_between_them(K, H, n):
-    """Both sides of every line of the rule that chooses the sampler's form: the
-    first and the last rows against calls of a few thousand, as the test above."""
+    """Sizes around waves of every shape of CTA: the first and the last rows are
+    those of calls of a few thousand, bit for bit."""
     f, _ = _flow(K, H, 80 + K, 0.3)
-    width = torch.tensor(HI - LO, dtype=torch.float32, device=DEV)
     th, lq = f.sample(n, seed=4, stream=1, first_index=10)
     for first in (0, n - 3001):
         t2, l2 = f.sample(3001, seed=4, stream=1, first_index=10 + first)
         part = slice(first, first + 3001)
-        assert ((th[part] - t2).abs() / width).amax(1).median().item() < 1e-5
-        assert (lq[part] - l2).abs().median().item() < 1e-4
+        assert torch.equal(th[part], t2) and torch.equal(lq[part], l2)
     f.close()
+
+
+@pytest.mark.parametrize("K,H", [(2, 112), (1, 128), (3, 256), (4, 256)])
+@pytest.mark.parametrize("tiles,extra", [(0, 1), (1, 0), (1, 1), (304, 0), (304, 1), (608, 0), (608, 1), (912, 0), (912, 1),
+                                         (1216, 0), (1216, 1)])
+def test_one_index_has_one_result_in_calls_of_any_size(K, H, tiles, extra):
+    """Both sides of every line of the rule that chooses a sampling CTA's groups
+    (on 152 SMs): the first and the last rows and their densities are those of
+    calls of a few hundred and a few thousand, bit for bit."""
+    f, _ = _flow(K, H, 80 + K, 0.3)
+    n = 128 * tiles + extra
+    th, lq = f.sample(n, seed=4, stream=1, first_index=10)
+    d = f.log_q(th)
+    for m in (min(n, 300), min(n, 3001)):
+        for first in (0, n - m):
+            part = slice(first, first + m)
+            t2, l2 = f.sample(m, seed=4, stream=1, first_index=10 + first)
+            assert torch.equal(th[part], t2) and torch.equal(lq[part], l2)
+            assert torch.equal(d[part], f.log_q(t2))
+    f.close()
+
 
 def test_zero_flow_draws_the_prior_from_the_documented_words():
     """A flow with zero parameters is the uniform prior: base coordinate c of
