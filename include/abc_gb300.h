@@ -431,13 +431,13 @@ int32_t abc_maf_flow_count(abc_maf maf);
  * bulk; a base broader than the fitted one keeps covering them. */
 abc_status abc_maf_set_proposal_scale(abc_maf maf, float tau);
 
-/* Testing hook for the gradient kernel's bounded waits. With hold != 0 the
- * thread that issues the kernel's tensor-core products issues none, so the
- * kernel's final wait for them runs out (after 2 s): abc_maf_gradient and the
- * training calls then return ABC_ERR_TIMEOUT and leave the flow's gradient
- * unspecified. hold = 0 (the default) restores normal operation; the CUDA
- * context stays usable throughout. Applies to launches after the call (a
- * captured training step is rebuilt). */
+/* Testing hook for the flow kernels' bounded waits. With hold != 0 the threads
+ * that issue the kernels' tensor-core products issue none, so the waits for them
+ * run out (after 2 s): abc_maf_gradient and the training calls then return
+ * ABC_ERR_TIMEOUT and leave the flow's gradient unspecified, sampling and density
+ * write NaN and abc_maf_check returns ABC_ERR_TIMEOUT. hold = 0 (the default)
+ * restores normal operation; the CUDA context stays usable throughout. Applies to
+ * launches after the call (a captured training step is rebuilt). */
 abc_status abc_maf_test_hold_products(abc_maf maf, int32_t hold);
 
 /* Random initial parameters: W1 ~ N(0, scale^2 / 8), W2 ~ N(0, scale^2 / hidden),
@@ -463,9 +463,8 @@ abc_status abc_maf_get_params(abc_maf maf, float* params);
  * float [n][8]; logq_out DEVICE float [n] (log q(theta)) or NULL. Async.
  * A draw depends on (seed, stream, i), or on its base draws, and the flow's
  * parameters alone: any split of the indices into calls gives the same bits.
- * The kernel's waits for its tensor-core products are bounded as in
- * abc_maf_gradient: one that runs out is reported by the next gradient, training
- * or sequential run. */
+ * The kernel's waits for its tensor-core products are bounded (2 s each): the
+ * rows of one that runs out are written as NaN, and abc_maf_check reports it. */
 abc_status abc_maf_sample(abc_maf maf, uint64_t n, const float* base_draws, uint64_t seed, uint32_t stream,
                           uint64_t first_index, float* theta_out, float* logq_out, void* cuda_stream);
 abc_status abc_maf_sample_at(abc_maf maf, int32_t flow, uint64_t n, const float* base_draws, uint64_t seed,
@@ -474,10 +473,16 @@ abc_status abc_maf_sample_at(abc_maf maf, int32_t flow, uint64_t n, const float*
 
 /* log q(theta) for n points (DEVICE float [n][8] inside the box) into logq_out
  * (DEVICE float [n]); a point's value does not depend on the others of its call.
- * Async, with bounded waits as abc_maf_sample. */
+ * Async; the points of a wait that runs out get NaN, as in abc_maf_sample. */
 abc_status abc_maf_log_q(abc_maf maf, uint64_t n, const float* theta, float* logq_out, void* cuda_stream);
 abc_status abc_maf_log_q_at(abc_maf maf, int32_t flow, uint64_t n, const float* theta, float* logq_out,
                             void* cuda_stream);
+
+/* ABC_ERR_TIMEOUT if a wait of an abc_maf_sample or abc_maf_log_q launch of this
+ * flow ran out since the last check (reported once; the rows concerned are NaN),
+ * else ABC_OK. Synchronizes cuda_stream, the stream of the launches in question.
+ * The sequential runs check their own launches. */
+abc_status abc_maf_check(abc_maf maf, void* cuda_stream);
 
 /* Gradient of the weighted mean of -log q_y(y(theta)) over n points (theta
  * DEVICE [n][8], weights DEVICE [n] >= 0 or NULL for all ones) into the flow's

@@ -178,6 +178,8 @@ def load(path=None):
         L.abc_maf_set_proposal_scale.restype = ctypes.c_int
         L.abc_maf_test_hold_products.argtypes = [pp, ctypes.c_int32]
         L.abc_maf_test_hold_products.restype = ctypes.c_int
+        L.abc_maf_check.argtypes = [pp, vp]
+        L.abc_maf_check.restype = ctypes.c_int
         L.abc_maf_sample_at.argtypes = [pp, i32, u64, vp, u64, u32, u64, vp, vp, vp]
         L.abc_maf_log_q_at.argtypes = [pp, i32, u64, vp, vp, vp]
         L.abc_maf_train_flows.argtypes = [pp, vp, vp, vp, i32, i32, ctypes.c_float, u64, ctypes.c_float, vp, vp]
@@ -714,9 +716,16 @@ class Flow:
         _check(self._L, self._L.abc_maf_set_proposal_scale(self._h, float(tau)))
 
     def test_hold_products(self, hold):
-        """Testing hook: the gradient kernel issues no tensor-core products, so
-        its bounded wait runs out and gradient/training raise ABC_ERR_TIMEOUT."""
+        """Testing hook: the kernels issue no tensor-core products, so their
+        bounded waits run out: gradient/training raise ABC_ERR_TIMEOUT, sample
+        and log_q give NaN and check raises."""
         _check(self._L, self._L.abc_maf_test_hold_products(self._h, int(bool(hold))))
+
+    def check(self, cuda_stream=None):
+        """Synchronise the stream and raise AbcError (ABC_ERR_TIMEOUT) if a wait
+        of a sample or log_q launch ran out since the last check; its rows are
+        NaN."""
+        _check(self._L, self._L.abc_maf_check(self._h, _stream(cuda_stream)))
 
     def set_params(self, params):
         """params: [n_params] (one flow) or [n_flows, n_params]."""
@@ -868,6 +877,10 @@ def abc_maf_set_proposal_scale(flow, tau):
 
 def abc_maf_test_hold_products(flow, hold):
     flow.test_hold_products(hold)
+
+
+def abc_maf_check(flow, cuda_stream=None):
+    flow.check(cuda_stream)
 
 
 def abc_maf_sample_at(flow, r, n, **kw):

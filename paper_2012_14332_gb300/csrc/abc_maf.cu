@@ -19,8 +19,10 @@
 // from shared memory on tcgen05 and accumulate in tensor memory per CTA.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstring>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <random>
@@ -524,9 +526,11 @@ __device__ __forceinline__ void stage_blocks_bulk(uint32_t* sm, const uint32_t* 
 // One thread of a group issues its products and commits them to the group's
 // mbarrier; the group's own named barrier orders its threads' shared and tensor
 // memory writes before the issue. Every wait is bounded: one that runs out sets
-// the flow's error word, later waits are skipped, and the kernel ends as usual.
+// the flow's error word for these kernels, later waits are skipped, the group's
+// rows are written as NaN, and the kernel ends as usual.
 // ---------------------------------------------------------------------------
 constexpr int kRowGroup = 128;
+constexpr float kNaN = std::numeric_limits<float>::quiet_NaN();
 
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, N >> 3 (bits 17-22), M >> 4 (bits 24-28)
@@ -535,11 +539,18 @@ __host__ __device__ constexpr uint32_t row_idesc(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kRowGroup >> 4) << 24);
 }
 
-// A group's products: its barrier, its tensor memory (column base), its rows'
-// layer-1 operand in shared memory ([16 row groups][2][8 rows][16 bytes]).
+// A group's mbarrier and whether a wait on it has run out, in shared memory.
+struct GroupBar {
+    uint64_t bar;
+    int failed, unused;
+};
+
+// A group's products: its GroupBar, its tensor memory (column base), its rows'
+// layer-1 operand in shared memory ([16 row groups][2][8 rows][16 bytes]), the row
+// that issues.
 struct RowGroup {
     uint32_t bar, tmem, lane_tmem, a1;   // lane_tmem: tmem at this warp's lane quarter
-    int id, row;
+    int id, row, issuer;
     uint32_t phase;
     bool ok;
     int* err;
@@ -551,17 +562,29 @@ struct RowGroup {
         tc_fence_before();
         asm volatile("bar.sync %0, %1;" ::"r"(1 + id), "n"(kRowGroup) : "memory");
     }
-    __device__ __forceinline__ bool issues() const { return row == 0; }
+    __device__ __forceinline__ bool issues() const { return row == issuer; }
+    __device__ __forceinline__ void fail()
+    {
+        ok = false;
+        asm volatile("st.shared.b32 [%0], %1;" ::"r"(bar + (uint32_t)offsetof(GroupBar, failed)), "r"(1) : "memory");
+        atomicExch(err, 1);
+    }
     // the committed products are complete
     __device__ __forceinline__ void after_commit()
     {
-        if (ok && !mbar_wait(bar, phase)) {
-            ok = false;
-            atomicExch(err, 1);
-        }
+        if (ok && !mbar_wait(bar, phase)) fail();
         phase ^= 1u;
         __syncwarp();
         tc_fence_after();
+    }
+    // after a tile's last wait: whether its row is sound. A wait of any thread of
+    // the group that ran out before the last issue spoils every row.
+    __device__ __forceinline__ bool sound()
+    {
+        int failed;
+        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(failed) : "r"(bar + (uint32_t)offsetof(GroupBar, failed)) : "memory");
+        ok = ok && !failed;
+        return ok;
     }
 };
 
@@ -595,11 +618,15 @@ __device__ __forceinline__ void relu_to_operand(uint32_t from, uint32_t to)
 // operands by bulk copy, the constant half of the rows' layer-1 operand.
 template <int GROUPS, int COLUMNS>
 __device__ __forceinline__ RowGroup row_setup(uint32_t* sm, const uint32_t* pub, int K, int from, int words, const Layout& L,
-                                              int* err, uint64_t (&bar)[GROUPS], uint64_t& bar_stage, uint32_t& tmem_s)
+                                              int* err, int issuer, GroupBar (&bar)[GROUPS], uint64_t& bar_stage,
+                                              uint32_t& tmem_s)
 {
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        for (int g = 0; g < GROUPS; ++g) mbar_init(smem_addr(&bar[g]), 1);
+        for (int g = 0; g < GROUPS; ++g) {
+            mbar_init(smem_addr(&bar[g].bar), 1);
+            bar[g].failed = 0;
+        }
         mbar_init(smem_addr(&bar_stage), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -620,13 +647,14 @@ __device__ __forceinline__ RowGroup row_setup(uint32_t* sm, const uint32_t* pub,
     __syncthreads();
     tc_fence_after();
     stage_blocks_bulk(sm, pub, K, from, words, L, smem_addr(&bar_stage));
-    g.bar = smem_addr(&bar[g.id]);
+    g.bar = smem_addr(&bar[g.id].bar);
     g.tmem = tmem_s + g.id * COLUMNS;
     g.lane_tmem = g.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     g.phase = 0;
+    g.issuer = issuer;
     g.err = err;
-    g.ok = mbar_wait(smem_addr(&bar_stage), 0);
-    if (!g.ok) atomicExch(err, 1);
+    g.ok = true;
+    if (!mbar_wait(smem_addr(&bar_stage), 0)) g.fail();
     __syncwarp();
     return g;
 }
@@ -670,13 +698,15 @@ __global__ void __launch_bounds__(kDensGroups * kRowGroup, kDensPerSm) logq_kern
                                                                           const __grid_constant__ Box box,
                                                                           const float* __restrict__ theta, uint64_t n,
                                                                           float inv_tau, float log_tau,
-                                                                          float* __restrict__ logq, int* __restrict__ err)
+                                                                          float* __restrict__ logq, int* __restrict__ err, int issuer)
 {
     extern __shared__ __align__(128) uint32_t row_sm[];
-    __shared__ __align__(8) uint64_t bar[kDensGroups], bar_stage;
+    __shared__ __align__(8) GroupBar bar[kDensGroups];
+    __shared__ __align__(8) uint64_t bar_stage;
     __shared__ uint32_t tmem_s;
     const Layout L = layout(H);
-    RowGroup g = row_setup<kDensGroups, kDensColumns>(row_sm, pub, K, L.d1, L.dens_words, L, err, bar, bar_stage, tmem_s);
+    RowGroup g =
+        row_setup<kDensGroups, kDensColumns>(row_sm, pub, K, L.d1, L.dens_words, L, err, issuer, bar, bar_stage, tmem_s);
     const int chunks = (H + kDensChunk - 1) / kDensChunk;
     const uint64_t tiles = (n + kRowGroup - 1) / kRowGroup;
     for (uint64_t tile = (uint64_t)blockIdx.x * kDensGroups + g.id; tile < tiles; tile += (uint64_t)gridDim.x * kDensGroups) {
@@ -752,7 +782,8 @@ __global__ void __launch_bounds__(kDensGroups * kRowGroup, kDensPerSm) logq_kern
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) lq.add(log_base(x[j] * inv_tau));
-        if (r < n) logq[r] = lq.plus(-sum_al - 8.f * log_tau);
+        const bool sound = g.sound();
+        if (r < n) logq[r] = sound ? lq.plus(-sum_al - 8.f * log_tau) : kNaN;
     }
     row_teardown<kDensGroups, kDensColumns>(tmem_s);
 }
@@ -769,13 +800,15 @@ template <int K, int CPD, int GROUPS>
 __global__ void __launch_bounds__(GROUPS * kRowGroup, GROUPS == 1 ? 4 : 8 / GROUPS) sample_kernel(
     const uint32_t* __restrict__ pub, int H, const __grid_constant__ Box box, const float* __restrict__ u_in,
     const __grid_constant__ ModelParams p, uint32_t ctr3, uint64_t first, uint64_t n, float tau, float log_tau,
-    float* __restrict__ theta_out, float* __restrict__ logq_out, int* __restrict__ err)
+    float* __restrict__ theta_out, float* __restrict__ logq_out, int* __restrict__ err, int issuer)
 {
     extern __shared__ __align__(128) uint32_t row_sm[];
-    __shared__ __align__(8) uint64_t bar[GROUPS], bar_stage;
+    __shared__ __align__(8) GroupBar bar[GROUPS];
+    __shared__ __align__(8) uint64_t bar_stage;
     __shared__ uint32_t tmem_s;
     const Layout L = layout(H);
-    RowGroup g = row_setup<GROUPS, kSampColumns>(row_sm, pub, K, L.s1, L.samp_words, L, err, bar, bar_stage, tmem_s);
+    RowGroup g =
+        row_setup<GROUPS, kSampColumns>(row_sm, pub, K, L.s1, L.samp_words, L, err, issuer, bar, bar_stage, tmem_s);
     const uint64_t tiles = (n + kRowGroup - 1) / kRowGroup;
     for (uint64_t tile = (uint64_t)blockIdx.x * GROUPS + g.id; tile < tiles; tile += (uint64_t)gridDim.x * GROUPS) {
         const uint64_t r = tile * kRowGroup + g.row;
@@ -861,11 +894,12 @@ __global__ void __launch_bounds__(GROUPS * kRowGroup, GROUPS == 1 ? 4 : 8 / GROU
             to_theta(box, j, x[j], th[j], jac);
             lq.add(-jac);
         }
+        const bool sound = g.sound();
         if (r < n) {
             float2* to = reinterpret_cast<float2*>(theta_out + 8 * r);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) to[j] = make_float2(th[2 * j], th[2 * j + 1]);
-            if (logq_out) logq_out[r] = lq.plus(-sum_al - 8.f * log_tau);
+            for (int j = 0; j < 4; ++j) to[j] = sound ? make_float2(th[2 * j], th[2 * j + 1]) : make_float2(kNaN, kNaN);
+            if (logq_out) logq_out[r] = sound ? lq.plus(-sum_al - 8.f * log_tau) : kNaN;
         }
     }
     row_teardown<GROUPS, kSampColumns>(tmem_s);
@@ -1924,8 +1958,8 @@ struct abc_maf_s {
     size_t part_floats = 0;    // allocated size of d_part
     uint32_t* d_pub = nullptr; // [R][K][pub_words] published BF16 operands
     float* d_sums = nullptr;   // [R][2] (weighted loss sum, weight sum)
-    int* d_err = nullptr;      // set by a gradient kernel whose bounded wait ran out
-    int hold = 0;              // testing: the gradient kernel issues no products
+    int* d_err = nullptr;      // [2], set by a bounded wait that ran out: the gradient's; sampling's and density's
+    int hold = 0;              // testing: no kernel issues its products
     int* d_step = nullptr;     // [0] the step of abc_maf_adam_step, [1] a training run's ticket counter
     maf::TrainSlot* d_slots = nullptr;   // [R] training data of each flow
     maf::TrainSlot* d_slots_val = nullptr;   // [R] validation data of each flow (early stopping)
@@ -1949,16 +1983,19 @@ namespace {
         if (_e != cudaSuccess) return plan_cuda_fail(_e, what); \
     } while (0)
 
-// After the stream has been synchronised: ABC_ERR_TIMEOUT if a gradient
-// kernel's bounded wait for its tensor-core products ran out (the word is
-// then cleared for the next call).
-abc_status take_err(abc_maf f)
+// After the stream has been synchronised: ABC_ERR_TIMEOUT if a bounded wait of
+// a gradient kernel (kErrGradient) or of a sampling or density kernel (kErrRows)
+// ran out since the last call (the word is then cleared for the next one).
+enum { kErrGradient = 0, kErrRows = 1 };
+abc_status take_err(abc_maf f, int which)
 {
     int h = 0;
-    MAF_TRY(cudaMemcpy(&h, f->d_err, sizeof h, cudaMemcpyDeviceToHost), "cudaMemcpy(error word)");
+    MAF_TRY(cudaMemcpy(&h, f->d_err + which, sizeof h, cudaMemcpyDeviceToHost), "cudaMemcpy(error word)");
     if (h) {
-        MAF_TRY(cudaMemset(f->d_err, 0, sizeof h), "cudaMemset(error word)");
-        return plan_fail(ABC_ERR_TIMEOUT, "a flow kernel's wait for its operands or tensor-core products ran out of time");
+        MAF_TRY(cudaMemset(f->d_err + which, 0, sizeof h), "cudaMemset(error word)");
+        return plan_fail(ABC_ERR_TIMEOUT, which == kErrGradient
+                                              ? "a flow gradient kernel's wait for its tensor-core products ran out of time"
+                                              : "a flow sampling or density kernel's wait ran out of time: its rows are NaN");
     }
     return ABC_OK;
 }
@@ -2056,6 +2093,9 @@ int row_grid(uint64_t tiles, int groups, size_t smem, int most)
     return (int)std::min((tiles + groups - 1) / groups, cap);
 }
 
+// the row of a group that issues its products (testing: none)
+int issuing_row(const abc_maf_s* f) { return f->hold ? maf::kRowGroup : 0; }
+
 uint64_t row_tiles(uint64_t n) { return n / maf::kRowGroup + (n % maf::kRowGroup != 0); }
 
 template <int K>
@@ -2066,7 +2106,8 @@ cudaError_t launch_logq(abc_maf f, int r, uint64_t n, const float* theta, float*
     if (e != cudaSuccess) return e;
     const int grid = row_grid(row_tiles(n), maf::kDensGroups, smem, maf::kDensPerSm);
     maf::logq_kernel<K><<<grid, maf::kDensGroups * maf::kRowGroup, smem, s>>>(flow_pub(f, r), f->H, f->box, theta, n,
-                                                                              1.f / f->tau, logf(f->tau), logq, f->d_err);
+                                                                              1.f / f->tau, logf(f->tau), logq,
+                                                                              f->d_err + kErrRows, issuing_row(f));
     return cudaGetLastError();
 }
 
@@ -2079,7 +2120,7 @@ cudaError_t launch_sample_g(abc_maf f, int r, uint64_t n, const float* u, const 
     if (e != cudaSuccess) return e;
     const int grid = row_grid(row_tiles(n), GROUPS, smem, 8 / GROUPS);
     maf::sample_kernel<K, CPD, GROUPS><<<grid, GROUPS * maf::kRowGroup, smem, s>>>(
-        flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, logf(f->tau), theta, logq, f->d_err);
+        flow_pub(f, r), f->H, f->box, u, p, ctr3, first, n, f->tau, logf(f->tau), theta, logq, f->d_err + kErrRows, issuing_row(f));
     return cudaGetLastError();
 }
 
@@ -2368,8 +2409,8 @@ cudaError_t launch_train_step(abc_maf f, uint32_t batch, const ModelParams& p, f
 }  // namespace
 
 // a wait that ran out in a sampling or density launch since the last check, for
-// callers that have synchronised and run no training after it
-abc_status abcgb::maf_take_error(abc_maf f) { return take_err(f); }
+// callers that have synchronised
+abc_status abcgb::maf_take_error(abc_maf f) { return take_err(f, kErrRows); }
 
 extern "C" {
 
@@ -2416,12 +2457,12 @@ abc_status abc_maf_create_multi(int32_t n_flows, int32_t n_blocks, int32_t hidde
         (e = cudaMalloc(&f->d_slots, sizeof(maf::TrainSlot) * f->R)) != cudaSuccess ||
         (e = cudaMalloc(&f->d_slots_val, sizeof(maf::TrainSlot) * f->R)) != cudaSuccess ||
         (e = cudaMallocHost(&f->h_io, sizeof(float) * (2 * (size_t)f->R + 4))) != cudaSuccess ||
-        (e = cudaMalloc(&f->d_err, sizeof(int))) != cudaSuccess)
+        (e = cudaMalloc(&f->d_err, 2 * sizeof(int))) != cudaSuccess)
         return fail_free(plan_cuda_fail(e, "cudaMalloc(flow)"));
     if ((e = cudaMemset(f->d_params, 0, np)) != cudaSuccess || (e = cudaMemset(f->d_m, 0, np)) != cudaSuccess ||
         (e = cudaMemset(f->d_v, 0, np)) != cudaSuccess || (e = cudaMemset(f->d_step, 0, 2 * sizeof(int))) != cudaSuccess ||
         (e = cudaMemset(f->d_slots, 0, sizeof(maf::TrainSlot) * f->R)) != cudaSuccess ||
-        (e = cudaMemset(f->d_err, 0, sizeof(int))) != cudaSuccess ||
+        (e = cudaMemset(f->d_err, 0, 2 * sizeof(int))) != cudaSuccess ||
         (e = publish(f, nullptr)) != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess)
         return fail_free(plan_cuda_fail(e, "flow initialisation"));
     *maf_out = f;
@@ -2436,6 +2477,15 @@ abc_status abc_maf_create(int32_t n_blocks, int32_t hidden, const abc_prior_box*
 int64_t abc_maf_param_count(abc_maf f) { return f ? f->n_params : -1; }
 
 int32_t abc_maf_flow_count(abc_maf f) { return f ? f->R : -1; }
+
+abc_status abc_maf_check(abc_maf f, void* cuda_stream)
+{
+    abc_status st;
+    if ((st = check(f)) != ABC_OK) return st;
+    MAF_TRY(cudaStreamSynchronize((cudaStream_t)cuda_stream), "cudaStreamSynchronize");
+    if ((st = take_err(f, kErrRows)) != ABC_OK) return st;
+    return plan_ok();
+}
 
 abc_status abc_maf_test_hold_products(abc_maf f, int32_t hold)
 {
@@ -2555,7 +2605,7 @@ abc_status abc_maf_gradient(abc_maf f, uint64_t n, const float* theta, const flo
     MAF_TRY(cudaMemcpyAsync(sums, f->d_sums, sizeof sums, cudaMemcpyDeviceToHost, s), "cudaMemcpyAsync(sums)");
     MAF_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
     {
-        const abc_status es = take_err(f);
+        const abc_status es = take_err(f, kErrGradient);
         if (es != ABC_OK) return es;
     }
     if (loss_out) *loss_out = sums[1] > 0.f ? sums[0] / sums[1] : 0.f;
@@ -2747,7 +2797,7 @@ abc_status abc_maf_train_flows(abc_maf f, const float* const* theta, const float
         MAF_TRY(cudaMemcpyAsync(fin.data(), d_st, stop_bytes, cudaMemcpyDeviceToHost, s), "cudaMemcpyAsync(early stopping)");
         MAF_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
         {
-            const abc_status es = take_err(f);
+            const abc_status es = take_err(f, kErrGradient);
             if (es != ABC_OK) return es;
         }
         if (loss_out)
@@ -2767,14 +2817,14 @@ abc_status abc_maf_train_flows(abc_maf f, const float* const* theta, const float
                 "cudaMemcpyAsync(sums)");
         MAF_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
         {
-            const abc_status es = take_err(f);
+            const abc_status es = take_err(f, kErrGradient);
             if (es != ABC_OK) return es;
         }
         for (int r = 0; r < f->R; ++r) loss_out[r] = sums[2 * r + 1] > 0.f ? sums[2 * r] / sums[2 * r + 1] : 0.f;
     } else {
         MAF_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
         {
-            const abc_status es = take_err(f);
+            const abc_status es = take_err(f, kErrGradient);
             if (es != ABC_OK) return es;
         }
     }

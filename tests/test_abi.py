@@ -195,6 +195,7 @@ def test_other_entry_points_validate(L):
                               ctypes.byref(n1), ctypes.byref(n2), None) == ABC_ERR_INVALID_ARG
     # flow calls on a NULL flow return before any CUDA call
     assert L.abc_maf_test_hold_products(None, 1) == ABC_ERR_INVALID_ARG
+    assert L.abc_maf_check(None, None) == ABC_ERR_INVALID_ARG
     assert "NULL" in L.abc_last_error().decode()
 
 

@@ -296,6 +296,39 @@ def test_gradient_wait_that_runs_out_reports_timeout_and_recovers():
     f.close()
 
 
+
+@pytest.mark.parametrize("n", [200, 60_000, 200_000])   # one, two and four groups a sampling CTA
+def test_sampling_and_density_waits_that_run_out_mark_their_rows_and_are_reported(n):
+    """With the products held every wait runs out after 2 s (a thread skips its
+    later ones): the rows are NaN, check reports it once, a gradient is not
+    charged with it, and the next calls give what they gave before."""
+    import time
+    f, _ = _flow(2, 256, 47, 0.3)
+    th, lq = f.sample(n, seed=1)
+    d = f.log_q(th)
+    loss, _ = f.gradient(th[:500])
+    f.check()
+    f.test_hold_products(True)
+    for call in (lambda: f.sample(n, seed=1), lambda: (f.log_q(th),), lambda: f.sample(n, seed=1, want_logq=False)[:1]):
+        t0 = time.monotonic()
+        out = call()
+        torch.cuda.synchronize()
+        assert time.monotonic() - t0 < 30
+        assert all(bool(torch.isnan(x).all()) for x in out)
+        f.test_hold_products(False)
+        assert f.gradient(th[:500])[0] == loss
+        with pytest.raises(abc.AbcError) as e:
+            f.check()
+        assert e.value.status == abc.binding.ABC_ERR_TIMEOUT
+        f.check()
+        f.test_hold_products(True)
+    f.test_hold_products(False)
+    th2, lq2 = f.sample(n, seed=1)
+    assert torch.equal(th2, th) and torch.equal(lq2, lq) and torch.equal(f.log_q(th), d)
+    f.check()
+    f.close()
+
+
 def test_adam_step_matches_oracle():
     K, H = 2, 32
     f, params = _flow(K, H, 41, 0.5)
