@@ -88,17 +88,22 @@ struct Whiten {
 };
 
 // a = L^-1 (theta - centre) for a row. Only differences of whitened rows are
-// used; a centre inside the population keeps them, and their roundings, small.
+// used; a centre inside the population keeps them, and their roundings, small. An
+// infinite coordinate meets the matrix's leading part alone: the other part's sign
+// may be the opposite one, and their sum no number.
 __device__ __forceinline__ void whiten(const Whiten& Li, const float* th, const float (&centre)[8], float a[8])
 {
-    float d[8];
+    float d[8], e[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) d[k] = th[k] - centre[k];
+    for (int k = 0; k < 8; ++k) {
+        d[k] = th[k] - centre[k];
+        e[k] = fabsf(d[k]) < __int_as_float(0x7F800000) ? d[k] : 0.f;
+    }
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         float v = 0.f;
 #pragma unroll
-        for (int k = 0; k <= r; ++k) v = __fmaf_rn(Li.lo.a[r * 8 + k], d[k], v);
+        for (int k = 0; k <= r; ++k) v = __fmaf_rn(Li.lo.a[r * 8 + k], e[k], v);
 #pragma unroll
         for (int k = 0; k <= r; ++k) v = __fmaf_rn(Li.hi.a[r * 8 + k], d[k], v);
         a[r] = v;

@@ -128,3 +128,30 @@ def test_weights_at_the_edges_of_the_split(n, m):
     rel = np.abs(got / want - 1)
     # an exponent of x bits carries x 2^-23 from FP32 distances: 1e-4 at 135, less nearer
     assert rel[:n - far].max(initial=0) < 1e-4 and rel[n - far:].max() < 1e-3 + 2.0 ** -13
+
+
+@pytest.mark.parametrize("column", [0, 3, 7])
+@pytest.mark.parametrize("value", [np.inf, -np.inf])
+def test_an_infinitely_far_particle_weighs_nothing(column, value):
+    """An old particle with an infinite coordinate adds nothing to any row (its
+    squared distance is infinite), and a new one has no density: weight +inf."""
+    n, m = 300, 500
+    old, w = _population(m, 3)
+    new, _ = _population(n, 4)
+    g = np.random.default_rng(5)
+    L = ((0.2 * np.eye(8) + 0.05 * np.tril(g.standard_normal((8, 8)), -1)) * (HI - LO)[:, None]).astype(np.float32)
+    Li = np.linalg.inv(L.astype(np.float64))
+    far_old, far_new = old.copy(), new.copy()
+    far_old[[0, 77, 499], column] = value
+    far_new[123, column] = value
+
+    def weights(a, b):
+        return abc.abc_pmc_weights(torch.from_numpy(a).to(DEV), torch.from_numpy(b).to(DEV), torch.from_numpy(w).to(DEV),
+                                   L).cpu().numpy()
+
+    keep = np.isfinite(far_old).all(1)
+    a, b = new.astype(np.float64) @ Li.T, old.astype(np.float64) @ Li.T
+    terms = np.exp(-0.5 * ((a[:, None] - b[None]) ** 2).sum(2)) * w
+    assert np.abs(weights(new, far_old) * terms[:, keep].sum(1) - 1).max() < 1e-4
+    got = weights(far_new, old)
+    assert got[123] == np.inf and np.abs(np.delete(got * terms.sum(1), 123) - 1).max() < 1e-4
