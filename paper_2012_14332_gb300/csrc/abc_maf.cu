@@ -138,10 +138,14 @@ __host__ __device__ inline Layout layout(int H)
 }
 
 // Part k (0..2) of b as bf16: each part is the rounding of what the ones before
-// left, so the three add up to b to its last bit (24 bits of significand).
+// left, so the three add up to b to its last bit (24 bits of significand); of a b
+// that rounds to an infinity (a unit held at 0 by -inf, say) the others are 0.
 __device__ __forceinline__ float bias_part(float b, int k)
 {
-    for (int i = 0; i < k; ++i) b -= __bfloat162float(__float2bfloat16_rn(b));
+    for (int i = 0; i < k; ++i) {
+        const float h = __bfloat162float(__float2bfloat16_rn(b));
+        b = fabsf(h) < __int_as_float(0x7F800000) ? b - h : 0.f;
+    }
     return b;
 }
 

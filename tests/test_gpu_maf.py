@@ -153,6 +153,30 @@ def test_one_index_has_one_result_in_calls_of_any_size(K, H, tiles, extra):
     f.close()
 
 
+
+@pytest.mark.parametrize("bias", [-np.inf, -3.4e38, -1e30])
+@pytest.mark.parametrize("H", [64, 256])
+def test_a_unit_held_at_zero_by_its_bias(H, bias):
+    """A hidden unit whose bias is -inf, or below the bf16 range, is 0 whatever
+    its inputs: density and sampling are those of the flow without the unit's
+    outgoing weights, bit for bit."""
+    K = 2
+    params = mo.init_params(np.random.default_rng(3), K=K, H=H, scale=0.3)
+    dead = np.random.default_rng(4).choice(H, 9, replace=False)
+    with_bias, without = (mo.unflat(mo.flat(params), K, H) for _ in range(2))
+    for p, q in zip(with_bias, without):
+        p["b1"][dead] = bias
+        q["W2"][:, dead] = 0.0
+    out = []
+    for ps in (with_bias, without):
+        f = abc.Flow(K, H)
+        f.set_params(mo.flat(ps).astype(np.float32))
+        out.append((f.log_q(torch.from_numpy(_thetas(700, 5)).to(DEV)),) + f.sample(700, seed=6))
+        f.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b) and bool(torch.isfinite(a).all())
+
+
 def test_zero_flow_draws_the_prior_from_the_documented_words():
     """A flow with zero parameters is the uniform prior: base coordinate c of
     sample j is logit(u), u = (2m + 1) 2^-24 from word c mod 4 of the Philox
