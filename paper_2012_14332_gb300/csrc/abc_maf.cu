@@ -675,8 +675,8 @@ __device__ __forceinline__ void row_teardown(uint32_t tmem_s)
 
 // log q of one row: the base's and the box map's 16 terms, whose sum is an order
 // larger than any of them, with the rounding errors carried along (Knuth's
-// two-sum). Plain sums in one thread would round at the total's size each time;
-// the mma.sync form spreads a row's over 4 lanes.
+// two-sum). Plain sums in one thread would round at the total's size each time.
+// An infinite term has no rounding error: the plain sum is the result.
 struct LogSum {
     float hi = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(float v)
@@ -685,7 +685,10 @@ struct LogSum {
         lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, w)), __fsub_rn(v, w));
         hi = t;
     }
-    __device__ __forceinline__ float plus(float v) const { return hi + (lo + v); }
+    __device__ __forceinline__ float plus(float v) const
+    {
+        return hi + (fabsf(hi) < __int_as_float(0x7F800000) ? lo + v : v);
+    }
 };
 
 // Density: a group a CTA, four CTAs an SM. Hidden units go through in chunks

@@ -177,6 +177,22 @@ def test_a_unit_held_at_zero_by_its_bias(H, bias):
         assert torch.equal(a, b) and bool(torch.isfinite(a).all())
 
 
+
+@pytest.mark.parametrize("K", [1, 3])
+def test_density_of_points_mapped_to_infinity(K):
+    """Where the last block's output overflows the base's density is 0 and log q
+    is -inf, not NaN."""
+    H = 64
+    params = mo.init_params(np.random.default_rng(3), K=K, H=H, scale=0.3)
+    params[-1]["b2"][5] = 1e38          # mu_5, and alpha_5 = -6: (x - mu) exp(6) overflows
+    params[-1]["b2"][8 + 5] = -1e3
+    f = abc.Flow(K, H)
+    f.set_params(mo.flat(params).astype(np.float32))
+    got = f.log_q(torch.from_numpy(_thetas(300, 5)).to(DEV))
+    assert bool((got == -torch.inf).all())
+    f.close()
+
+
 def test_zero_flow_draws_the_prior_from_the_documented_words():
     """A flow with zero parameters is the uniform prior: base coordinate c of
     sample j is logit(u), u = (2m + 1) 2^-24 from word c mod 4 of the Philox
