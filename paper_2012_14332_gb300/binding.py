@@ -995,15 +995,20 @@ def abc_smc_run_regions(regions, rounds=16, shrink_rounds=4, sims_per_round=1 <<
 def abc_project(theta, sample_index, init_ard, T, N_pop, seed, quantiles=(0.05, 0.5, 0.95), stream=0, mode="fast",
                 cuda_stream=None):
     """Quantile bands [n_q, T+1, 3] (A, R, D) of trajectories simulated from
-    theta [B, 8] (CUDA f32) with sample_index [B] (CUDA int64)."""
+    theta [B, 8] (CUDA f32) with sample_index [B] (CUDA int64). On a cuda_stream
+    other than the current one the call returns when the bands are complete."""
     L = load()
     B = theta.shape[0]
     q = np.ascontiguousarray(np.asarray(quantiles, dtype=np.float64))
     bands = torch.empty((len(q), T + 1, 3), dtype=torch.float32, device=theta.device)
     a, a_p = _host_i32(init_ard)
+    raw = _stream(cuda_stream)
     _check(L, L.abc_project(_dev(theta, torch.float32, (B, 8)), _dev(sample_index, torch.int64, (B,)), B, a_p,
                             int(T), int(N_pop), int(seed), int(stream), _mode(mode), q.ctypes.data, len(q),
-                            bands.data_ptr(), _stream(cuda_stream)))
+                            bands.data_ptr(), raw))
+    if raw != _stream(None):
+        # the caller reads the bands, and gives the inputs' memory back, on the current stream
+        (torch.cuda.ExternalStream(raw) if raw else torch.cuda.default_stream()).synchronize()
     return bands
 
 

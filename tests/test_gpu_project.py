@@ -40,3 +40,28 @@ def test_bands_equal_oracle_order_statistics(B):
         assert np.array_equal(bands[k], want), (k, qq)
     # the first 49 days of the projection are the accepted trajectories' own days
     assert np.all(bands[0] <= bands[2]) and np.all(bands[2] <= bands[4])
+
+
+@pytest.mark.parametrize("n_q", [3, 40])
+@pytest.mark.parametrize("as_int", [False, True])
+def test_bands_on_another_stream_are_complete_on_return(n_q, as_int):
+    """A call on a busy stream of its own returns complete bands: they are read
+    on the current stream at once, and the inputs' memory is given back to it."""
+    P, T, B = 10**6, 40, 300
+    th = torch.from_numpy(inputs.random_thetas(B, 3)).cuda()
+    idx = torch.arange(B, device="cuda")
+    q = np.linspace(0.01, 0.99, n_q)
+    want = abc.abc_project(th, idx, [100, 3, 0], T, P, 5, quantiles=q)
+    torch.cuda.synchronize()
+    s, x = torch.cuda.Stream(), torch.zeros(4096, 4096, device="cuda")
+    with torch.cuda.stream(s):
+        for _ in range(30):
+            x = x @ x
+    th2, idx2 = th.clone(), idx.clone()
+    torch.cuda.current_stream().synchronize()
+    got = abc.abc_project(th2, idx2, [100, 3, 0], T, P, 5, quantiles=q, cuda_stream=s.cuda_stream if as_int else s)
+    del th2, idx2
+    junk = [torch.full((B, 8), 7.0, device="cuda"), torch.full((B,), 7, device="cuda")]
+    assert torch.equal(got, want)
+    torch.cuda.synchronize()
+    del junk
