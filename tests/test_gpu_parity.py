@@ -245,8 +245,8 @@ def _top_range_observed(kind):
 def test_distance_at_the_top_of_its_range(kind):
     """Eq. 7 with the exact uint64 sum saturating at 2^63: every distance
     (abc_distances) equals the oracle's, including sqrt(2^63) for saturated
-    sums; the accept sets of abc_reject_kernel (abc_sample) and of
-    abc_batch_kernel (a one-region plan) equal the oracle's at an eps just
+    sums; the accept sets of abc_sample (20,000 samples: the staged rejection
+    kernel) and of abc_batch_kernel (a one-region plan) equal the oracle's at an eps just
     below 2^31 (threshold below 2^62: the kernels' clamped accumulation), at
     an eps whose threshold lies between 2^62 and 2^63 (accepted sums in that
     range) and at eps = sqrt(2^63) (saturated sums accepted too)."""

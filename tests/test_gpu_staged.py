@@ -1,6 +1,7 @@
 """Small calls run on the staged kernels, larger ones on a thread per sample:
-both give the same distances, accept sets and trajectories, bit for bit, at the
-edges of blocks, stages and horizons; bands are the order statistics of the
+both give the same distances, accept sets and (exact) trajectories, bit for bit,
+at the edges of blocks, stages and horizons (fast trajectories are always staged:
+calls of different sizes agree); bands are the order statistics of the
 trajectories at the edges of their two block shapes."""
 import numpy as np
 import pytest
