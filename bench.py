@@ -238,7 +238,7 @@ def bench_config1(abc, torch, dev, reps=20, warmup=3):
     """Plain ABC on region_1e6_T49 (P = 1e6, T = 49): 65,536 prior samples,
     exact mode, eps at the 0.1 % distance quantile. One run is the whole
     pipeline through the public calls: every distance and prior draw, eps as
-    the k-th smallest, k = ceil(0.001 n) = 66 (radix select on the device),
+    the k-th smallest, k = ceil(0.001 n) = 66 (selected on the device),
     then the samples at or below that eps from those distances (the same
     accepted set as a rejection launch at eps, without simulating again).
     Timed as one abc_sample_quantile call, and beside it as the three calls
@@ -372,7 +372,7 @@ def bench_projection(abc, torch, w, B=8192, T=120, reps=10):
     ms = timed(lambda: abc.abc_project(th, idx, w["observed"][:, 0], T, w["P"], w["seed"], cuda_stream=s))
     ms_sim = timed(lambda: abc.abc_simulate(th, idx, w["observed"][:, 0], T, w["P"], w["seed"], mode="fast",
                                             cuda_stream=s))
-    # one thread per trajectory: 8192 trajectories are 1.7 warps per SM, so the
+    # 8192 trajectories are 256 blocks of 32 samples, their days one chain: the
     # call is latency-bound by its size (Sec. 5 projects 100 samples)
     return {"workload": "%d accepted samples of region_6e7_T100 simulated %d days from its initial condition, "
                         "bands at the 5, 50, 95 %% quantiles, fast mode" % (m, T),

@@ -11,7 +11,8 @@
 
 namespace abcgb {
 
-// Stage the observed (A, R, D, 0) series of days 0..T into shared memory.
+// Stage the observed series of days 0..T (A, R, D and the extinction terms) into
+// shared memory.
 __device__ __forceinline__ void stage_observed(int4* obs_s, const int4* __restrict__ obs, int32_t T)
 {
     for (int32_t d = threadIdx.x; d <= T; d += blockDim.x) obs_s[d] = obs[d];

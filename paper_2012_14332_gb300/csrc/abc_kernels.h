@@ -159,8 +159,9 @@ cudaError_t launch_reject(const ModelParams& p, const RejectArgs& a, int mode, c
 cudaError_t launch_distances(const ModelParams& p, const DistanceArgs& a, int mode, cudaStream_t s);
 cudaError_t launch_simulate(const ModelParams& p, const SimulateArgs& a, int mode, cudaStream_t s);
 cudaError_t launch_step(const ModelParams& p, const StepArgs& a, int mode, cudaStream_t s);
-// the same for calls of at most one wave of staged blocks (abc_staged.cu):
-// *taken tells whether the call was one; the three above ask these first
+// the same for calls that run on the staged kernels (abc_staged.cu: up to one wave
+// of their blocks, rejection up to three, fast trajectories always): *taken tells
+// whether the call was one; the three above ask these first
 cudaError_t launch_staged_reject(const ModelParams& p, const RejectArgs& a, int mode, cudaStream_t s, int* blocks_out,
                                  bool* taken);
 cudaError_t launch_staged_distances(const ModelParams& p, const DistanceArgs& a, int mode, cudaStream_t s, bool* taken);
@@ -197,8 +198,8 @@ cudaError_t launch_kth_bracket(const double* dist, uint64_t n, uint64_t k, Selec
 cudaError_t launch_kth_radix(const double* dist, uint64_t n, uint64_t k, SelectWork* w, cudaStream_t s);
 // Compaction of the samples with dist[j] <= eps (theta, theta_out may both be
 // NULL); *count (zeroed by the caller) receives the number of accepts. With
-// eps_key set, eps is the value whose bit pattern is eps_key->prefix (the
-// radix select's k-th smallest, computed on the device) instead of `eps`.
+// eps_key set, eps is the value whose bit pattern is eps_key->prefix (the k-th
+// smallest, found on the device) instead of `eps`.
 struct SelectArgs {
     const double* dist;
     const float* theta;

@@ -916,8 +916,8 @@ __global__ void __launch_bounds__(GROUPS * kRowGroup, GROUPS == 1 ? 4 : 8 / GROU
 // gradient of sum_r w_r (-log q_y(y_r)) (unnormalised; Adam divides by sum w)
 // ---------------------------------------------------------------------------
 // The forward pass and the backward products of each row (g_h = g_out W2,
-// g_x = g_a1 W1) run in the warp's registers on mma.sync, as in the density
-// kernel. The weight gradients reduce over rows:
+// g_x = g_a1 W1) run in the warp's registers on mma.sync. The weight gradients
+// reduce over rows:
 //   dW2^T [l][o]       = sum over rows of h[row][l] g_out[row][o]
 //   [dW1 | db1] [l][j] = sum over rows of g_a1[row][l] [x | 1][row][j]
 // (j < 8: dW1, j = 8: db1). Per warp tile both are products of M = 128 hidden

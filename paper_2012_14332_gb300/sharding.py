@@ -36,8 +36,7 @@ def _host(a):
 
 def local_k_smallest(dist, k):
     """This rank's k smallest distances (a CUDA f64 tensor, e.g. from
-    abc_distances), found on the device: its k-th smallest by the radix select,
-    then the accept step at that value (ties included). Returns them ascending
+    abc_distances), found on the device: its k-th smallest, then the accept step at that value (ties included). Returns them ascending
     in host memory, min(k, n) values."""
     from . import binding
     n = dist.numel()

@@ -481,9 +481,9 @@ def test_flow_set_members_equal_single_flows():
 @pytest.mark.parametrize("K,H,R", [(3, 256, 1), (2, 64, 1), (3, 112, 3), (4, 256, 2), (1, 208, 1)])
 def test_training_steps_publish_what_a_full_publish_writes(K, H, R):
     """A training step's Adam launch republishes each parameter it updates, one
-    thread per parameter, into every layout the kernels read (density,
-    gradient and the sampler's degree-grouped copy), and training without
-    validation ends on that. The densities, draws and gradient after training
+    thread per parameter, into the gradient's layout, and a run ends with a full
+    publish (density and the sampler's degree-grouped copy too). The densities,
+    draws and gradient after training
     then equal those after a full republish of the same parameters, bit for
     bit: a parameter written to a wrong place, or not at all, would change
     them. Shapes: the paired and unpaired gradient forms, a set of flows, and
